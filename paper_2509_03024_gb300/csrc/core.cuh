@@ -45,8 +45,17 @@ struct Prime {
     u64 mu;
     u64 one_s;  // floor(2^64 / q): Shoup companion of 1, for lazy reduction of any 64-bit value
     u32 b;
+    u32 cls;    // arithmetic of the transforms and of products with constants (Arith in ntt_core.cuh)
+    u32 delta;  // near primes: 2^b - q
     u32 pad;
 };
+
+// Constants modulo a near prime (q = 2^b - delta) are kept as two words W0 = w and W1 = 2^32 w mod q,
+// each split in a low and a high part (low | high << 32); see ntt_core.cuh. Transform twiddles and
+// other single products split at nttc::split_at; the base conversions into 50-bit primes, which sum
+// several products before reducing, at kConvSplit.
+inline u64 split_word(u64 w, int at) { return (w & (((u64)1 << at) - 1)) | ((w >> at) << 32); }
+constexpr int kConvSplit = 21;
 
 __host__ __device__ __forceinline__ u64 add_mod(u64 a, u64 b, u64 q) {
     u64 s = a + b;
@@ -249,26 +258,25 @@ struct Ctx {
 
     // device tables
     Prime* d_primes = nullptr;        // [n_ext]
-    u64* d_psi = nullptr;             // [n_ext][N]  psi^brev(i)   (forward twiddles)
-    u64* d_psi_s = nullptr;           // Shoup companions
-    u64* d_ipsi = nullptr;            // [n_ext][N]  psi^-brev(i)  (inverse twiddles)
-    u64* d_ipsi_s = nullptr;
-    u64* d_ninv = nullptr;            // [n_ext][2] N^-1 and its Shoup companion
-    // NTT twiddles interleaved with their Shoup companions (one 128-bit load each):
-    // column / single-pass tables [prime][i] = (psi^brev(i), companion), inverse alike;
-    // row-pass tables of the two-pass NTT laid out [prime][stage s'][group g][row r]
-    // (value = psi^brev(2^(S1+s') + r 2^s' + g)), so that consecutive rows are contiguous
+    u64* d_ninv = nullptr;            // [n_ext][2] words of N^-1
+    // Constants of products are stored as the two words their multiplication takes (const_words in
+    // ctx.cu): (w, Shoup companion) or, for near primes, (w, 2^32 w mod q), each split.
+    // NTT twiddles, one 128-bit load each:
+    // column / single-pass tables [prime][i] = words of psi^brev(i), inverse alike;
+    // row-pass tables of the two-pass NTT [prime][row r][N2], entry = words of
+    // psi^brev(2^(S1+s) + r 2^s + grp) for stage s and group grp of the row, a stage's groups ordered
+    // so that the threads of a row read consecutive entries (build_tables)
     ulonglong2* d_tw = nullptr;
     ulonglong2* d_itw = nullptr;
     ulonglong2* d_tw2 = nullptr;
     ulonglong2* d_itw2 = nullptr;
     int ntt_s1 = 0;                   // column stages of the two-pass NTT (0: single pass)
-    u64* d_resc = nullptr;            // [L+1][L+1][2] q_l^-1 mod q_i (+ Shoup)
-    u64* d_up_inv = nullptr;          // [L+1][L+1][2] digit-local qhat_i^-1 mod q_i at level l
+    u64* d_resc = nullptr;            // [L+1][L+1][2] q_l^-1 mod q_i and its Shoup companion
+    u64* d_resc_w = nullptr;          // [L+1][L+1][2] words of q_l^-1 mod q_i
+    // base-conversion constants (conv_words in ctx.cu)
     u64* d_up_hat = nullptr;          // [L+1][L+1][n_ext][2] digit-local qhat_i mod prime t at level l
     u64* d_up_ninv = nullptr;         // [L+1][L+1][2] N^-1 * qhat_i^-1 mod q_i (ModUp input scaling)
     u64* d_down_ninv = nullptr;       // [alpha][2]   N^-1 * Phat_k^-1 mod p_k (ModDown input scaling)
-    u64* d_down_inv = nullptr;        // [alpha][2]   Phat_k^-1 mod p_k
     u64* d_down_hat = nullptr;        // [alpha][L+1][2] Phat_k mod q_i
     u64* d_pinv = nullptr;            // [L+1][2]     P^-1 mod q_i
     u64* d_pmod = nullptr;            // [L+1]        P mod q_i

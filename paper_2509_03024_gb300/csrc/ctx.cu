@@ -7,10 +7,15 @@
 
 #include "core.cuh"
 #include "ks_inner.cuh"
+#include "ntt_core.cuh"
 
 namespace fhe {
 
 // ============================================================================ errors
+
+using nttc::AR_NEAR50;
+using nttc::AR_NEAR60;
+using nttc::AR_SHOUP;
 
 void fail(int code, const std::string& msg) { throw FheException(code, msg); }
 
@@ -64,8 +69,8 @@ u64* Ctx::scratch_u64(const std::string& name, size_t words) {
 Ctx::~Ctx() {
     cudaSetDevice(device);
     cudaDeviceSynchronize();
-    void* bufs[] = {d_primes, d_psi, d_psi_s, d_ipsi, d_ipsi_s, d_ninv, d_tw, d_itw, d_tw2, d_itw2, d_up_ninv, d_down_ninv, d_resc, d_up_inv, d_up_hat,
-                    d_down_inv, d_down_hat, d_pinv, d_pmod, d_fd_ninv, d_fd_hat, d_fd_minv, d_fd_pq, d_cos, d_sin, d_pow5, d_sk, d_pk, rlk.d};
+    void* bufs[] = {d_primes, d_ninv, d_tw, d_itw, d_tw2, d_itw2, d_up_ninv, d_down_ninv, d_resc, d_resc_w, d_up_hat,
+                    d_down_hat, d_pinv, d_pmod, d_fd_ninv, d_fd_hat, d_fd_minv, d_fd_pq, d_cos, d_sin, d_pow5, d_sk, d_pk, rlk.d};
     for (void* p : bufs)
         if (p) cudaFree(p);
     for (auto& kv : rot)
@@ -140,13 +145,35 @@ static unsigned bit_reverse(unsigned x, int bits) {
 }
 
 static Prime make_prime(u64 q) {
-    Prime p;
+    Prime p{};
     p.q = q;
     p.b = 64 - __builtin_clzll(q);
     p.mu = (u64)(((u128)1 << (2 * p.b)) / q);
     p.one_s = h_shoup(1, q);
-    p.pad = 0;
+    const u64 delta = ((u64)1 << p.b) - q;
+    p.cls = AR_SHOUP;
+    if (p.b == 50 && delta <= ((u64)1 << 26)) p.cls = AR_NEAR50;
+    if (p.b == 60 && delta <= ((u64)1 << 26)) p.cls = AR_NEAR60;
+    p.delta = p.cls == AR_SHOUP ? 0 : (u32)delta;
     return p;
+}
+
+// The two words a product with the constant w < q takes (ntt_core.cuh): near primes the split words of
+// w and 2^32 w mod q, else w and its Shoup companion.
+static ulonglong2 words_at(u64 w, const Prime& p, int at) {
+    return make_ulonglong2(split_word(w, at), split_word(h_mul(w, ((u64)1 << 32) % p.q, p.q), at));
+}
+static void const_words(u64 w, const Prime& p, u64* out) {
+    const ulonglong2 t = p.cls == AR_SHOUP ? make_ulonglong2(w, h_shoup(w, p.q)) : words_at(w, p, nttc::split_at(p.cls));
+    out[0] = t.x;
+    out[1] = t.y;
+}
+// The same for a base-conversion constant.
+static void conv_words(u64 w, const Prime& p, u64* out) {
+    if (p.cls != AR_NEAR50) return const_words(w, p, out);
+    const ulonglong2 t = words_at(w, p, kConvSplit);
+    out[0] = t.x;
+    out[1] = t.y;
 }
 
 // ============================================================================ sampling (SplitMix64 streams)
@@ -233,7 +260,7 @@ static void sample_gaussian(u64 key, const GaussTable& T, int8_t* out, int n) {
 
 static void build_tables(Ctx& c) {
     const int n = c.n, L = c.L, ne = c.n_ext, A = c.alpha;
-    std::vector<u64> psi((size_t)ne * n), psi_s(psi.size()), ipsi(psi.size()), ipsi_s(psi.size());
+    std::vector<u64> psi((size_t)ne * n), ipsi(psi.size());
     std::vector<u64> ninv(2 * ne);
     for (int t = 0; t < ne; t++) {
         u64 q = c.primes[t];
@@ -249,58 +276,58 @@ static void build_tables(Ctx& c) {
             unsigned r = bit_reverse((unsigned)i, c.log_n);
             size_t o = (size_t)t * n + i;
             psi[o] = pw[r];
-            psi_s[o] = h_shoup(pw[r], q);
             ipsi[o] = ipw[r];
-            ipsi_s[o] = h_shoup(ipw[r], q);
         }
         u64 ni = h_inv((u64)n % q, q);
-        ninv[2 * t] = ni;
-        ninv[2 * t + 1] = h_shoup(ni, q);
+        const_words(ni, c.hprimes[t], &ninv[2 * t]);
     }
-    c.d_psi = dupload(psi);
-    c.d_psi_s = dupload(psi_s);
-    c.d_ipsi = dupload(ipsi);
-    c.d_ipsi_s = dupload(ipsi_s);
     c.d_ninv = dupload(ninv);
     std::vector<ulonglong2> tw((size_t)ne * n), itw(tw.size());
     for (size_t i = 0; i < tw.size(); i++) {
-        tw[i] = make_ulonglong2(psi[i], psi_s[i]);
-        itw[i] = make_ulonglong2(ipsi[i], ipsi_s[i]);
+        const Prime& p = c.hprimes[i / n];
+        const int at = nttc::split_at(p.cls);
+        tw[i] = p.cls == AR_SHOUP ? make_ulonglong2(psi[i], h_shoup(psi[i], p.q)) : words_at(psi[i], p, at);
+        itw[i] = p.cls == AR_SHOUP ? make_ulonglong2(ipsi[i], h_shoup(ipsi[i], p.q)) : words_at(ipsi[i], p, at);
     }
     c.d_tw = dupload(tw);
     c.d_itw = dupload(itw);
-    // transposed row-pass tables of the two-pass transform (N >= 2^14)
+    // row-pass tables of the two-pass transform (N >= 2^14): row r of N2 entries; stage s of the row
+    // transform in entries 2^s .. 2^(s+1) - 1, its group grp = t K + k (T = N2 / 16 threads per row, K =
+    // 2^s / T sub-groups per thread) at 2^s + k T + t from stage 4 on, at 2^s + grp before
     c.ntt_s1 = c.log_n >= 14 ? (c.log_n == 15 ? 7 : c.log_n / 2) : 0;
     if (c.ntt_s1) {
-        const int S1 = c.ntt_s1, N1 = 1 << S1, LM2 = c.log_n - S1;
+        const int S1 = c.ntt_s1, N1 = 1 << S1, N2 = n >> S1, T = N2 / 16;
         std::vector<ulonglong2> t2((size_t)ne * n, make_ulonglong2(0, 0)), it2(t2.size(), make_ulonglong2(0, 0));
-        for (int t = 0; t < ne; t++) {
-            size_t o = (size_t)t * n;
-            for (int sp = 0; sp < LM2; sp++)
-                for (int g = 0; g < (1 << sp); g++)
-                    for (int r = 0; r < N1; r++) {
-                        size_t src = (size_t)t * n + ((size_t)1 << (S1 + sp)) + ((size_t)r << sp) + g;
-                        t2[o] = make_ulonglong2(psi[src], psi_s[src]);
-                        it2[o] = make_ulonglong2(ipsi[src], ipsi_s[src]);
-                        o++;
-                    }
-        }
+        for (int t = 0; t < ne; t++)
+            for (int r = 0; r < N1; r++)
+                for (int e = 1; e < N2; e++) {
+                    int sp = 0;
+                    while ((2 << sp) <= e) sp++;
+                    const int at = e - (1 << sp);
+                    const int grp = sp < 4 ? at : (at % T) * ((1 << sp) / T) + at / T;
+                    const size_t src = (size_t)t * n + ((size_t)1 << (S1 + sp)) + ((size_t)r << sp) + grp;
+                    const size_t o = (size_t)t * n + (size_t)r * N2 + e;
+                    t2[o] = tw[src];
+                    it2[o] = itw[src];
+                }
         c.d_tw2 = dupload(t2);
         c.d_itw2 = dupload(it2);
     }
 
     // rescale: q_l^-1 mod q_i
-    std::vector<u64> resc((size_t)2 * (L + 1) * (L + 1), 0);
+    std::vector<u64> resc((size_t)2 * (L + 1) * (L + 1), 0), resc_w(resc.size(), 0);
     for (int l = 1; l <= L; l++)
         for (int i = 0; i < l; i++) {
             u64 v = h_inv(c.primes[l] % c.primes[i], c.primes[i]);
             resc[2 * ((size_t)l * (L + 1) + i)] = v;
             resc[2 * ((size_t)l * (L + 1) + i) + 1] = h_shoup(v, c.primes[i]);
+            const_words(v, c.hprimes[i], &resc_w[2 * ((size_t)l * (L + 1) + i)]);
         }
     c.d_resc = dupload(resc);
+    c.d_resc_w = dupload(resc_w);
 
     // ModUp: per level l, limb i <= l belongs to digit j = i / alpha = [j A, min((j+1)A, l+1))
-    std::vector<u64> up_inv((size_t)2 * (L + 1) * (L + 1), 0);
+    std::vector<u64> up_inv((size_t)(L + 1) * (L + 1), 0);
     std::vector<u64> up_hat((size_t)2 * (L + 1) * (L + 1) * ne, 0);
     for (int l = 0; l <= L; l++)
         for (int i = 0; i <= l; i++) {
@@ -312,47 +339,41 @@ static void build_tables(Ctx& c) {
                 if (i2 != i) hat_i = h_mul(hat_i, c.primes[i2] % qi, qi);
             u64 inv = h_inv(hat_i, qi);
             size_t o = (size_t)l * (L + 1) + i;
-            up_inv[2 * o] = inv;
-            up_inv[2 * o + 1] = h_shoup(inv, qi);
+            up_inv[o] = inv;
             for (int t = 0; t < ne; t++) {
                 u64 p = c.primes[t];
                 u64 h = 1 % p;
                 for (int i2 = lo; i2 < hi; i2++)
                     if (i2 != i) h = h_mul(h, c.primes[i2] % p, p);
-                up_hat[2 * (o * ne + t)] = h;
-                up_hat[2 * (o * ne + t) + 1] = h_shoup(h, p);
+                conv_words(h, c.hprimes[t], &up_hat[2 * (o * ne + t)]);
             }
         }
-    c.d_up_inv = dupload(up_inv);
     c.d_up_hat = dupload(up_hat);
-    std::vector<u64> up_ninv(up_inv.size(), 0);
+    std::vector<u64> up_ninv(2 * up_inv.size(), 0);
     for (int l = 0; l <= L; l++)
         for (int i = 0; i <= l; i++) {
             size_t o = (size_t)l * (L + 1) + i;
             u64 qi = c.primes[i];
-            u64 v = h_mul(up_inv[2 * o], h_inv((u64)n % qi, qi), qi);
-            up_ninv[2 * o] = v;
-            up_ninv[2 * o + 1] = h_shoup(v, qi);
+            u64 v = h_mul(up_inv[o], h_inv((u64)n % qi, qi), qi);
+            const_words(v, c.hprimes[i], &up_ninv[2 * o]);
         }
     c.d_up_ninv = dupload(up_ninv);
 
     // ModDown constants
-    std::vector<u64> dinv(2 * A), dhat((size_t)2 * A * (L + 1)), pinv(2 * (L + 1)), pmod(L + 1);
+    std::vector<u64> dinv(A), dhat((size_t)2 * A * (L + 1)), pinv(2 * (L + 1)), pmod(L + 1);
     for (int k = 0; k < A; k++) {
         u64 pk = c.primes[L + 1 + k];
         u64 h = 1;
         for (int k2 = 0; k2 < A; k2++)
             if (k2 != k) h = h_mul(h, c.primes[L + 1 + k2] % pk, pk);
         u64 inv = h_inv(h, pk);
-        dinv[2 * k] = inv;
-        dinv[2 * k + 1] = h_shoup(inv, pk);
+        dinv[k] = inv;
         for (int i = 0; i <= L; i++) {
             u64 q = c.primes[i];
             u64 hq = 1;
             for (int k2 = 0; k2 < A; k2++)
                 if (k2 != k) hq = h_mul(hq, c.primes[L + 1 + k2] % q, q);
-            dhat[2 * ((size_t)k * (L + 1) + i)] = hq;
-            dhat[2 * ((size_t)k * (L + 1) + i) + 1] = h_shoup(hq, q);
+            conv_words(hq, c.hprimes[i], &dhat[2 * ((size_t)k * (L + 1) + i)]);
         }
     }
     for (int i = 0; i <= L; i++) {
@@ -361,16 +382,13 @@ static void build_tables(Ctx& c) {
         for (int k = 0; k < A; k++) P = h_mul(P, c.primes[L + 1 + k] % q, q);
         pmod[i] = P;
         u64 inv = h_inv(P, q);
-        pinv[2 * i] = inv;
-        pinv[2 * i + 1] = h_shoup(inv, q);
+        const_words(inv, c.hprimes[i], &pinv[2 * i]);
     }
-    c.d_down_inv = dupload(dinv);
     std::vector<u64> dninv(2 * A);
     for (int k = 0; k < A; k++) {
         u64 pk = c.primes[L + 1 + k];
-        u64 v = h_mul(dinv[2 * k], h_inv((u64)n % pk, pk), pk);
-        dninv[2 * k] = v;
-        dninv[2 * k + 1] = h_shoup(v, pk);
+        u64 v = h_mul(dinv[k], h_inv((u64)n % pk, pk), pk);
+        const_words(v, c.hprimes[L + 1 + k], &dninv[2 * k]);
     }
     c.d_down_ninv = dupload(dninv);
     c.d_down_hat = dupload(dhat);
@@ -390,26 +408,21 @@ static void build_tables(Ctx& c) {
                 for (int s2 = 0; s2 < S; s2++)
                     if (s2 != sidx) hat_m = h_mul(hat_m, src(s2) % m, m);
                 const u64 v = h_mul(h_inv(hat_m, m), h_inv((u64)n % m, m), m);
-                fninv[2 * ((size_t)l * S + sidx)] = v;
-                fninv[2 * ((size_t)l * S + sidx) + 1] = h_shoup(v, m);
+                const_words(v, c.hprimes[sidx < A ? L + 1 + sidx : l], &fninv[2 * ((size_t)l * S + sidx)]);
                 for (int i = 0; i < l; i++) {
                     const u64 q = c.primes[i];
                     u64 h = 1;
                     for (int s2 = 0; s2 < S; s2++)
                         if (s2 != sidx) h = h_mul(h, src(s2) % q, q);
-                    const size_t o = 2 * (((size_t)l * S + sidx) * (L + 1) + i);
-                    fhat[o] = h;
-                    fhat[o + 1] = h_shoup(h, q);
+                    conv_words(h, c.hprimes[i], &fhat[2 * (((size_t)l * S + sidx) * (L + 1) + i)]);
                 }
             }
             for (int i = 0; i < l; i++) {
                 const u64 q = c.primes[i];
                 const u64 inv = h_inv(h_mul(pmod[i], c.primes[l] % q, q), q);
-                fminv[2 * ((size_t)l * (L + 1) + i)] = inv;
-                fminv[2 * ((size_t)l * (L + 1) + i) + 1] = h_shoup(inv, q);
+                const_words(inv, c.hprimes[i], &fminv[2 * ((size_t)l * (L + 1) + i)]);
             }
-            fpq[2 * l] = pmod[l];
-            fpq[2 * l + 1] = h_shoup(pmod[l], c.primes[l]);
+            const_words(pmod[l], c.hprimes[l], &fpq[2 * l]);
         }
         c.d_fd_ninv = dupload(fninv);
         c.d_fd_hat = dupload(fhat);

@@ -43,8 +43,6 @@ const char* const ksp::kKsTileNames[ksp::KS_N_TILES] = {"r16", "r8", "r8x"};
 namespace {
 
 using namespace ksp;
-using nttc::reduce4;
-using nttc::shoup_lazy;
 
 [[maybe_unused]] inline unsigned grid1(size_t work) {
     size_t b = (work + 255) / 256;
@@ -278,7 +276,7 @@ void ks_run(Ctx& c, const std::vector<KsItem>& all, int level, const HoistKeys* 
                         r5.push_back(r);
                     }
             CombineArgs cr{d_items, acc, c.d_fd_minv + 2 * (size_t)level * (L + 1), next,
-                           c.d_resc + 2 * (size_t)level * (L + 1)};
+                           c.d_resc_w + 2 * (size_t)level * (L + 1)};
             const KsRow* d_r5 = c.arena.push_vec(r5, s);
             ks_transform<false, LD_CONV, ST_COMBINE_RS>(c, d_r5, (int)r5.size(), cr, K_NTT_FWD, 16.0 * r5.size() * n, s);
             continue;
@@ -414,7 +412,7 @@ void rescale_run(Ctx& c, const std::vector<const u64*>& in, const std::vector<co
                     q.galois = 1;
                     q.src2 = x + (size_t)i * n;
                     q.src3 = prod ? pt[b0 + t] + (size_t)i * n : nullptr;
-                    q.cst2 = c.d_resc + 2 * ((size_t)level * (L + 1) + i);
+                    q.cst2 = c.d_resc_w + 2 * ((size_t)level * (L + 1) + i);
                     q.out2 = out[b0 + t] + (size_t)p * pw + (size_t)i * n;
                     rb.push_back(q);
                 }

@@ -3,6 +3,8 @@
 // last pass of a transform, the pass kernel and its launchers. See ks.cu for the algorithm.
 #pragma once
 
+#include <algorithm>
+
 #include "ks_inner.cuh"
 #include "ntt_core.cuh"
 
@@ -10,16 +12,13 @@ namespace fhe {
 
 namespace ksp {
 
-using nttc::reduce4;
-using nttc::shoup_lazy;
-
 enum LoadMode { LD_PLAIN = 0, LD_GATHER = 1, LD_CONV = 2, LD_AXPY = 3, LD_CENTRED = 4, LD_MUL = 5 };
 enum StoreMode { ST_LAZY = 0, ST_LAST = 1, ST_SCALE = 2, ST_COMBINE = 3, ST_COMBINE_RS = 4, ST_RESCALE = 5 };
 
 struct KsRow {
     u64* dst;        // the row's buffer (N residues)
     const u64* src;  // LD_GATHER: source row; LD_CONV: first source limb (limb stride N)
-    const u64* cst;  // LD_CONV: Shoup pair of the first source limb for this row's prime; ST_SCALE: (w, ws)
+    const u64* cst;  // LD_CONV: constant words of the first source limb for this row's prime; ST_SCALE: words of the factor
     int prime;       // prime index of the row
     int galois;      // LD_GATHER: automorphism applied on load (1 = none)
     int src_cnt;     // LD_CONV: number of source limbs
@@ -27,7 +26,7 @@ struct KsRow {
     int item, half, limb;  // ST_COMBINE(_RS): output item, component and limb
     int pack;              // ST_LAST (forward): store the residue split at bit 25 (key_pack)
     const u64* src2;       // LD_AXPY / LD_MUL: second source row (LD_AXPY: null = none); ST_RESCALE: the input limb
-    const u64* cst2;       // LD_AXPY: Shoup pair of its factor; ST_RESCALE: q_l^-1 mod the row's prime
+    const u64* cst2;       // LD_AXPY: words of its factor; ST_RESCALE: words of q_l^-1 mod the row's prime
     u64* out2;             // ST_RESCALE: output row
     const u64* src3;       // ST_RESCALE: when set, the input limb is src2 (.) src3 (a plaintext product)
 };
@@ -44,306 +43,394 @@ struct HoistKeys {
 struct CombineArgs {
     const KsItem* items;
     const u64* acc;    // [items][2][next][N]
-    const u64* pinv;   // [L+1][2] P^-1 mod q_i (ST_COMBINE) or (P q_l)^-1 mod q_i (ST_COMBINE_RS)
+    const u64* pinv;   // [L+1][2] words of P^-1 mod q_i (ST_COMBINE) or (P q_l)^-1 mod q_i (ST_COMBINE_RS)
     int next;
-    const u64* qlinv;  // ST_COMBINE_RS: [L+1][2] q_l^-1 mod q_i
+    const u64* qlinv;  // ST_COMBINE_RS: [L+1][2] words of q_l^-1 mod q_i
 };
 
-// Per-row constants of the first pass's loads, read once per CTA: the row's prime and, for the base
-// conversion, the Shoup pairs of its (at most kConvMax) source limbs.
+__device__ __forceinline__ ulonglong2 words(const u64* p) { return make_ulonglong2(p[0], p[1]); }
+
+// Base conversion sum_i y_i c_i mod a 50-bit near prime: every c_i as two words split at bit 21, A and B
+// the sums of the low and high partial products (y_i below 2^61: A below 2^55.2, B below 2^63.2 for
+// four sources), folded once at 2^53 = 8 delta. The result, below 2^60.4, enters the forward transform
+// as it is.
+struct ConvSum {
+    u64 A = 0, B = 0;
+    __device__ __forceinline__ void add(u64 y, const ulonglong2& w) {
+        const u32 y0 = (u32)y, y1 = (u32)(y >> 32);
+        A = nttc::mad_wide(y1, (u32)w.y, nttc::mad_wide(y0, (u32)w.x, A));
+        B = nttc::mad_wide(y1, (u32)(w.y >> 32), nttc::mad_wide(y0, (u32)(w.x >> 32), B));
+    }
+    __device__ __forceinline__ u64 value(u32 delta) const {
+        return nttc::mad_wide((u32)(B >> 32), delta << 3, A + ((u64)(u32)B << kConvSplit));
+    }
+};
+
+// Per-row constants of the first pass's loads, read once per row: the words of the (at most kConvMax)
+// source limbs' constants of a base conversion, and the last limb's prime of a centred load.
 constexpr int kConvMax = 4;
 struct RowConst {
-    u64 q, one_s, ql;
-    u64 w[kConvMax], ws[kConvMax];
+    u64 ql;
+    ulonglong2 w[kConvMax];
 };
 
 template <int LOAD>
 __device__ __forceinline__ RowConst row_const(const KsRow& r, const Prime* __restrict__ pr) {
     RowConst c;
-    c.q = pr[r.prime].q;
-    c.one_s = pr[r.prime].one_s;
     c.ql = LOAD == LD_CENTRED ? pr[r.limb].q : 0;
 #pragma unroll
-    for (int i = 0; i < kConvMax; i++) {
-        const bool on = LOAD == LD_CONV && i < r.src_cnt;
-        c.w[i] = on ? r.cst[(size_t)i * r.cst_stride] : 0;
-        c.ws[i] = on ? r.cst[(size_t)i * r.cst_stride + 1] : 0;
-    }
+    for (int i = 0; i < kConvMax; i++)
+        c.w[i] = LOAD == LD_CONV && i < r.src_cnt ? words(r.cst + (size_t)i * r.cst_stride) : make_ulonglong2(0, 0);
     return c;
 }
 
-template <int LOAD>
-__device__ __forceinline__ u64 load_elem(const KsRow& r, size_t k, int log_n, const Prime* __restrict__ pr,
-                                         const RowConst& rc) {
-    if (LOAD == LD_PLAIN) return r.dst[k];
-    if (LOAD == LD_GATHER) return r.src[r.galois == 1 ? (int)k : auto_src((int)k, r.galois, log_n)];
-    if (LOAD == LD_CENTRED) {  // the centred representative of src[k] (mod q_limb) reduced mod the row's prime
-        const u64 ql = rc.ql, v = r.src[k];
-        const bool neg = v > (ql >> 1);
-        const u64 m = nttc::reduce_any(neg ? ql - v : v, rc.q, rc.one_s);
-        return neg ? (m ? rc.q - m : 0) : m;
-    }
-    if (LOAD == LD_MUL) return mul_mod(r.src[k], r.src2[k], pr[r.prime]);
-    if (LOAD == LD_AXPY) {  // src + cst2 * src2 (both reduced)
-        const u64 p = rc.q;
-        u64 v = r.src[k];
-        if (r.src2) v = add_mod(v, mul_shoup(r.src2[k], r.cst2[0], r.cst2[1], p), p);
-        return v;
-    }
-    // LD_CONV: sum of the converted source limbs. For primes below 2^58 the forward transform that
-    // follows runs without intermediate reduction, so the sum stays lazy (each term below 2p, at most
-    // 8 terms, so below 16p; 16 stages add less than 32p: below 48p < 2^64); otherwise fully reduced.
-    // Up to kConvMax sources: every source load is issued before the products (fixed trip count,
-    // predicated), so a thread's loads are in flight together.
-    const u64 p = rc.q;
-    if (r.src_cnt <= kConvMax) {
-        u64 x[kConvMax];
+// LD_CONV: the base conversion of residue k, sum_i src_i[k] c_i, over CNT sources (loads unconditional,
+// all issued before the products; constants in rc) or any number of them (CNT = 0).
+template <int AR, int CNT>
+__device__ __forceinline__ u64 conv_elem(const KsRow& r, size_t k, int log_n, const nttc::Mod<AR>& m, const RowConst& rc) {
+    if constexpr (CNT > 0) {
+        u64 x[CNT];
 #pragma unroll
-        for (int i = 0; i < kConvMax; i++) x[i] = i < r.src_cnt ? r.src[((size_t)i << log_n) + k] : 0;
-        if (p < ((u64)1 << 58)) {
-            u64 lazy = 0;
+        for (int i = 0; i < CNT; i++) x[i] = r.src[((size_t)i << log_n) + k];
+        if constexpr (AR == nttc::AR_NEAR50) {
+            ConvSum s;
 #pragma unroll
-            for (int i = 0; i < kConvMax; i++)
-                if (i < r.src_cnt) lazy += shoup_lazy(x[i], rc.w[i], rc.ws[i], p);
-            return lazy;
+            for (int i = 0; i < CNT; i++) s.add(x[i], rc.w[i]);
+            return s.value(m.delta);
+        } else {
+            u64 acc = m.mul(x[0], rc.w[0]);
+#pragma unroll
+            for (int i = 1; i < CNT; i++) acc = m.fold(acc) + m.mul(x[i], rc.w[i]);
+            return acc;
         }
+    } else {
         u64 acc = 0;
-#pragma unroll
-        for (int i = 0; i < kConvMax; i++)
-            if (i < r.src_cnt) {
-                u64 t = shoup_lazy(x[i], rc.w[i], rc.ws[i], p);
-                t = t >= p ? t - p : t;
-                acc += t;
-                acc = acc >= p ? acc - p : acc;
+        for (int i0 = 0; i0 < r.src_cnt; i0 += kConvMax) {
+            ConvSum s;
+            for (int i = i0; i < min(i0 + kConvMax, r.src_cnt); i++) {
+                const u64 x = r.src[((size_t)i << log_n) + k];
+                const ulonglong2 w = words(r.cst + (size_t)i * r.cst_stride);
+                if constexpr (AR == nttc::AR_NEAR50) s.add(x, w);
+                else acc = m.fold(acc) + m.mul(x, w);
             }
+            if constexpr (AR == nttc::AR_NEAR50) acc += m.fold(s.value(m.delta));
+        }
         return acc;
     }
-    if (p < ((u64)1 << 58) && r.src_cnt <= 8) {
-        u64 lazy = 0;
-        for (int i = 0; i < r.src_cnt; i++) {
-            const u64* c = r.cst + (size_t)i * r.cst_stride;
-            lazy += shoup_lazy(r.src[((size_t)i << log_n) + k], c[0], c[1], p);
-        }
-        return lazy;
-    }
-    u64 acc = 0;
-    for (int i = 0; i < r.src_cnt; i++) {
-        const u64* c = r.cst + (size_t)i * r.cst_stride;
-        u64 t = shoup_lazy(r.src[((size_t)i << log_n) + k], c[0], c[1], p);
-        t = t >= p ? t - p : t;
-        acc += t;
-        acc = acc >= p ? acc - p : acc;
-    }
-    return acc;
+}
+// f is called with the number of sources as a compile-time constant (0: more than kConvMax).
+template <class F>
+__device__ __forceinline__ void with_count(int cnt, F&& f) {
+    if (cnt == 1) f(nttc::Tag<1>{});
+    else if (cnt == 2) f(nttc::Tag<2>{});
+    else if (cnt == 3) f(nttc::Tag<3>{});
+    else if (cnt == 4) f(nttc::Tag<4>{});
+    else f(nttc::Tag<0>{});
 }
 
-template <bool INV, int STORE>
-__device__ __forceinline__ void store_elem(const KsRow& r, size_t k, u64 v, const Prime* __restrict__ prow, u64 q, u64 one_s,
+// Residue k of the row as the transform takes it (LD_CONV: conv_elem): a congruent value, for a forward
+// transform within 2^60.4 (NEAR50, signed), below 16 q (NEAR60) or 8 q (SHOUP); reduced for an inverse one.
+template <int LOAD, int AR>
+__device__ __forceinline__ u64 load_elem(const KsRow& r, size_t k, int log_n, const Prime& P, const nttc::Mod<AR>& m,
+                                         const RowConst& rc) {
+    if constexpr (LOAD == LD_PLAIN) {
+        return r.dst[k];
+    } else if constexpr (LOAD == LD_GATHER) {
+        return r.src[r.galois == 1 ? (int)k : auto_src((int)k, r.galois, log_n)];
+    } else if constexpr (LOAD == LD_CENTRED) {  // the centred representative of src[k] (mod q_limb)
+        const u64 ql = rc.ql, v = r.src[k];
+        const bool neg = v > (ql >> 1);
+        if constexpr (AR == nttc::AR_NEAR50) {
+            return neg ? v - ql : v;  // signed, magnitude at most 2^60
+        } else {
+            const u64 mag = neg ? ql - v : v;
+            const u64 t = nttc::reduce_any(mag, P.q, P.one_s);
+            return neg ? (t ? P.q - t : 0) : t;
+        }
+    } else if constexpr (LOAD == LD_MUL) {
+        return mul_mod(r.src[k], r.src2[k], P);
+    } else {  // LD_AXPY: src + cst2 * src2
+        static_assert(LOAD == LD_AXPY, "load mode");
+        const u64 v = r.src[k];
+        return r.src2 ? m.canon(v + m.mul(r.src2[k], words(r.cst2)), P.one_s) : v;
+    }
+}
+
+// Residue k of the row from the transform's (unreduced) value v.
+template <bool INV, int STORE, int AR>
+__device__ __forceinline__ void store_elem(const KsRow& r, size_t k, u64 v, const Prime& P, const nttc::Mod<AR>& m,
                                            const u64* __restrict__ ninv, const CombineArgs& ca, int log_n) {
+    const u64 q = m.q, one_s = P.one_s;
     if (STORE == ST_LAZY) {
         r.dst[k] = v;
         return;
     }
-    if (STORE == ST_LAST) {
-        if (INV) {
-            u64 t = shoup_lazy(v, ninv[2 * r.prime], ninv[2 * r.prime + 1], q);
-            r.dst[k] = t >= q ? t - q : t;
-        } else {
-            const u64 t = nttc::reduce_any(v, q, one_s);
-            r.dst[k] = r.pack ? key_pack(t) : t;
-        }
+    if (STORE == ST_LAST || STORE == ST_SCALE) {  // inverse: times N^-1, or the row's constant in its place
+        const u64 t = m.canon(INV ? m.mul(v, words(STORE == ST_SCALE ? r.cst : ninv + 2 * r.prime)) : v, one_s);
+        r.dst[k] = r.pack ? key_pack(t) : t;
         return;
     }
+    const u64 t = m.canon(v, one_s);
     if (STORE == ST_RESCALE) {  // forward: out = (x - [x_l]) q_l^-1 with the transformed [x_l] in v
-        const u64 t = nttc::reduce_any(v, q, one_s);
-        const u64 x = r.src3 ? mul_mod(r.src2[k], r.src3[k], *prow) : r.src2[k];
-        r.out2[k] = mul_shoup(sub_mod(x, t, q), r.cst2[0], r.cst2[1], q);
+        const u64 x = r.src3 ? mul_mod(r.src2[k], r.src3[k], P) : r.src2[k];
+        r.out2[k] = m.canon(m.mul(x + q - t, words(r.cst2)), one_s);
         return;
     }
-    if (STORE == ST_SCALE) {  // inverse transforms only: times the row's constant instead of N^-1
-        u64 t = shoup_lazy(v, r.cst[0], r.cst[1], q);
-        r.dst[k] = t >= q ? t - q : t;
-        return;
-    }
+    // out_h = (acc_h - v) P^-1 + add terms (Mod::mul's range and two reduced terms fit 64 bits)
     const KsItem& it = ca.items[r.item];
     const size_t row_off = (size_t)r.limb << log_n;
-    u64 conv = nttc::reduce_any(v, q, one_s);
-    u64 a = ca.acc[((((size_t)r.item * 2 + r.half) * ca.next + r.limb) << log_n) + k];
-    u64 d = a >= conv ? a - conv : a + q - conv;
+    const u64 a = ca.acc[((((size_t)r.item * 2 + r.half) * ca.next + r.limb) << log_n) + k];
+    u64 s = m.mul(a + q - t, words(ca.pinv + 2 * r.limb));
     if (STORE == ST_COMBINE_RS) {
         // fused ModDown + rescale: out_h = (acc_h - conv) (P q_l)^-1 + c_h q_l^-1
         const u64* c_h = r.half == 0 ? it.addI0 : it.addI1;
-        u64 t = mul_shoup(d, ca.pinv[2 * r.limb], ca.pinv[2 * r.limb + 1], q);
-        t = add_mod(t, mul_shoup(c_h[row_off + k], ca.qlinv[2 * r.limb], ca.qlinv[2 * r.limb + 1], q), q);
-        (r.half == 0 ? it.out0 : it.out1)[row_off + k] = t;
-        return;
-    }
-    // ST_COMBINE (forward): out_h = (acc_h - v) * P^-1 + add terms
-    u64 t = shoup_lazy(d, ca.pinv[2 * r.limb], ca.pinv[2 * r.limb + 1], q);
-    t = t >= q ? t - q : t;
-    if (r.half == 0) {
-        if (it.addP0) {
-            int src = it.galois == 1 ? (int)k : auto_src((int)k, (int)it.galois, log_n);
-            t = add_mod(t, it.addP0[row_off + src], q);
-        }
-        if (it.addI0) t = add_mod(t, it.addI0[row_off + k], q);
-        it.out0[row_off + k] = t;
+        s += m.mul(c_h[row_off + k], words(ca.qlinv + 2 * r.limb));
+    } else if (r.half == 0) {
+        if (it.addP0) s += it.addP0[row_off + (it.galois == 1 ? (int)k : auto_src((int)k, (int)it.galois, log_n))];
+        if (it.addI0) s += it.addI0[row_off + k];
     } else {
-        if (it.addI1) t = add_mod(t, it.addI1[row_off + k], q);
-        it.out1[row_off + k] = t;
+        if (it.addI1) s += it.addI1[row_off + k];
     }
+    (r.half == 0 ? it.out0 : it.out1)[row_off + k] = m.canon(s, one_s);
 }
 
-// One NTT pass over a row table (PASS 0: column tiles / single pass; PASS 1: row tiles).
-constexpr int ks_min_blocks(int rb, int threads) {
-    return (rb == 3 ? 1024 : 768) / threads > 0 ? (rb == 3 ? 1024 : 768) / threads : 1;
-}
+// ---------------------------------------------------------------- pass kernels
 
-// LOOSE halves the CTAs per SM the launch bounds ask for, which doubles the registers a thread may use
-// (fewer spills, lower occupancy).
-template <int LOGN, int LOGM, int R, bool INV, int PASS, int LOAD, int STORE, int RB, bool LOOSE = false>
-__global__ void __launch_bounds__(R * (1 << LOGM) / (1 << RB),
-                                  (ks_min_blocks(RB, R * (1 << LOGM) / (1 << RB)) + (LOOSE ? 1 : 0)) / (LOOSE ? 2 : 1))
-ks_ntt_kernel(const KsRow* __restrict__ rows, const Prime* __restrict__ primes, const ulonglong2* __restrict__ tw,
-              const u64* __restrict__ ninv, CombineArgs ca) {
-    constexpr int log_n = LOGN;  // the ring size is a compile-time constant of each launch
-    constexpr int M = 1 << LOGM;
-    constexpr int P = R == 1 ? 1 : R + 1;
-    constexpr int V = 1 << RB;
-    constexpr int T = R * M / V;
+// Rows of a launch: a descriptor table in device memory, or the regular rows of a PolyBatch (plain NTT).
+struct RowTable {
+    const KsRow* rows;
+    __device__ __forceinline__ KsRow get(int i, int) const { return rows[i]; }
+};
+struct RowBatch {
+    PolyBatch pb;
+    __device__ __forceinline__ KsRow get(int i, int log_n) const {
+        const int li = i % pb.n_limbs, rest = i / pb.n_limbs, limb = pb.limb_lo + li;
+        KsRow r{};
+        r.dst = pb.base + (size_t)(rest / pb.n_parts) * pb.item_stride + (size_t)(rest % pb.n_parts) * pb.part_stride +
+                ((size_t)(limb - pb.addr_lo) << log_n);
+        r.prime = pb.prime_of(limb);
+        return r;
+    }
+};
+
+// Whole transform of one row per CTA (rings up to 2^13).
+template <class ROWS, int LOGN, bool INV, int LOAD, int STORE>
+__global__ void __launch_bounds__((1 << LOGN) / 8, 1024 / ((1 << LOGN) / 8))
+single_pass_kernel(ROWS rows, const Prime* __restrict__ primes, const ulonglong2* __restrict__ tw,
+                   const u64* __restrict__ ninv, CombineArgs ca) {
+    constexpr int N = 1 << LOGN, T = N / 8;
     extern __shared__ u64 sm[];
-    const int tid = threadIdx.x;
-    const KsRow r = rows[blockIdx.x];
-    const RowConst rc = row_const<LOAD>(r, primes);
-    const u64 q = primes[r.prime].q;
-    const ulonglong2* W = tw + ((size_t)r.prime << log_n);
-    const int log_n2 = PASS == 0 ? log_n - LOGM : LOGM;
-    const int S1 = log_n - log_n2;
-    const int t0 = blockIdx.y * R;
-    if (PASS == 0 && R > 1) {
-        // column tiles: the first and last register blocks read and write global memory directly
-        constexpr int NB = (LOGM + RB - 1) / RB;
-        const int qq = tid % R, g = tid / R;
-        const int fb = INV ? NB - 1 : 0, lb = INV ? 0 : NB - 1;
-        u64 v[V];
+    const KsRow r = rows.get(blockIdx.x, LOGN);
+    const Prime& P = primes[r.prime];
+    nttc::with_arith(P, [&](auto ar) {
+        const nttc::Mod<decltype(ar)::value> m(P);
+        const RowConst rc = row_const<LOAD>(r, primes);
+        if constexpr (LOAD == LD_CONV) {
+            with_count(r.src_cnt, [&](auto cnt) {
+#pragma unroll 4
+                for (int e = threadIdx.x; e < N; e += T)
+                    sm[e] = conv_elem<decltype(ar)::value, decltype(cnt)::value>(r, e, LOGN, m, rc);
+            });
+        } else {
+#pragma unroll 4
+            for (int e = threadIdx.x; e < N; e += T) sm[e] = load_elem<LOAD>(r, e, LOGN, P, m, rc);
+        }
+        __syncthreads();
+        nttc::single_blocks<LOGN, 0, INV>(sm, tw + ((size_t)r.prime << LOGN), m);
+#pragma unroll 2
+        for (int e = threadIdx.x; e < N; e += T) store_elem<INV, STORE>(r, e, sm[e], P, m, ninv, ca, LOGN);
+    });
+}
+
+// One pass of the two-pass transform of a ring of 2^LOGN = N1 x N2 (N1 rows of N2): PASS 0 transforms
+// columns of N1 = M points (R consecutive columns per CTA), PASS 1 rows of N2 = M points (R rows per CTA).
+// A thread holds 2^RB residues. With RB = 4 and M = 128 or 256 that is two register blocks, so a residue
+// makes one trip through shared memory between its global load and its store (two in a row pass, whose
+// other side is a transposition that keeps the global access coalesced), where radix-8 tiles filled from
+// and drained to shared memory made four; the T = M / 2^RB threads of one row of PASS 1 lie inside a warp,
+// so its exchanges need no CTA barrier.
+//   shared memory: PASS 0 element x of column c at x R + c (plus R per 2^RB elements when R < 16, which
+//   puts the two element runs a half-warp reads on different banks); PASS 1 element x of a row at
+//   x + x / 16, the rows M + M / 16 apart (stride-16 reads hit 16 different bank pairs).
+//   twiddles: PASS 0 the column table (equal for all columns: broadcast loads); PASS 1 with RB = 4 the
+//   table laid out so that the threads of a row read consecutive entries (see Ctx::d_tw2), RB = 3 the
+//   natural table. A row pass's twiddles are as many words as its data, so a CTA takes `per_cta`
+//   consecutive rows of the launch at the same tile and finds them in L1 when the rows share a prime.
+// What bounds it: the 32-bit multiply pipe (ntt_core.cuh) and, in passes whose loads convert, the latency
+// of their loads. Plain forward + inverse transform of 256 rows, N = 2^15 / 2^16 (ms): radix-8 tiles filled
+// from shared memory with Shoup products 0.205 / 0.424, the same with split products 0.176 / 0.372,
+// these passes 0.140 / 0.306; ModUp conversion pass set of 64 top-level inputs 1.032 / 4.66 -> 0.717 / 3.00.
+template <class ROWS, int LOGN, int LOGM, int R, bool INV, int PASS, int LOAD, int STORE, int RB, int MINB>
+__global__ void __launch_bounds__(R * (1 << LOGM) / (1 << RB), MINB)
+pass_kernel(ROWS rows, int n_rows, int per_cta, const Prime* __restrict__ primes, const ulonglong2* __restrict__ tw,
+            const u64* __restrict__ ninv, CombineArgs ca) {
+    constexpr int M = 1 << LOGM, V = 1 << RB, T = M >> RB, NB = (LOGM + RB - 1) / RB;
+    constexpr int LOGN2 = PASS == 0 ? LOGN - LOGM : LOGM;
+    constexpr int S1 = LOGN - LOGN2;
+    extern __shared__ u64 sm_all[];
+    const int lane_q = PASS == 0 ? threadIdx.x % R : threadIdx.x / T;  // column or row of the tile
+    const int g = PASS == 0 ? threadIdx.x / R : threadIdx.x % T;       // thread within the sub-transform
+    const int t0 = blockIdx.y * R + lane_q;                            // column or row of the ring
+    u64* const sm = PASS == 0 ? sm_all + lane_q : sm_all + lane_q * (M + M / 16);
+    auto at = [&](int x) -> u64& { return PASS == 0 ? sm[x * R + (R < 16 ? (x >> RB) * R : 0)] : sm[x + (x >> 4)]; };
+    auto sync = [&] {
+        if (PASS == 0) __syncthreads();
+        else __syncwarp();
+    };
+    auto addr = [&](int x) -> size_t { return PASS == 0 ? (size_t)t0 + ((size_t)x << LOGN2) : ((size_t)t0 << LOGM) + x; };
+    const int i1 = min(n_rows, (int)(blockIdx.x + 1) * per_cta);
+    for (int i = blockIdx.x * per_cta; i < i1; i++) {
+        const KsRow r = rows.get(i, LOGN);
+        const Prime& P = primes[r.prime];
+        const ulonglong2* const W = tw + ((size_t)r.prime << LOGN) + (PASS == 1 && RB == 4 ? (size_t)t0 << LOGM : 0);
+        nttc::with_arith(P, [&](auto ar) {
+            constexpr int AR = decltype(ar)::value;
+            const nttc::Mod<AR> m(P);
+            u64 v[V];
+            // register u holds element g + T u before block 0 and outside the blocks of a row pass (arrangement
+            // -1), block_elem(k, g, u) in block k
+            auto elem = [&](int blk, int u) { return blk < 0 ? g + T * u : nttc::block_elem<LOGM, RB>(blk, g, u); };
+            auto put = [&](int blk) {
 #pragma unroll
-        for (int u = 0; u < V; u++)
-            v[u] = load_elem<LOAD>(r, (size_t)(t0 + qq) + ((size_t)nttc::block_elem<LOGM, RB>(fb, g, u) << log_n2),
-                                   log_n, primes, rc);
-        if (!INV && q < ((u64)1 << 58))
-            nttc::tile_stages<LOGM, R, INV, PASS, false, true, true, RB>(sm, W, q, S1, t0, v);
-        else
-            nttc::tile_stages<LOGM, R, INV, PASS, true, true, true, RB>(sm, W, q, S1, t0, v);
-        const u64 one_s = primes[r.prime].one_s;
+                for (int u = 0; u < V; u++) at(elem(blk, u)) = v[u];
+            };
+            auto take = [&](int blk) {
 #pragma unroll
-        for (int u = 0; u < V; u++)
-            store_elem<INV, STORE>(r, (size_t)(t0 + qq) + ((size_t)nttc::block_elem<LOGM, RB>(lb, g, u) << log_n2), v[u], primes + r.prime,
-                                   q, one_s, ninv, ca, log_n);
-        return;
-    }
-    if (PASS == 0) {
+                for (int u = 0; u < V; u++) v[u] = at(elem(blk, u));
+            };
+            auto exchange = [&](int from, int to) {
+                put(from);
+                sync();
+                take(to);
+                sync();
+            };
+            auto block = [&](auto tag) {
+                constexpr int BLK = decltype(tag)::value, S0 = RB * BLK;
+                const int tb = nttc::block_elem<LOGM, RB>(BLK, g, 0) >> (LOGM - S0);
+                nttc::block_stages<LOGM, RB, BLK, INV, PASS == 0 || BLK != NB - 1>(v, m, [&](int s, int k) {
+                    const int grp = (tb << (s - S0)) + k;
+                    if (PASS == 0) return W[(1 << s) + grp];
+                    if (RB == 4) return W[(1 << s) + (BLK == 0 ? grp : k * T + g)];
+                    return W[(1 << (S1 + s)) + (t0 << s) + grp];
+                });
+            };
+            // loads and stores with arithmetic of their own run in short loops over the thread's own
+            // shared-memory elements: unrolled over the registers they overflow the instruction cache
+            if constexpr (LOAD == LD_CONV) {
+                const RowConst rc = row_const<LOAD>(r, primes);
+                with_count(r.src_cnt, [&](auto cnt) {
+#pragma unroll 8
+                    for (int u = 0; u < V; u++)
+                        at(g + T * u) = conv_elem<AR, decltype(cnt)::value>(r, addr(g + T * u), LOGN, m, rc);
+                });
+                take(-1);
+            } else {
+                const RowConst rc = row_const<LOAD>(r, primes);
+#pragma unroll
+                for (int u = 0; u < V; u++) {
+                    const int x = INV && PASS == 0 ? elem(NB - 1, u) : g + T * u;
+                    v[u] = load_elem<LOAD>(r, addr(x), LOGN, P, m, rc);
+                }
+            }
+            if constexpr (!INV) {
+                block(nttc::Tag<0>{});
+                if constexpr (NB > 1) {
+                    exchange(0, 1);
+                    block(nttc::Tag<1>{});
+                }
+                if constexpr (NB > 2) {
+                    exchange(1, 2);
+                    block(nttc::Tag<2>{});
+                }
+            } else {
+                if (PASS == 1) exchange(-1, NB - 1);
+                if constexpr (NB > 2) {
+                    block(nttc::Tag<2>{});
+                    exchange(2, 1);
+                }
+                if constexpr (NB > 1) {
+                    block(nttc::Tag<1>{});
+                    exchange(1, 0);
+                }
+                block(nttc::Tag<0>{});
+            }
+            if (!INV && PASS == 1) {
+                put(NB - 1);
+                sync();
 #pragma unroll 4
-        for (int e = tid; e < R * M; e += T) {
-            int x = e / R, qq = e % R;
-            sm[x * P + qq] = load_elem<LOAD>(r, (size_t)(t0 + qq) + ((size_t)x << log_n2), log_n, primes, rc);
-        }
-    } else {
-#pragma unroll 4
-        for (int e = tid; e < R * M; e += T) {
-            int x = e & (M - 1), qq = e >> LOGM;
-            sm[x * P + qq] = load_elem<LOAD>(r, ((size_t)(t0 + qq) << LOGM) + x, log_n, primes, rc);
-        }
-    }
-    __syncthreads();
-    if (!INV && q < ((u64)1 << 58)) nttc::tile_stages<LOGM, R, INV, PASS, false, RB>(sm, W, q, S1, t0);
-    else nttc::tile_stages<LOGM, R, INV, PASS, true, RB>(sm, W, q, S1, t0);
-    const u64 one_s = primes[r.prime].one_s;
-    if (PASS == 0) {
-#pragma unroll 4
-        for (int e = tid; e < R * M; e += T) {
-            int x = e / R, c = e % R;
-            store_elem<INV, STORE>(r, (size_t)(t0 + c) + ((size_t)x << log_n2), sm[x * P + c], primes + r.prime, q,
-                                   one_s, ninv, ca, log_n);
-        }
-    } else {
-#pragma unroll 4
-        for (int e = tid; e < R * M; e += T) {
-            int x = e & (M - 1), c = e >> LOGM;
-            store_elem<INV, STORE>(r, ((size_t)(t0 + c) << LOGM) + x, sm[x * P + c], primes + r.prime, q, one_s,
-                                   ninv, ca, log_n);
-        }
+                for (int u = 0; u < V; u++) store_elem<INV, STORE>(r, addr(g + T * u), at(g + T * u), P, m, ninv, ca, LOGN);
+                sync();
+            } else {
+#pragma unroll
+                for (int u = 0; u < V; u++)
+                    store_elem<INV, STORE>(r, addr(!INV ? elem(NB - 1, u) : g + T * u), v[u], P, m, ninv, ca, LOGN);
+            }
+        });
     }
 }
 
-// The fused passes keep radix-8 register blocks: with 16 residues per thread their load and
-// store stages run out of registers (measured slower, unlike the plain transform).
-template <int LOGN, int LOGM, int R, bool INV, int PASS, int LOAD, int STORE, int RB = 3, bool LOOSE = false>
-void launch_pass(const Ctx& c, const KsRow* rows, int n_rows, int tiles, const CombineArgs& ca, int cls, double bytes,
-                 cudaStream_t s) {
-    if (n_rows == 0) return;
-    constexpr int T = R * (1 << LOGM) / (1 << RB);
-    constexpr size_t smem = sizeof(u64) * (1 << LOGM) * (R == 1 ? 1 : R + 1);
-    const ulonglong2* tw = PASS == 1 ? (INV ? c.d_itw2 : c.d_tw2) : (INV ? c.d_itw : c.d_tw);
-    if (smem > 48 * 1024)
-        CK(cudaFuncSetAttribute(ks_ntt_kernel<LOGN, LOGM, R, INV, PASS, LOAD, STORE, RB, LOOSE>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+template <class ROWS, int LOGN, int LOGM, int R, bool INV, int PASS, int LOAD, int STORE, int RB, int TPS>
+void launch_pass(const Ctx& c, const ROWS& rows, int n_rows, const CombineArgs& ca, int cls, double bytes, cudaStream_t s) {
+    constexpr int M = 1 << LOGM, threads = R * M / (1 << RB), tiles = (1 << LOGN) / M / R;
+    constexpr int MINB = TPS / threads > 0 ? TPS / threads : 1;
+    constexpr size_t smem = sizeof(u64) * (PASS == 0 ? R * (M + (R < 16 ? M >> RB : 0)) : R * (M + M / 16));
+    const ulonglong2* tw = PASS == 1 && RB == 4 ? (INV ? c.d_itw2 : c.d_tw2) : (INV ? c.d_itw : c.d_tw);
+    auto kernel = pass_kernel<ROWS, LOGN, LOGM, R, INV, PASS, LOAD, STORE, RB, MINB>;
+    if (smem > 48 * 1024) CK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    // a row pass takes several rows per CTA while at least eight waves of CTAs remain
+    int per_cta = 1;
+    if (PASS == 1) per_cta = (int)std::min<long long>(4, std::max<long long>(1, (long long)n_rows * tiles / (152 * MINB * 8)));
     LaunchScope _ls(c.prof, cls, bytes, s, (double)n_rows * ((size_t)1 << (c.log_n - 1)) * LOGM);
-    ks_ntt_kernel<LOGN, LOGM, R, INV, PASS, LOAD, STORE, RB, LOOSE><<<dim3(n_rows, tiles), T, smem, s>>>(
-        rows, c.d_primes, tw, c.d_ninv, ca);
+    kernel<<<dim3((n_rows + per_cta - 1) / per_cta, tiles), threads, smem, s>>>(rows, n_rows, per_cta, c.d_primes, tw,
+                                                                             c.d_ninv, ca);
     CK(cudaGetLastError());
 }
 
-// A full forward (INV = false) or inverse transform over a row table: the first pass applies
-// LOAD, the last pass applies STORE (single-pass rings do both in one kernel).
-template <bool INV, int LOAD, int STORE, int R, bool LOOSE = false>
-void ks_transform_t(const Ctx& c, const KsRow* rows, int n_rows, const CombineArgs& ca, int cls, double bytes,
-                    cudaStream_t s) {
-    constexpr int FIRST_ST = ST_LAZY;
-    switch (c.log_n) {
-#define SINGLE(LG)                                                                        \
-    case LG:                                                                              \
-        launch_pass<LG, LG, 1, INV, 0, LOAD, STORE, 3>(c, rows, n_rows, 1, ca, cls, bytes, s); \
+template <class ROWS, int LOGN, bool INV, int LOAD, int STORE>
+void launch_single(const Ctx& c, const ROWS& rows, int n_rows, const CombineArgs& ca, int cls, double bytes, cudaStream_t s) {
+    constexpr size_t smem = sizeof(u64) << LOGN;
+    auto kernel = single_pass_kernel<ROWS, LOGN, INV, LOAD, STORE>;
+    if (smem > 48 * 1024) CK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    LaunchScope _ls(c.prof, cls, bytes, s, (double)n_rows * ((size_t)1 << (LOGN - 1)) * LOGN);
+    kernel<<<n_rows, (1 << LOGN) / 8, smem, s>>>(rows, c.d_primes, INV ? c.d_itw : c.d_tw, c.d_ninv, ca);
+    CK(cudaGetLastError());
+}
+
+// A full forward (INV = false) or inverse transform over the rows: the first pass applies LOAD, the
+// last pass applies STORE (rings up to 2^13 do both in one kernel). The column passes of a ring of 2^15
+// have 2^7 points, its row passes 2^8. TPS: threads per SM the register cap of the kernels leaves room for.
+template <class ROWS, bool INV, int LOAD, int STORE, int R, int RB, int TPS>
+void transform_t(const Ctx& c, const ROWS& rows, int n_rows, const CombineArgs& ca, int cls, double bytes, cudaStream_t s) {
+    if (n_rows == 0) return;
+    if constexpr (R == 16 && RB == 4) {  // single-pass rings: one shape, instantiated with the first one
+        switch (c.log_n) {
+            case 9: launch_single<ROWS, 9, INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s); return;
+            case 10: launch_single<ROWS, 10, INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s); return;
+            case 11: launch_single<ROWS, 11, INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s); return;
+            case 12: launch_single<ROWS, 12, INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s); return;
+            case 13: launch_single<ROWS, 13, INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s); return;
+            default: break;
+        }
+    }
+#define TWO(LG, LC)                                                                                              \
+    case LG:                                                                                                     \
+        launch_pass<ROWS, LG, INV ? LG - LC : LC, R, INV, INV ? 1 : 0, LOAD, ST_LAZY, RB, TPS>(c, rows, n_rows, ca, cls, bytes, s); \
+        launch_pass<ROWS, LG, INV ? LC : LG - LC, R, INV, INV ? 0 : 1, LD_PLAIN, STORE, RB, TPS>(c, rows, n_rows, ca, cls, bytes, s); \
         return;
-        SINGLE(9)
-        SINGLE(10)
-        SINGLE(11)
-        SINGLE(12)
-        SINGLE(13)
-#undef SINGLE
-        case 14:
-            if (!INV) {
-                launch_pass<14, 7, R, false, 0, LOAD, FIRST_ST, 3, LOOSE>(c, rows, n_rows, 128 / R, ca, cls, bytes, s);
-                launch_pass<14, 7, R, false, 1, LD_PLAIN, STORE, 3, LOOSE>(c, rows, n_rows, 128 / R, ca, cls, bytes, s);
-            } else {
-                launch_pass<14, 7, R, true, 1, LOAD, FIRST_ST, 3, LOOSE>(c, rows, n_rows, 128 / R, ca, cls, bytes, s);
-                launch_pass<14, 7, R, true, 0, LD_PLAIN, STORE, 3, LOOSE>(c, rows, n_rows, 128 / R, ca, cls, bytes, s);
-            }
-            return;
-        case 15:
-            if (!INV) {
-                launch_pass<15, 7, R, false, 0, LOAD, FIRST_ST, 3, LOOSE>(c, rows, n_rows, 256 / R, ca, cls, bytes, s);
-                launch_pass<15, 8, R, false, 1, LD_PLAIN, STORE, 3, LOOSE>(c, rows, n_rows, 128 / R, ca, cls, bytes, s);
-            } else {
-                launch_pass<15, 8, R, true, 1, LOAD, FIRST_ST, 3, LOOSE>(c, rows, n_rows, 128 / R, ca, cls, bytes, s);
-                launch_pass<15, 7, R, true, 0, LD_PLAIN, STORE, 3, LOOSE>(c, rows, n_rows, 256 / R, ca, cls, bytes, s);
-            }
-            return;
-        case 16:
-            if (!INV) {
-                launch_pass<16, 8, R, false, 0, LOAD, FIRST_ST, 3, LOOSE>(c, rows, n_rows, 256 / R, ca, cls, bytes, s);
-                launch_pass<16, 8, R, false, 1, LD_PLAIN, STORE, 3, LOOSE>(c, rows, n_rows, 256 / R, ca, cls, bytes, s);
-            } else {
-                launch_pass<16, 8, R, true, 1, LOAD, FIRST_ST, 3, LOOSE>(c, rows, n_rows, 256 / R, ca, cls, bytes, s);
-                launch_pass<16, 8, R, true, 0, LD_PLAIN, STORE, 3, LOOSE>(c, rows, n_rows, 256 / R, ca, cls, bytes, s);
-            }
-            return;
+    switch (c.log_n) {
+        TWO(14, 7)
+        TWO(15, 7)
+        TWO(16, 8)
         default: fail(FHE_ERR_INVALID_ARG, "unsupported ring degree");
     }
+#undef TWO
 }
 
 // The tile shapes of the fused passes the autotuner chooses between (family "ks_pass"): rows or
-// columns per tile of the two-pass rings (r8x: 8 with the register cap of LOOSE launch bounds); every
-// shape computes the same bits. Each shape's instantiations live in a translation unit of their own
+// columns per tile of the two-pass rings, 16 residues per thread under a cap of 64 registers (r8x: 8 rows
+// with 80 registers: fewer spills, a quarter fewer threads per SM); every shape computes the same bits.
+// The exact rescale of 64 ciphertexts at N = 2^15 / 2^16 (ms): r16 0.355 / 1.12, r8 0.355 / 1.10, r8x
+// 0.394 / 1.25; under 80 registers r16 took 0.396 / 1.25 (the loads' latency needs the warps). Each shape's instantiations live in a translation unit of their own
 // (ks_pass16.cu, ks_pass8.cu, ks_pass8x.cu).
 enum KsTile { KS_R16 = 0, KS_R8, KS_R8X, KS_N_TILES };
 extern const char* const kKsTileNames[KS_N_TILES];
@@ -373,7 +460,8 @@ void ks_transform_r8x(const Ctx& c, const KsRow* rows, int n_rows, const Combine
 template <bool INV, int LOAD, int STORE>
 void ks_transform(const Ctx& c, const KsRow* rows, int n_rows, const CombineArgs& ca, int cls, double bytes,
                   cudaStream_t s) {
-    if (c.tune.ks == KS_R8) ks_transform_r8<INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s);
+    if (c.log_n < 14) ks_transform_r16<INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s);
+    else if (c.tune.ks == KS_R8) ks_transform_r8<INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s);
     else if (c.tune.ks == KS_R8X) ks_transform_r8x<INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s);
     else ks_transform_r16<INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s);
 }

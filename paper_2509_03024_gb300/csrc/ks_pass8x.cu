@@ -9,7 +9,7 @@ namespace ksp {
 template <bool INV, int LOAD, int STORE>
 void ks_transform_r8x(const Ctx& c, const KsRow* rows, int n_rows, const CombineArgs& ca, int cls, double bytes,
                      cudaStream_t s) {
-    ks_transform_t<INV, LOAD, STORE, 8, true>(c, rows, n_rows, ca, cls, bytes, s);
+    transform_t<RowTable, INV, LOAD, STORE, 8, 4, 768>(c, RowTable{rows}, n_rows, ca, cls, bytes, s);
 }
 
 #define INST(I, L, S)                                                                                   \

@@ -1,6 +1,6 @@
-// ntt_core.cuh — butterfly arithmetic and the register-blocked tile stages
-// shared by the plain NTT launches (ntt.cu) and the fused key-switch passes
-// (ks.cu). See ntt.cu for the decomposition and the lazy value ranges.
+// ntt_core.cuh — butterfly arithmetic and the register-blocked stages shared by
+// the plain NTT launches (ntt.cu) and the fused key-switch passes (ks.cu). See
+// ntt.cu for the decomposition.
 #pragma once
 
 #include "core.cuh"
@@ -8,10 +8,125 @@
 namespace fhe {
 namespace nttc {
 
-// Residues per thread of the plain two-pass NTT tiles: 2^kTileRB (register blocks of kTileRB
-// stages). Radix-16 blocks halve the shared-memory exchanges of the plain transform (1 GiB
-// forward at N = 2^15: 1.71 -> 1.52 ms; inverse 1.93 -> 1.74 ms).
-constexpr int kTileRB = 4;
+// Arithmetic of the transforms and of products with constants, a property of the prime (Prime::cls,
+// uniform in a CTA). What bounds the transforms is the 32-bit multiply pipe: a mad.wide.u32 holds it
+// for four cycles per warp, a 32-bit mad.lo for two, so the products are formed from as few wide
+// multiplies as possible.
+//
+// Near primes, q = 2^b - delta with delta <= 2^26, b = 50 or 60 (the library's primes are the largest
+// of their size that are 1 mod 2N, so this is the usual case). For a constant w the tables hold W0 = w
+// and W1 = 2^32 w mod q, so y w = y0 W0 + y1 W1 (mod q) for any y = y0 + 2^32 y1. Both are split at bit
+// `at`: A = y0 W0l + y1 W1l and B = y0 W0h + y1 W1h need no carries, the product is A + 2^at B, and
+// 2^(32 + at) = 2^(32 + at - b) delta (mod q) folds the high word of B back in with one multiply. Six
+// wide multiplies in all, where a Shoup product takes four wide ones for its quotient and two wide and
+// four narrow ones for its low products.
+//   AR_NEAR50  at = 20, y and the product signed: |y w| < T = 1.54 2^58. With 64 bits for a 50-bit prime
+//              nothing is reduced between the stages of a forward transform (each adds at most T:
+//              below 2^60.4 + 16 T < 2^63 at the end), and signed differences need no multiple of q;
+//              the inverse folds every value once per register block
+//   AR_NEAR60  at = 29, unsigned: y w < 2^62 + 2^61 + 2^59 < 7 q; values stay below 16 q < 2^64 with the
+//              first operand folded in every other forward stage, the sum in every inverse one
+//   AR_SHOUP   any prime up to 61 bits: Shoup products with a quotient from the three upper partial
+//              products (at most two below the true one), y w < 4 q; values below 8 q, the first
+//              operand of each butterfly brought below 4 q
+// Register-only rate of the forward butterfly (GB300, 10^9 per second, unrolled radix-8 blocks): Shoup
+// with the exact quotient 998, NEAR50 1420 (13 instructions); the same with B's low word shifted by
+// shift and add 1290, with unsigned values and a multiple of q in the difference 1120.
+enum Arith { AR_SHOUP = 0, AR_NEAR50 = 1, AR_NEAR60 = 2 };
+__host__ __device__ constexpr int split_at(int ar) { return ar == AR_NEAR50 ? 20 : 29; }
+
+__device__ __forceinline__ u64 mul_wide(u32 a, u32 b) {
+    u64 r;
+    asm("mul.wide.u32 %0, %1, %2;" : "=l"(r) : "r"(a), "r"(b));
+    return r;
+}
+__device__ __forceinline__ u64 mad_wide(u32 a, u32 b, u64 c) {
+    u64 r;
+    asm("mad.wide.u32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+    return r;
+}
+// the same with both factors signed (b is below 2^31 here, so only a's sign matters)
+__device__ __forceinline__ u64 mad_wide_s(u32 a, u32 b, u64 c) {
+    u64 r;
+    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+    return r;
+}
+
+// Constants of one prime's arithmetic.
+template <int AR>
+struct Mod {
+    u64 q;
+    u64 K;      // multiple of q: 2^13 q (NEAR50: makes any signed value non-negative), 7 q (NEAR60), 4 q (SHOUP)
+    u32 delta;  // near primes
+    __device__ __forceinline__ explicit Mod(const Prime& p) : q(p.q) {
+        K = AR == AR_NEAR50 ? p.q << 13 : AR == AR_NEAR60 ? p.q * 7 : p.q << 2;
+        delta = p.delta;
+    }
+    // y w mod q for any y (NEAR50: signed), w a constant's two words; ranges above
+    __device__ __forceinline__ u64 mul(u64 y, const ulonglong2& w) const {
+        const u32 y0 = (u32)y, y1 = (u32)(y >> 32);
+        const u32 a0 = (u32)w.x, a1 = (u32)(w.x >> 32), b0 = (u32)w.y, b1 = (u32)(w.y >> 32);
+        if constexpr (AR == AR_SHOUP) {
+            const u64 c0 = mul_wide(y0, b1), c1 = mul_wide(y1, b0);
+            const u64 qh = mad_wide(y1, b1, (c0 >> 32) + (c1 >> 32));
+            return y * w.x - qh * q;
+        } else if constexpr (AR == AR_NEAR50) {
+            const u64 A = mad_wide_s(y1, b0, mul_wide(y0, a0));
+            const u64 B = mad_wide_s(y1, b1, mul_wide(y0, a1));
+            return mad_wide_s((u32)(B >> 32), delta << 2, mad_wide((u32)B, 1u << 20, A));
+        } else {
+            const u64 A = mad_wide(y1, b0, mul_wide(y0, a0));
+            const u64 B = mad_wide(y1, b1, mul_wide(y0, a1));
+            return mad_wide((u32)(B >> 32), delta << 1, mad_wide((u32)B, 1u << 29, A));
+        }
+    }
+    // a congruent value: NEAR50 any signed v to (-2^39, 2^50 + 2^39), NEAR60 any v below 2^60 + 2^30,
+    // SHOUP v < 8 q below 4 q
+    __device__ __forceinline__ u64 fold(u64 v) const {
+        if constexpr (AR == AR_SHOUP) return v >= K ? v - K : v;
+        else if constexpr (AR == AR_NEAR50) return mad_wide_s((u32)((i64)v >> 50), delta, v & (((u64)1 << 50) - 1));
+        else return mad_wide((u32)(v >> 60), delta, v & (((u64)1 << 60) - 1));
+    }
+    // any v in the ranges above reduced to [0, q)
+    __device__ __forceinline__ u64 canon(u64 v, u64 one_s) const {
+        if constexpr (AR == AR_SHOUP) {
+            v -= __umul64hi(v, one_s) * q;
+        } else if constexpr (AR == AR_NEAR50) {
+            v += K;  // in [0, 2^64)
+            v = mad_wide((u32)(v >> 50), delta, v & (((u64)1 << 50) - 1));
+        } else {
+            v = fold(v);
+        }
+        const u64 d = v - q;  // v < 2 q < 2^62
+        return (i64)d < 0 ? v : d;
+    }
+    // Forward Cooley-Tukey butterfly X <- X + W Y, Y <- X - W Y, in the i-th stage of a register block.
+    __device__ __forceinline__ void ct(u64& x, u64& y, const ulonglong2& w, int i) const {
+        const u64 t = mul(y, w);
+        if constexpr (AR == AR_NEAR50) {
+            y = x - t;
+            x += t;
+        } else {
+            const u64 a = AR == AR_SHOUP || (i & 1) == 0 ? fold(x) : x;
+            x = a + t;
+            y = a + K - t;
+        }
+    }
+    // Inverse Gentleman-Sande butterfly X <- X + Y, Y <- (X - Y) W. NEAR50: the block's inputs were folded,
+    // so magnitudes are below 2^51, T, 2 T, 4 T before its four stages and 8 T < 2^63 after them. NEAR60
+    // and SHOUP: values below 7 q, 4 q.
+    __device__ __forceinline__ void gs(u64& x, u64& y, const ulonglong2& w) const {
+        if constexpr (AR == AR_NEAR50) {
+            const u64 d = x - y;
+            x += y;
+            y = mul(d, w);
+        } else {
+            const u64 d = x + K - y;
+            x = fold(x + y);
+            y = mul(d, w);
+        }
+    }
+};
 
 // Shoup product without the final correction: a * w mod q in [0, 2q) for any a < 2^64.
 __device__ __forceinline__ u64 shoup_lazy(u64 a, u64 w, u64 ws, u64 q) {
@@ -19,37 +134,10 @@ __device__ __forceinline__ u64 shoup_lazy(u64 a, u64 w, u64 ws, u64 q) {
     return a * w - qh * q;
 }
 
-// Forward CT butterfly: X <- X + W Y, Y <- X - W Y with W Y in [0, 2q) (lazy).
-// RED: inputs in [0, 4q), X first reduced below 2q, outputs in [0, 4q).
-// !RED: no reduction; each stage adds less than 2q, so after s stages from [0, q)
-//       values are below (2s + 1) q (used for q < 2^58 and at most 16 stages).
-template <bool RED>
-__device__ __forceinline__ void ct_bfly(u64& x, u64& y, u64 w, u64 ws, u64 q, u64 q2) {
-    u64 a = RED ? (x >= q2 ? x - q2 : x) : x;
-    u64 t = shoup_lazy(y, w, ws, q);
-    x = a + t;
-    y = a + q2 - t;
-}
-
 // Any 64-bit value reduced to [0, q): a lazy Shoup product by 1, then one correction.
 __device__ __forceinline__ u64 reduce_any(u64 x, u64 q, u64 one_s) {
     u64 t = x - __umul64hi(x, one_s) * q;
     return t >= q ? t - q : t;
-}
-
-// Inverse GS butterfly on values in [0, 2q): X <- X + Y, Y <- (X - Y) W (outputs in [0, 2q)).
-__device__ __forceinline__ void gs_bfly(u64& x, u64& y, u64 w, u64 ws, u64 q, u64 q2) {
-    u64 s = x + y;
-    s = s >= q2 ? s - q2 : s;
-    u64 d = x + q2 - y;
-    x = s;
-    y = shoup_lazy(d, w, ws, q);
-}
-
-__device__ __forceinline__ u64 reduce4(u64 x, u64 q) {
-    u64 q2 = q << 1;
-    x = x >= q2 ? x - q2 : x;
-    return x >= q ? x - q : x;
 }
 
 // Element x (within its sub-transform) that register u of the 2^RB-element group g holds in
@@ -63,90 +151,64 @@ __device__ __forceinline__ int block_elem(int blk, int g, int u) {
     return (g / d) * ((1 << RB) * d) + (g % d) + u * d;
 }
 
-// Butterfly stages of one tile: R sub-transforms of M = 2^LOGM points, element x of
-// sub-transform q at sm[x * P + q] between register blocks. Each thread owns V = 2^RB values and
-// runs RB stages in registers per block. PASS 0: column transforms (stages [0, LOGM), twiddles
-// W[2^s + group]); PASS 1: row transforms (stages [S1, S1 + LOGM), transposed twiddles, tile
-// rows t0..t0+R-1).
-// IN_REG: the first block takes its values from v (the caller loaded the elements
-// block_elem(first block, g, u) from global memory) instead of from sm; otherwise the caller
-// fills sm and synchronises before. OUT_REG: the last block leaves its values in v (elements
-// block_elem(last block, g, u)) and neither stores nor synchronises; otherwise the result is in
-// sm after a final __syncthreads(). The first block is 0 (forward) or NB - 1 (inverse).
-template <int LOGM, int R, bool INV, int PASS, bool RED = true, bool IN_REG = false, bool OUT_REG = false,
-          int RB = 3>
-__device__ __forceinline__ void tile_stages(u64* sm, const ulonglong2* __restrict__ W, u64 q, int S1, int t0,
-                                            u64 (&v)[1 << RB]) {
-    constexpr int M = 1 << LOGM;
-    constexpr int V = 1 << RB;
-    constexpr int P = R == 1 ? 1 : R + 1;
-    const int tid = threadIdx.x;
-    const u64 q2 = q << 1;
-    const int qq = tid % R;  // sub-transform of this thread
-    const int g = tid / R;   // V-element group within the sub-transform
-    const int row_off = PASS == 1 ? t0 + qq : 0;
-
-    // register blocks of stages; forward runs stages 0..LOGM-1, inverse LOGM-1..0
-    constexpr int NB = (LOGM + RB - 1) / RB;
+// Butterfly stages of one register block of a transform of M = 2^LOGM points: the 2^RB values of
+// thread group g, elements block_elem(BLK, g, u), through stages [RB BLK, min(RB BLK + RB, LOGM))
+// (forward ascending, inverse descending). tw(s, k) returns the twiddle of this thread's k-th
+// sub-group at stage s (a block of b stages over 2^RB values holds 2^(RB-b+j) sub-groups at its stage j).
+// FOLD: the inverse NEAR50 values may be large (every block but the first after reduced inputs).
+template <int LOGM, int RB, int BLK, bool INV, bool FOLD, int AR, class TW>
+__device__ __forceinline__ void block_stages(u64 (&v)[1 << RB], const Mod<AR>& m, TW&& tw) {
+    constexpr int V = 1 << RB, S0 = RB * BLK;
+    constexpr int b = (LOGM - S0) < RB ? (LOGM - S0) : RB;
+    if (INV && FOLD && AR == AR_NEAR50) {
 #pragma unroll
-    for (int bi = 0; bi < NB; bi++) {
-        // forward: block bi covers stages [RB bi, min(RB bi + RB, LOGM));
-        // inverse: the same blocks in reverse order, stages inside a block descending
-        const int blk_id = INV ? NB - 1 - bi : bi;
-        const int s0 = RB * blk_id;
-        const int b = (LOGM - s0) < RB ? (LOGM - s0) : RB;
-        const int d = M >> (s0 + b);
-        const int base = (g / d) * (V * d) + (g % d);
-        if (!(IN_REG && bi == 0)) {
+        for (int u = 0; u < V; u++) v[u] = m.fold(v[u]);
+    }
 #pragma unroll
-            for (int u = 0; u < V; u++) v[u] = sm[(base + u * d) * P + qq];
-        }
-        // Twiddle of the pair (u, u + dist) at block stage j: its group index at stage s0 + j is
-        // tb * 2^j + (u >> (b - j)), with tb = base >> (LOGM - s0) the thread's group at s0.
-        const int tb = base >> (LOGM - s0);
-        if (!INV) {
+    for (int i = 0; i < b; i++) {
+        const int j = INV ? b - 1 - i : i;
+        const int dist = 1 << (b - 1 - j);
 #pragma unroll
-            for (int j = 0; j < RB; j++) {
-                if (j >= b) break;
-                const int s = s0 + j;
-                const int dist = 1 << (b - 1 - j);
-#pragma unroll
-                for (int u = 0; u < V; u++) {
-                    if (u & dist) continue;
-                    const int grp = (tb << j) + (u >> (b - j));
-                    const int wi = PASS == 1 ? ((((1 << s) - 1 + grp)) << S1) + row_off : (1 << s) + grp;
-                    const ulonglong2 w = W[wi];
-                    ct_bfly<RED>(v[u], v[u + dist], w.x, w.y, q, q2);
-                }
-            }
-        } else {
-#pragma unroll
-            for (int j = RB - 1; j >= 0; j--) {
-                if (j >= b) continue;
-                const int s = s0 + j;
-                const int dist = 1 << (b - 1 - j);
-#pragma unroll
-                for (int u = 0; u < V; u++) {
-                    if (u & dist) continue;
-                    const int grp = (tb << j) + (u >> (b - j));
-                    const int wi = PASS == 1 ? ((((1 << s) - 1 + grp)) << S1) + row_off : (1 << s) + grp;
-                    const ulonglong2 w = W[wi];
-                    gs_bfly(v[u], v[u + dist], w.x, w.y, q, q2);
-                }
-            }
-        }
-        if (!(OUT_REG && bi == NB - 1)) {
-#pragma unroll
-            for (int u = 0; u < V; u++) sm[(base + u * d) * P + qq] = v[u];
-            __syncthreads();
+        for (int u = 0; u < V; u++) {
+            if (u & dist) continue;
+            const ulonglong2 w = tw(S0 + j, u >> (b - j));
+            if (INV) m.gs(v[u], v[u + dist], w);
+            else m.ct(v[u], v[u + dist], w, i);
         }
     }
 }
 
-template <int LOGM, int R, bool INV, int PASS, bool RED = true, int RB = 3>
-__device__ __forceinline__ void tile_stages(u64* sm, const ulonglong2* __restrict__ W, u64 q, int S1, int t0) {
-    u64 v[1 << RB];
-    tile_stages<LOGM, R, INV, PASS, RED, false, false, RB>(sm, W, q, S1, t0, v);
+// f is called with the arithmetic of prime p as a compile-time constant.
+template <int V>
+struct Tag {
+    static constexpr int value = V;
+};
+template <class F>
+__device__ __forceinline__ void with_arith(const Prime& p, F&& f) {
+    if (p.cls == AR_NEAR50) f(Tag<AR_NEAR50>{});
+    else if (p.cls == AR_NEAR60) f(Tag<AR_NEAR60>{});
+    else f(Tag<AR_SHOUP>{});
+}
+
+// The whole transform of one row of M = 2^LOGM points held in sm (element x at sm[x]) by M / 8
+// threads, radix-8 register blocks between shared-memory exchanges (single-pass rings). The caller
+// fills sm and synchronises before; the result is in sm after a final __syncthreads().
+template <int LOGM, int BI, bool INV, int AR>
+__device__ __forceinline__ void single_blocks(u64* sm, const ulonglong2* __restrict__ W, const Mod<AR>& m) {
+    constexpr int RB = 3, V = 8, NB = (LOGM + RB - 1) / RB;
+    if constexpr (BI < NB) {
+        constexpr int BLK = INV ? NB - 1 - BI : BI, S0 = RB * BLK;
+        const int g = threadIdx.x;
+        u64 v[V];
+#pragma unroll
+        for (int u = 0; u < V; u++) v[u] = sm[block_elem<LOGM, RB>(BLK, g, u)];
+        const int tb = block_elem<LOGM, RB>(BLK, g, 0) >> (LOGM - S0);  // the thread's first group at stage S0
+        block_stages<LOGM, RB, BLK, INV, (BI > 0)>(v, m, [&](int s, int k) { return W[(1 << s) + (tb << (s - S0)) + k]; });
+#pragma unroll
+        for (int u = 0; u < V; u++) sm[block_elem<LOGM, RB>(BLK, g, u)] = v[u];
+        __syncthreads();
+        single_blocks<LOGM, BI + 1, INV>(sm, W, m);
+    }
 }
 
 }  // namespace nttc

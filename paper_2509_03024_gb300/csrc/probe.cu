@@ -2,10 +2,9 @@
 //
 // The batched NTT passes are bound by the integer pipe, not by HBM. To put a
 // measured ceiling beside the one derived from lane counts and clocks, this
-// kernel runs exactly the forward transform's arithmetic — lazy Shoup
-// Cooley-Tukey butterflies without intermediate reduction (values stay below
-// (2s+1)q after s stages, as in the transform for primes below 2^58), three
-// stages per radix-8 block, a full reduction after every 15 stages — on
+// kernel runs exactly the forward transform's arithmetic for the context's
+// first prime (Cooley-Tukey butterflies with that prime's arithmetic, ntt_core.cuh),
+// three stages per radix-8 block, a full reduction after every 15 stages, on
 // values held in registers, with no shared-memory exchange, no twiddle loads
 // inside the loop and no global traffic. Its butterflies per second are what
 // the transform could reach if moving data were free.
@@ -20,10 +19,12 @@ namespace {
 constexpr int kProbeThreads = 256;
 constexpr int kProbeBlocksPerSm = 3;
 
+template <int AR>
 __global__ void __launch_bounds__(kProbeThreads, kProbeBlocksPerSm)
 bfly_probe_kernel(u64* out, const ulonglong2* __restrict__ tw, const Prime* __restrict__ pr, int prime, int log_n,
                   int reps) {
-    const u64 q = pr[prime].q, one_s = pr[prime].one_s, q2 = q << 1;
+    const u64 q = pr[prime].q, one_s = pr[prime].one_s;
+    const nttc::Mod<AR> m(pr[prime]);
     const int tid = blockIdx.x * blockDim.x + threadIdx.x;
     const int mask = (1 << log_n) - 1;
     const ulonglong2* W = tw + ((size_t)prime << log_n);
@@ -37,15 +38,15 @@ bfly_probe_kernel(u64* out, const ulonglong2* __restrict__ tw, const Prime* __re
 #pragma unroll
         for (int blk = 0; blk < 5; blk++) {  // 15 stages
 #pragma unroll
-            for (int u = 0; u < 4; u++) nttc::ct_bfly<false>(v[u], v[u + 4], w[0].x, w[0].y, q, q2);
+            for (int u = 0; u < 4; u++) m.ct(v[u], v[u + 4], w[0], 0);
 #pragma unroll
             for (int u = 0; u < 8; u++)
-                if (!(u & 2)) nttc::ct_bfly<false>(v[u], v[u + 2], w[1 + (u >> 2)].x, w[1 + (u >> 2)].y, q, q2);
+                if (!(u & 2)) m.ct(v[u], v[u + 2], w[1 + (u >> 2)], 1);
 #pragma unroll
-            for (int u = 0; u < 8; u += 2) nttc::ct_bfly<false>(v[u], v[u + 1], w[3 + (u >> 1)].x, w[3 + (u >> 1)].y, q, q2);
+            for (int u = 0; u < 8; u += 2) m.ct(v[u], v[u + 1], w[3 + (u >> 1)], 2);
         }
 #pragma unroll
-        for (int u = 0; u < 8; u++) v[u] = nttc::reduce_any(v[u], q, one_s);
+        for (int u = 0; u < 8; u++) v[u] = m.canon(v[u], one_s);
     }
     u64 acc = 0;
 #pragma unroll
@@ -75,10 +76,13 @@ extern "C" int fhe_probe_butterfly_rate(fhe_ctx* ctx, int32_t reps, double* gbfl
         CK(cudaEventCreate(&e0));
         CK(cudaEventCreate(&e1));
         // one warm-up launch, then the timed one
-        bfly_probe_kernel<<<blocks, kProbeThreads>>>(out, c.d_tw, c.d_primes, 0, c.log_n, 1);
+        auto kernel = c.hprimes[0].cls == nttc::AR_NEAR50   ? bfly_probe_kernel<nttc::AR_NEAR50>
+                      : c.hprimes[0].cls == nttc::AR_NEAR60 ? bfly_probe_kernel<nttc::AR_NEAR60>
+                                                            : bfly_probe_kernel<nttc::AR_SHOUP>;
+        kernel<<<blocks, kProbeThreads>>>(out, c.d_tw, c.d_primes, 0, c.log_n, 1);
         CK(cudaGetLastError());
         CK(cudaEventRecord(e0));
-        bfly_probe_kernel<<<blocks, kProbeThreads>>>(out, c.d_tw, c.d_primes, 0, c.log_n, reps);
+        kernel<<<blocks, kProbeThreads>>>(out, c.d_tw, c.d_primes, 0, c.log_n, reps);
         CK(cudaGetLastError());
         CK(cudaEventRecord(e1));
         CK(cudaEventSynchronize(e1));
