@@ -48,6 +48,7 @@ struct Prime {
     u32 cls;    // arithmetic of the transforms and of products with constants (Arith in ntt_core.cuh)
     u32 delta;  // near primes: 2^b - q
     u32 pad;
+    u64 w64[2], w50[2];  // words of 2^64 and 2^50 mod q (near primes)
 };
 
 // Constants modulo a near prime (q = 2^b - delta) are kept as two words W0 = w and W1 = 2^32 w mod q,
@@ -147,7 +148,7 @@ inline PolyBatch poly_batch(u64* base, size_t item_stride, size_t part_stride, i
 
 // ----------------------------------------------------------------------------- keys
 
-// Hybrid key-switching key: [dnum_top][2 (b, a)][n_ext][N], evaluation domain.
+// Hybrid key-switching key: [dnum_top][n_ext][N][2 (b, a)], evaluation domain.
 struct EvalKey {
     u64* d = nullptr;
     int galois = 0;  // 0 for the relinearisation key

@@ -144,6 +144,16 @@ static unsigned bit_reverse(unsigned x, int bits) {
     return r;
 }
 
+// The two words a product with the constant w < q takes (ntt_core.cuh): near primes the split words of
+// w and 2^32 w mod q, else w and its Shoup companion.
+static ulonglong2 words_at(u64 w, const Prime& p, int at) {
+    return make_ulonglong2(split_word(w, at), split_word(h_mul(w, ((u64)1 << 32) % p.q, p.q), at));
+}
+static void const_words(u64 w, const Prime& p, u64* out) {
+    const ulonglong2 t = p.cls == AR_SHOUP ? make_ulonglong2(w, h_shoup(w, p.q)) : words_at(w, p, nttc::split_at(p.cls));
+    out[0] = t.x;
+    out[1] = t.y;
+}
 static Prime make_prime(u64 q) {
     Prime p{};
     p.q = q;
@@ -155,19 +165,13 @@ static Prime make_prime(u64 q) {
     if (p.b == 50 && delta <= ((u64)1 << 26)) p.cls = AR_NEAR50;
     if (p.b == 60 && delta <= ((u64)1 << 26)) p.cls = AR_NEAR60;
     p.delta = p.cls == AR_SHOUP ? 0 : (u32)delta;
+    if (p.cls != AR_SHOUP) {
+        const_words((u64)(((u128)1 << 64) % q), p, p.w64);
+        const_words(((u64)1 << 50) % q, p, p.w50);
+    }
     return p;
 }
 
-// The two words a product with the constant w < q takes (ntt_core.cuh): near primes the split words of
-// w and 2^32 w mod q, else w and its Shoup companion.
-static ulonglong2 words_at(u64 w, const Prime& p, int at) {
-    return make_ulonglong2(split_word(w, at), split_word(h_mul(w, ((u64)1 << 32) % p.q, p.q), at));
-}
-static void const_words(u64 w, const Prime& p, u64* out) {
-    const ulonglong2 t = p.cls == AR_SHOUP ? make_ulonglong2(w, h_shoup(w, p.q)) : words_at(w, p, nttc::split_at(p.cls));
-    out[0] = t.x;
-    out[1] = t.y;
-}
 // The same for a base-conversion constant.
 static void conv_words(u64 w, const Prime& p, u64* out) {
     if (p.cls != AR_NEAR50) return const_words(w, p, out);
@@ -486,13 +490,13 @@ __global__ void evk_kernel(u64* b, const u64* __restrict__ a, const u64* __restr
     }
 }
 
-// The data-prime rows (limbs 0..L) of one key digit's two halves, stored split at bit 25.
-__global__ void key_pack_kernel(u64* kb, u64* ka, int L, int log_n) {
-    const size_t total = (size_t)(L + 1) << log_n;
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total;
-         i += (size_t)gridDim.x * blockDim.x) {
-        kb[i] = key_pack(kb[i]);
-        ka[i] = key_pack(ka[i]);
+// One digit of a key from its halves b and a: interleaved (b, a) per coefficient, the data-prime rows
+// (limbs 0..L) split at bit 25 when `packed`.
+__global__ void key_store_kernel(ulonglong2* key, const u64* __restrict__ kb, const u64* __restrict__ ka, size_t total,
+                                 int L, int log_n, bool packed) {
+    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total; i += (size_t)gridDim.x * blockDim.x) {
+        const bool pk = packed && (int)(i >> log_n) <= L;
+        key[i] = make_ulonglong2(pk ? key_pack(kb[i]) : kb[i], pk ? key_pack(ka[i]) : ka[i]);
     }
 }
 
@@ -923,11 +927,11 @@ static void make_evk(Ctx& c, EvalKey& key, const u64* d_s2, u64 obj, cudaStream_
     std::vector<int8_t> he(n);
     int8_t* d_e8 = (int8_t*)c.scratch_bytes("kg_e8", n);
     u64* d_e = c.scratch_u64("kg_e", (size_t)ne * n);
+    u64* kb = c.scratch_u64("kg_b", (size_t)ne * n);
+    u64* ka = c.scratch_u64("kg_a", (size_t)ne * n);
     for (int j = 0; j < dn; j++) {
         for (int t = 0; t < ne; t++) sample_uniform(stream_key(c.seed, kEvkA, obj, j, t), c.primes[t], &ha[(size_t)t * n], n);
         sample_gaussian(stream_key(c.seed, kEvkE, obj, j, 0), T, he.data(), n);
-        u64* kb = key.d + (size_t)(j * 2 + 0) * ne * n;
-        u64* ka = key.d + (size_t)(j * 2 + 1) * ne * n;
         CK(cudaMemcpyAsync(ka, ha.data(), sizeof(u64) * ha.size(), cudaMemcpyHostToDevice, s));
         CK(cudaMemcpyAsync(d_e8, he.data(), n, cudaMemcpyHostToDevice, s));
         ntt_forward(c, poly_batch(ka, 0, 0, 1, 1, 0, ne), s);
@@ -939,10 +943,9 @@ static void make_evk(Ctx& c, EvalKey& key, const u64* d_s2, u64 obj, cudaStream_
             evk_kernel<<<blocks_for((size_t)ne * n), kT, 0, s>>>(kb, ka, c.d_sk, d_e, d_s2, ne, c.L, lo, hi,
                                                                  c.log_n, c.d_primes, c.d_pmod);
             CK(cudaGetLastError());
-            if (c.keys_packed) {
-                key_pack_kernel<<<blocks_for((size_t)(c.L + 1) * n), kT, 0, s>>>(kb, ka, c.L, c.log_n);
-                CK(cudaGetLastError());
-            }
+            key_store_kernel<<<blocks_for((size_t)ne * n), kT, 0, s>>>(
+                reinterpret_cast<ulonglong2*>(key.d) + (size_t)j * ne * n, kb, ka, (size_t)ne * n, c.L, c.log_n, c.keys_packed);
+            CK(cudaGetLastError());
         }
         CK(cudaStreamSynchronize(s));  // host staging buffers are reused
     }

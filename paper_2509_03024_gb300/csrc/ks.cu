@@ -147,7 +147,8 @@ void ks_run(Ctx& c, const std::vector<KsItem>& all, int level, const HoistKeys* 
         CombineArgs ca{d_items, acc, c.d_pinv, next, nullptr};
         const CombineArgs none{nullptr, nullptr, nullptr, 0, nullptr};
 
-        // K1: y_i = INTT(perm(d_i)) * qhat_i^-1 (fan-out: once per source, no permutation)
+        // K1: y_i = INTT(perm(d_i)) * qhat_i^-1 (fan-out: once per source, no permutation); its loads also
+        // store perm(d_i) as limb i of its own raised digit
         std::vector<KsRow> r1;
         r1.reserve((size_t)n_sources * l1);
         for (int sx = 0; sx < n_sources; sx++)
@@ -159,6 +160,8 @@ void ks_run(Ctx& c, const std::vector<KsItem>& all, int level, const HoistKeys* 
                 r.cst = c.d_up_ninv + 2 * ((size_t)level * (L + 1) + i);
                 r.prime = i;
                 r.galois = fan ? 1 : (int)x0.galois;
+                r.out2 = ext + (((size_t)sx * dn + i / A) * next + i) * n;
+                r.pack = c.keys_packed;
                 r1.push_back(r);
             }
         const KsRow* d_r1 = c.arena.push_vec(r1, s);
@@ -209,10 +212,8 @@ void ks_run(Ctx& c, const std::vector<KsItem>& all, int level, const HoistKeys* 
                             8.0 * n * ((double)items * dn * next + (double)nkeys * dn * 2 * next + (double)items * 2 * next),
                             s, 2.0 * items * next * n * dn);
             bool shared = !fan;
-            for (int t = 1; t < items && shared; t++)
-                shared = it[t].key == it[0].key && it[t].galois == it[0].galois;
+            for (int t = 1; t < items && shared; t++) shared = it[t].key == it[0].key;
             ia.shared_key = shared ? it[0].key : nullptr;
-            ia.shared_galois = shared ? it[0].galois : 1;
             launch_ks_inner(ia, fan, c.tune.inner, c.max_data_prime_bits, s);
         } else {
             // reads: the raised digits and c0 once per item, every key once; writes acc and c0sum

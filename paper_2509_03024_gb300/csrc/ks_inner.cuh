@@ -26,19 +26,17 @@ struct HoistStep {
 struct InnerArgs {
     u64* acc;                 // [items][2][next][N]
     u64* c0sum;               // hoisted: [items][l1][N] c0 + sum_r phi_r(c0)
-    const u64* ext;           // [sources][dn][next][N] raised digits (own-digit limbs unused)
+    const u64* ext;           // [sources][dn][next][N] raised digits, the limbs of the digit itself included
     const KsItem* tab;        // device item table
     const int* src_of;        // fan-out: source of each item
     const HoistStep* steps;   // hoisted: device table of the rotations
     int n_steps;
     int items, dn, alpha, next, level, L, n_ext, log_n;
     const Prime* pr;
-    const u64* shared_key;    // plain: non-null when every item uses this key ...
-    long long shared_galois;  // ... and this automorphism (then several items per thread may run)
+    const u64* shared_key;    // plain: non-null when every item uses this key (then several items per thread may run)
     int split25;              // set by the launchers: data limbs use the split-at-bit-25 sums
     int keys_packed;          // the keys' data-prime rows, and the raised digits' data limbs (ext rows
-                              // x <= level), are stored split at bit 25 (key_unpack); the own-digit
-                              // rows read from the input are not
+                              // x <= level), are stored split at bit 25 (key_unpack)
 };
 
 // A data-prime key residue stored split at bit 25 (every data prime below 2^50): the low 25 bits in
@@ -54,8 +52,7 @@ enum InnerVariant {
     INNER_P1,       // ... 32-bit schoolbook carry chain; 1 item per thread
     INNER_S1,       // ... data limbs split at bit 25 into carry-free column sums, special limbs P32
     INNER_S2,       // S1 with 2 items per thread sharing the key loads (plain: when the items share a key)
-    INNER_S2L,      // S2 reading each permuted residue with its own 64-bit load instead of a pair load and
-                    // two selects (hoisted only; the plain kernel runs S2)
+    INNER_S2L,      // S2 with three instead of four wide multiplies per data-limb product (Karatsuba)
     INNER_N_VARIANTS
 };
 extern const char* const kInnerVariantNames[INNER_N_VARIANTS];

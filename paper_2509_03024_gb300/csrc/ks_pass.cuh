@@ -24,10 +24,10 @@ struct KsRow {
     int src_cnt;     // LD_CONV: number of source limbs
     int cst_stride;  // LD_CONV: words between consecutive source limbs' constant pairs
     int item, half, limb;  // ST_COMBINE(_RS): output item, component and limb
-    int pack;              // ST_LAST (forward): store the residue split at bit 25 (key_pack)
+    int pack;              // ST_LAST (forward), out2 of LD_GATHER: store the residue split at bit 25 (key_pack)
     const u64* src2;       // LD_AXPY / LD_MUL: second source row (LD_AXPY: null = none); ST_RESCALE: the input limb
     const u64* cst2;       // LD_AXPY: words of its factor; ST_RESCALE: words of q_l^-1 mod the row's prime
-    u64* out2;             // ST_RESCALE: output row
+    u64* out2;             // ST_RESCALE: output row; LD_GATHER: second copy of the loaded row (null = none)
     const u64* src3;       // ST_RESCALE: when set, the input limb is src2 (.) src3 (a plaintext product)
 };
 
@@ -136,7 +136,9 @@ __device__ __forceinline__ u64 load_elem(const KsRow& r, size_t k, int log_n, co
     if constexpr (LOAD == LD_PLAIN) {
         return r.dst[k];
     } else if constexpr (LOAD == LD_GATHER) {
-        return r.src[r.galois == 1 ? (int)k : auto_src((int)k, r.galois, log_n)];
+        const u64 v = r.src[r.galois == 1 ? (int)k : auto_src((int)k, r.galois, log_n)];
+        if (r.out2) r.out2[k] = r.pack ? key_pack(v) : v;
+        return v;
     } else if constexpr (LOAD == LD_CENTRED) {  // the centred representative of src[k] (mod q_limb)
         const u64 ql = rc.ql, v = r.src[k];
         const bool neg = v > (ql >> 1);
@@ -167,7 +169,7 @@ __device__ __forceinline__ void store_elem(const KsRow& r, size_t k, u64 v, cons
     }
     if (STORE == ST_LAST || STORE == ST_SCALE) {  // inverse: times N^-1, or the row's constant in its place
         const u64 t = m.canon(INV ? m.mul(v, words(STORE == ST_SCALE ? r.cst : ninv + 2 * r.prime)) : v, one_s);
-        r.dst[k] = r.pack ? key_pack(t) : t;
+        r.dst[k] = !INV && r.pack ? key_pack(t) : t;
         return;
     }
     const u64 t = m.canon(v, one_s);

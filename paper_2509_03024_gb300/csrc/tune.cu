@@ -89,7 +89,7 @@ void tune_inner(Ctx& c, int level, std::vector<fhe_tune_result>& out) {
     u64* c0 = tmp.get((size_t)items * (c.L + 1) * n);
     u64* acc = tmp.get((size_t)items * 2 * next * n);
     u64* c0sum = tmp.get((size_t)items * l1 * n);
-    // the key rows are laid out [digit][2][n_ext]; residues below the smallest prime serve every row
+    // the key rows are laid out [digit][n_ext][N][2]; residues below the smallest prime serve every row
     fill_residues<<<1024, 256>>>(ext, (size_t)items * dn * next * n, c.log_n, 1, c.d_primes, 1);
     fill_residues<<<1024, 256>>>(keys, (size_t)steps * key_words, c.log_n, 1, c.d_primes, 2);
     fill_residues<<<1024, 256>>>(din, (size_t)items * (c.L + 1) * n, c.log_n, 1, c.d_primes, 3);
@@ -134,7 +134,6 @@ void tune_inner(Ctx& c, int level, std::vector<fhe_tune_result>& out) {
             a.n_steps = steps;
         } else {
             a.shared_key = keys;
-            a.shared_galois = 1;
         }
         double best = 1e30;
         int best_v = 0;
