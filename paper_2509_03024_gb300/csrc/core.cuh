@@ -287,6 +287,7 @@ struct Ctx {
     u64* d_fd_minv = nullptr;         // [L+1][L+1][2]           M'^-1 mod q_i, i < l
     u64* d_fd_pq = nullptr;           // [L+1][2]                P mod q_l
     double* d_cos = nullptr;          // [2N] cos(pi e / N)
+    double* d_cos_t = nullptr;        // [N/32][64] the same for the encoding, entry e at [e mod N/32][e / (N/32)]
     double* d_sin = nullptr;          // [2N] sin(pi e / N)
     u32* d_pow5 = nullptr;            // [N/2] 5^t mod 2N
 

@@ -70,7 +70,7 @@ Ctx::~Ctx() {
     cudaSetDevice(device);
     cudaDeviceSynchronize();
     void* bufs[] = {d_primes, d_ninv, d_tw, d_itw, d_tw2, d_itw2, d_up_ninv, d_down_ninv, d_resc, d_resc_w, d_up_hat,
-                    d_down_hat, d_pinv, d_pmod, d_fd_ninv, d_fd_hat, d_fd_minv, d_fd_pq, d_cos, d_sin, d_pow5, d_sk, d_pk, rlk.d};
+                    d_down_hat, d_pinv, d_pmod, d_fd_ninv, d_fd_hat, d_fd_minv, d_fd_pq, d_cos, d_cos_t, d_sin, d_pow5, d_sk, d_pk, rlk.d};
     for (void* p : bufs)
         if (p) cudaFree(p);
     for (auto& kv : rot)
@@ -247,6 +247,23 @@ static GaussTable gauss_table(double sigma) {
         T.t[k] = (u64)(cdf * 9223372036854775808.0);
     }
     return T;
+}
+
+// State z with mix64(z) = 2^64 - 1, the one output the ternary sampler rejects (2^64 = 1 mod 3).
+static u64 ternary_reject_state() {
+    auto inv = [](u64 a) {  // inverse of an odd number modulo 2^64 (Newton)
+        u64 x = a;
+        for (int i = 0; i < 6; i++) x *= 2 - a * x;
+        return x;
+    };
+    auto unshift = [](u64 y, int s) {  // inverse of x ^ (x >> s)
+        u64 x = y;
+        for (int i = 0; i < 64; i += s) x = y ^ (x >> s);
+        return x;
+    };
+    u64 z = unshift(~(u64)0, 31);
+    z = unshift(z * inv(0x94D049BB133111EBULL), 27);
+    return unshift(z * inv(0xBF58476D1CE4E5B9ULL), 30);
 }
 
 static void sample_gaussian(u64 key, const GaussTable& T, int8_t* out, int n) {
@@ -441,6 +458,9 @@ static void build_tables(Ctx& c) {
         sn[e] = std::sin(M_PI * (double)e / (double)n);
     }
     c.d_cos = dupload(cs);
+    std::vector<double> cs_t(cs.size());  // encode_kernel's layout
+    for (int e = 0; e < 2 * n; e++) cs_t[(size_t)(e % (n / 32)) * 64 + e / (n / 32)] = cs[e];
+    c.d_cos_t = dupload(cs_t);
     c.d_sin = dupload(sn);
     std::vector<u32> p5(c.slots);
     u64 x = 1;
@@ -565,45 +585,129 @@ __global__ void seeded_c0_kernel(u64* out, const u64* __restrict__ me, const u64
     }
 }
 
-__global__ void add_compact_kernel(u64* out, const u64* __restrict__ a, size_t total, int l1, int log_n,
-                                   const Prime* __restrict__ pr) {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < total;
-         i += (size_t)gridDim.x * blockDim.x) {
-        int limb = (int)((i >> log_n) % l1);
-        out[i] = add_mod(out[i], a[i], pr[limb].q);
+// Stream key and samplers as on the host (sampling section above), one draw per coefficient k: the
+// Gaussian takes output k + 1 of its stream; the ternary sampler too, but past the stream's one rejected
+// output (state z_rej, reached at counter (z_rej - h) / gamma mod 2^64) the one after it.
+__device__ __forceinline__ u64 stream_key_dev(u64 seed, u64 purpose, u64 obj) {
+    u64 h = seed;
+    h = mix64_dev((h ^ purpose) + 0x9E3779B97F4A7C15ULL);
+    h = mix64_dev((h ^ obj) + 0x9E3779B97F4A7C15ULL);
+    h = mix64_dev(h + 0x9E3779B97F4A7C15ULL);  // poly 0
+    return mix64_dev(h + 0x9E3779B97F4A7C15ULL);  // limb 0
+}
+__device__ __forceinline__ int gaussian_dev(u64 h, u64 k, const GaussTable& T) {
+    const u64 x = mix64_dev(h + (k + 1) * 0x9E3779B97F4A7C15ULL), u = x >> 1;
+    int mag = 0;
+#pragma unroll
+    for (int i = 0; i < 19; i++) mag += u >= T.t[i];
+    return (x & 1) ? -mag : mag;
+}
+constexpr u64 kGammaInv = 0xF1DE83E19937733DULL;  // 0x9E3779B97F4A7C15^-1 mod 2^64
+static_assert(kGammaInv * 0x9E3779B97F4A7C15ULL == 1, "inverse of gamma");
+__device__ __forceinline__ int ternary_dev(u64 h, u64 k, u64 z_rej) {
+    u64 c = k + 1;
+    if (c >= (z_rej - h) * kGammaInv) c++;
+    return (int)(mix64_dev(h + c * 0x9E3779B97F4A7C15ULL) % 3) - 1;
+}
+// m mod q for a signed m; e mod q for a small e
+__device__ __forceinline__ u64 signed_residue(i64 m, const Prime& P) {
+    const u64 mag = m < 0 ? (u64)0 - (u64)m : (u64)m;
+    u64 r = mag - __umul64hi(mag, P.one_s) * P.q;
+    r = r >= P.q ? r - P.q : r;
+    return m < 0 && r ? P.q - r : r;
+}
+__device__ __forceinline__ u64 small_residue(int e, u64 q) { return e >= 0 ? (u64)e : q - (u64)(-e); }
+
+constexpr int kEncChunk = 32;  // messages per launch
+struct Objs {
+    u64 o[kEncChunk];
+};
+
+// Per message t and coefficient k, every limb i < l1: v (ternary), e0 + m and e1, coefficient form; out
+// [3][count][l1][N].
+__global__ void enc_sample_kernel(u64* out, const i64* __restrict__ m, size_t m_stride, Objs nonces, u64 seed, GaussTable T,
+                                  u64 z_rej, int count, int l1, int log_n, const Prime* __restrict__ pr) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x, t = blockIdx.y;
+    const u64 obj = nonces.o[t];
+    const int v = ternary_dev(stream_key_dev(seed, kEncV, obj), k, z_rej);
+    const int e0 = gaussian_dev(stream_key_dev(seed, kEncE0, obj), k, T);
+    const int e1 = gaussian_dev(stream_key_dev(seed, kEncE1, obj), k, T);
+    const i64 mk = m[(size_t)t * m_stride + k];
+    u64* o = out + (((size_t)t * l1) << log_n) + k;
+    const size_t part = ((size_t)count * l1) << log_n;
+    for (int i = 0; i < l1; i++, o += (size_t)1 << log_n) {
+        const Prime P = pr[i];
+        o[0] = small_residue(v, P.q);
+        o[part] = add_mod(small_residue(e0, P.q), signed_residue(mk, P), P.q);
+        o[2 * part] = small_residue(e1, P.q);
+    }
+}
+
+// me[t][i] = m_t + e_t (the Gaussian of stream purpose kSeededE), compact [count][l1][N].
+__global__ void seeded_sample_kernel(u64* me, const i64* __restrict__ m, size_t m_stride, Objs objs, u64 seed, GaussTable T,
+                                     int l1, int log_n, const Prime* __restrict__ pr) {
+    const int k = blockIdx.x * blockDim.x + threadIdx.x, t = blockIdx.y;
+    const int e = gaussian_dev(stream_key_dev(seed, kSeededE, objs.o[t]), k, T);
+    const i64 mk = m[(size_t)t * m_stride + k];
+    u64* o = me + (((size_t)t * l1) << log_n) + k;
+    for (int i = 0; i < l1; i++, o += (size_t)1 << log_n) {
+        const Prime P = pr[i];
+        o[0] = add_mod(small_residue(e, P.q), signed_residue(mk, P), P.q);
     }
 }
 
 // Encoding: coefficient j of vector v = rint(factor * sum_t val_t * cos(pi (j 5^t mod 2N) / N)),
 // the sum over the vector's non-zero slots in ascending slot order, each step an
 // IEEE double multiply then add (no fused multiply-add).
-__global__ void encode_kernel(i64* out, const int* __restrict__ idx, const double* __restrict__ val,
-                              const int* __restrict__ offsets, const double* __restrict__ cos_tab,
-                              const u32* __restrict__ pow5, int log_n, double factor) {
-    __shared__ u32 s_p[256];
-    __shared__ double s_v[256];
-    const int v = blockIdx.y;
-    const int n = 1 << log_n;
-    const u32 mask = 2u * n - 1u;
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
+//
+// The order makes it a chain per coefficient; what bounds it is the double-precision pipe (two lanes per
+// SM) and the cosine reads. The table is stored [e mod N/32][e / (N/32)], and the lanes of a warp take
+// coefficients N/32 apart, so the 32 cosines of one term lie in one 512-byte row. Where few distinct
+// values multiply many terms (a factor vector repeated in every block, ratings, masks), their products
+// with the whole table are formed once (PRE), which leaves one double-precision operation per term.
+// 32768 terms of 16 values, N = 2^16 (ms): 14.8 with scattered reads, 5.0 as here (3.7 of them the additions).
+constexpr int kEncThreads = 64;
+constexpr int kEncDistinct = 32;  // distinct values whose products are tabulated (1 MiB each at N = 2^16)
+
+__global__ void cos_products_kernel(double* tab, const double* __restrict__ vals, const double* __restrict__ cos_t, int n2) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n2) tab[(size_t)blockIdx.y * n2 + i] = __dmul_rn(vals[blockIdx.y], cos_t[i]);
+}
+
+// PRE: tab holds the products of the distinct values, which[t] the value of term t; else tab is the cosine
+// table and val[t] the values.
+template <bool PRE>
+__global__ void __launch_bounds__(kEncThreads) encode_kernel(i64* out, const int* __restrict__ idx, const double* __restrict__ val,
+                                                             const int* __restrict__ which, const int* __restrict__ offsets,
+                                                             const double* __restrict__ tab, const u32* __restrict__ pow5,
+                                                             int log_n, double factor) {
+    constexpr int CH = 256;
+    __shared__ u32 s_p[CH];
+    __shared__ double s_v[PRE ? 1 : CH];
+    __shared__ u32 s_o[PRE ? CH : 1];
+    const int v = blockIdx.y, lane = threadIdx.x & 31;
+    const int rows_log = log_n - 5;  // log2(N / 32)
+    const u32 j0 = blockIdx.x * (kEncThreads / 32) + (threadIdx.x >> 5), j = j0 + ((u32)lane << rows_log);
     const int beg = offsets[v], end = offsets[v + 1];
     double acc = 0.0;
-    for (int c0 = beg; c0 < end; c0 += 256) {
-        int cnt = min(256, end - c0);
+    for (int c0 = beg; c0 < end; c0 += CH) {
+        const int cnt = min(CH, end - c0);
         __syncthreads();
-        for (int t = threadIdx.x; t < cnt; t += blockDim.x) {
+        for (int t = threadIdx.x; t < cnt; t += kEncThreads) {
             s_p[t] = pow5[idx[c0 + t]];
-            s_v[t] = val[c0 + t];
+            if (PRE) s_o[t] = (u32)which[c0 + t] << (log_n + 1);
+            else s_v[t] = val[c0 + t];
         }
         __syncthreads();
-        if (j < n) {
-            for (int t = 0; t < cnt; t++) {
-                u32 e = (u32)(((unsigned long long)j * s_p[t]) & mask);
-                acc = __dadd_rn(acc, __dmul_rn(s_v[t], cos_tab[e]));
-            }
+#pragma unroll 8
+        for (int t = 0; t < cnt; t++) {
+            const u32 p = s_p[t], e0 = j0 * p;  // modulo 2N: row e0 mod N/32, column e0 / (N/32) + lane p
+            const u32 at = ((e0 & ((1u << rows_log) - 1)) << 6) + (((e0 >> rows_log) + lane * p) & 63u);
+            if (PRE) acc = __dadd_rn(acc, tab[s_o[t] + at]);
+            else acc = __dadd_rn(acc, __dmul_rn(s_v[t], tab[at]));
         }
     }
-    if (j < n) out[(size_t)v * n + j] = __double2ll_rn(__dmul_rn(acc, factor));
+    out[((size_t)v << log_n) + j] = __double2ll_rn(__dmul_rn(acc, factor));
 }
 
 // decryption: m_i = c0_i + c1_i * s_i for limbs < nl (evaluation domain)
@@ -617,23 +721,18 @@ __global__ void dec_kernel(u64* m, const u64* __restrict__ ct, size_t part_strid
     }
 }
 
-// centred CRT lift of 1 or 2 limbs to a double
-__global__ void crt_kernel(double* out, const u64* __restrict__ m, int nl, int log_n, u64 q0, u64 q1,
-                           u64 q0inv_mod_q1) {
-    const int n = 1 << log_n;
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n; j += gridDim.x * blockDim.x) {
-        if (nl == 1) {
-            u64 x = m[j];
-            out[j] = x > q0 / 2 ? -(double)(q0 - x) : (double)x;
-        } else {
-            u64 x0 = m[j], x1 = m[n + j];
-            u64 d = x1 >= x0 % q1 ? x1 - x0 % q1 : x1 + q1 - x0 % q1;
-            u64 k = (u64)(((u128)d * q0inv_mod_q1) % q1);
-            u128 v = (u128)k * q0 + x0;
-            u128 Q = (u128)q0 * q1;
-            out[j] = v > Q / 2 ? -(double)(Q - v) : (double)v;
-        }
-    }
+// The integer coefficient of residues x0 mod q0 (nl = 1) or x0, x1 mod q0, q1 (nl = 2), centred, as a double.
+struct Lift {
+    u64 q0, q1, q0inv;  // q0inv: q0^-1 mod q1
+    int nl;
+};
+__device__ __forceinline__ double centred_lift(u64 x0, u64 x1, const Lift& l) {
+    if (l.nl == 1) return x0 > l.q0 / 2 ? -(double)(l.q0 - x0) : (double)x0;
+    const u64 r = x0 % l.q1;
+    const u64 d = x1 >= r ? x1 - r : x1 + l.q1 - r;
+    const u64 k = (u64)(((u128)d * l.q0inv) % l.q1);
+    const u128 v = (u128)k * l.q0 + x0, Q = (u128)l.q0 * l.q1;
+    return v > Q / 2 ? -(double)(Q - v) : (double)v;
 }
 
 // exact centred lift of 1 or 2 limbs to int64 (refresh); flags values outside int64
@@ -662,24 +761,63 @@ __global__ void crt_int64_kernel(i64* out, const u64* __restrict__ m, int nl, in
     }
 }
 
-// z_t = sum_j m_j cos(pi (j 5^t mod 2N) / N) / Delta, one block per slot
-__global__ void decode_kernel(double* z, const double* __restrict__ m, const double* __restrict__ cos_tab,
-                              const u32* __restrict__ pow5, int log_n, double inv_scale, int n_slots) {
-    __shared__ double red[256];
-    const int t = blockIdx.x;
-    if (t >= n_slots) return;
-    const int n = 1 << log_n;
-    const u32 mask = 2u * n - 1u;
-    const u32 p = pow5[t];
-    double acc = 0.0;
-    for (int j = threadIdx.x; j < n; j += blockDim.x) acc += m[j] * cos_tab[((u64)j * p) & mask];
-    red[threadIdx.x] = acc;
-    __syncthreads();
-    for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
+// Decoding: z_t = Re m(zeta^(5^t)) / Delta with zeta = exp(i pi / N). 5^t = 4 k + 1, and zeta^(N/2 (4k+1)) = i,
+// so m(zeta^(4k+1)) = sum_{j < n} (m_j + i m_(j+n)) zeta^j exp(2 pi i j k / n) for n = N/2: one complex
+// transform of n points gives every slot, where a sum of N terms per slot read N scattered cosines each
+// (6.9 ms for the 2^15 slots of N = 2^16, one ciphertext). Four-step form n = n1 n2, one small transform
+// per CTA; j = j1 n2 + j2, k = k1 + n1 k2.
+
+// In-place decimation-in-frequency transform of M = blockDim.x * 2 points in shared memory; entry i holds
+// output brev(i) after it. tab_step: 2N / M, the table step of exp(2 pi i / M).
+__device__ void fft_block(double2* x, int log_m, int tab_step, const double* __restrict__ cs, const double* __restrict__ sn) {
+    const int t = threadIdx.x;
+    for (int h = 1 << (log_m - 1), step = tab_step; h; h >>= 1, step <<= 1) {
+        const int p = t & (h - 1), i = ((t - p) << 1) + p;
+        const double2 a = x[i], b = x[i + h];
+        const double c = cs[p * step], s = sn[p * step], dx = a.x - b.x, dy = a.y - b.y;
+        x[i] = make_double2(a.x + b.x, a.y + b.y);
+        x[i + h] = make_double2(dx * c - dy * s, dx * s + dy * c);
         __syncthreads();
     }
-    if (threadIdx.x == 0) z[t] = red[0] * inv_scale;
+}
+
+// Columns j2 (blockIdx.x): lift, twist by zeta^j, n1-point transform over j1, times exp(2 pi i j2 k1 / n).
+__global__ void decode_columns(double2* y, const u64* __restrict__ m, Lift lift, int log_n, int log_n1,
+                               const double* __restrict__ cs, const double* __restrict__ sn) {
+    extern __shared__ double2 fx[];
+    const int n = 1 << (log_n - 1), log_n2 = log_n - 1 - log_n1, n2 = 1 << log_n2, j2 = blockIdx.x;
+    for (int j1 = threadIdx.x; j1 < 1 << log_n1; j1 += blockDim.x) {
+        const int j = (j1 << log_n2) + j2;
+        const u64* hi = m + (size_t)2 * n;  // second limb
+        const double re = centred_lift(m[j], lift.nl == 2 ? hi[j] : 0, lift);
+        const double im = centred_lift(m[j + n], lift.nl == 2 ? hi[j + n] : 0, lift);
+        fx[j1] = make_double2(re * cs[j] - im * sn[j], re * sn[j] + im * cs[j]);
+    }
+    __syncthreads();
+    fft_block(fx, log_n1, 1 << (log_n + 1 - log_n1), cs, sn);
+    for (int i = threadIdx.x; i < 1 << log_n1; i += blockDim.x) {
+        const int k1 = (int)(__brev((unsigned)i) >> (32 - log_n1)), e = 4 * k1 * j2;  // below 4 n = 2N
+        const double2 v = fx[i];
+        y[(size_t)k1 * n2 + j2] = make_double2(v.x * cs[e] - v.y * sn[e], v.x * sn[e] + v.y * cs[e]);
+    }
+}
+
+// Rows k1 (blockIdx.x): n2-point transform over j2, the real parts of outputs k1 + n1 k2.
+__global__ void decode_rows(double* re, const double2* __restrict__ y, int log_n, int log_n1, const double* __restrict__ cs,
+                            const double* __restrict__ sn) {
+    extern __shared__ double2 fx[];
+    const int log_n2 = log_n - 1 - log_n1, n2 = 1 << log_n2, k1 = blockIdx.x;
+    for (int j = threadIdx.x; j < n2; j += blockDim.x) fx[j] = y[(size_t)k1 * n2 + j];
+    __syncthreads();
+    fft_block(fx, log_n2, 1 << (log_n + 1 - log_n2), cs, sn);
+    for (int i = threadIdx.x; i < n2; i += blockDim.x)
+        re[((size_t)(__brev((unsigned)i) >> (32 - log_n2)) << log_n1) + k1] = fx[i].x;
+}
+
+__global__ void decode_slots(double* z, const double* __restrict__ re, const u32* __restrict__ pow5, double inv_scale,
+                             int n_slots) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < n_slots) z[t] = re[(pow5[t] - 1) >> 2] * inv_scale;
 }
 
 }  // namespace
@@ -707,13 +845,46 @@ void encode_many_device(Ctx& c, const std::vector<int>& idx, const std::vector<d
     }
     CK(cudaMemcpyAsync(d_off, offsets.data(), sizeof(int) * offsets.size(), cudaMemcpyHostToDevice, s));
     const double factor = std::ldexp(1.0, c.log_scale + 1 - c.log_n);  // 2 Delta / N
+    // few distinct values over many terms: tabulate their products, when that is an eighth of the terms' work
+    std::vector<double> distinct;
+    std::vector<int> which;
+    bool pre = nz >= 8;
+    if (pre) {
+        which.resize(nz);
+        int last = -1;
+        for (size_t t = 0; t < nz && pre; t++) {
+            if (last < 0 || std::memcmp(&distinct[last], &val[t], sizeof(double)) != 0) {
+                for (last = 0; last < (int)distinct.size(); last++)
+                    if (std::memcmp(&distinct[last], &val[t], sizeof(double)) == 0) break;
+                if (last == (int)distinct.size()) {
+                    distinct.push_back(val[t]);
+                    pre = (int)distinct.size() <= kEncDistinct && distinct.size() * 8 <= nz;
+                }
+            }
+            which[t] = last;
+        }
+    }
+    const int n2 = 2 * c.n;
+    double* tab = c.d_cos_t;
+    int* d_which = nullptr;
+    if (pre) {
+        tab = (double*)c.scratch_bytes("enc_tab", sizeof(double) * n2 * distinct.size());
+        d_which = (int*)c.scratch_bytes("enc_which", sizeof(int) * nz);
+        double* d_dist = (double*)c.scratch_bytes("enc_dist", sizeof(double) * kEncDistinct);
+        CK(cudaMemcpyAsync(d_which, which.data(), sizeof(int) * nz, cudaMemcpyHostToDevice, s));
+        CK(cudaMemcpyAsync(d_dist, distinct.data(), sizeof(double) * distinct.size(), cudaMemcpyHostToDevice, s));
+        LaunchScope _ls(c.prof, K_ENCODE, 8.0 * n2 * (distinct.size() + 1), s);
+        cos_products_kernel<<<dim3((n2 + kT - 1) / kT, (unsigned)distinct.size()), kT, 0, s>>>(tab, d_dist, c.d_cos_t, n2);
+        CK(cudaGetLastError());
+    }
     for (int v0 = 0; v0 < count; v0 += 65535) {
         int cnt = std::min(65535, count - v0);
-        dim3 grid((c.n + 255) / 256, cnt);
+        dim3 grid(c.n / kEncThreads, cnt);
         {
             LaunchScope _ls(c.prof, K_ENCODE, 8.0 * cnt * c.n + 12.0 * nz, s);
-            encode_kernel<<<grid, 256, 0, s>>>(out_dev + (size_t)v0 * c.n, d_idx, d_val, d_off + v0, c.d_cos,
-                                               c.d_pow5, c.log_n, factor);
+            auto kernel = pre ? encode_kernel<true> : encode_kernel<false>;
+            kernel<<<grid, kEncThreads, 0, s>>>(out_dev + (size_t)v0 * c.n, d_idx, d_val, d_which, d_off + v0, tab, c.d_pow5,
+                                                c.log_n, factor);
             CK(cudaGetLastError());
         }
     }
@@ -764,24 +935,18 @@ void encrypt_seeded_device(Ctx& c, const i64* m_dev, size_t m_stride, int count,
     if (level < 0 || level > c.L) fail(FHE_ERR_INVALID_ARG, "level out of range");
     const int n = c.n, l1 = level + 1;
     const GaussTable T = gauss_table(c.sigma);
-    const int chunk = 32;
-    std::vector<int8_t> host((size_t)chunk * n);
+    const int chunk = kEncChunk;
     for (int t0 = 0; t0 < count; t0 += chunk) {
         const int cnt = std::min(chunk, count - t0);
-        for (int t = 0; t < cnt; t++)
-            sample_gaussian(stream_key(c.seed, kSeededE, objs[t0 + t], 0, 0), T, host.data() + (size_t)t * n, n);
-        int8_t* d_e = (int8_t*)c.scratch_bytes("senc_e", (size_t)chunk * n);
+        Objs o{};
+        for (int t = 0; t < cnt; t++) o.o[t] = objs[t0 + t];
         u64* me = c.scratch_u64("senc_me", (size_t)chunk * l1 * n);
-        u64* ee = c.scratch_u64("senc_ee", (size_t)chunk * l1 * n);
         u64* a = c.scratch_u64("senc_a", (size_t)chunk * l1 * n);
-        CK(cudaMemcpyAsync(d_e, host.data(), (size_t)cnt * n, cudaMemcpyHostToDevice, s));
         const size_t st = (size_t)l1 * n;
-        k_int_to_rns(c, me, st, m_dev + (size_t)t0 * m_stride, m_stride, cnt, l1, s);
-        k_int8_to_rns(c, ee, st, d_e, (size_t)n, cnt, l1, 1 << 30, 0, s);
         {
-            LaunchScope _ls(c.prof, K_ELEMENTWISE, 24.0 * cnt * st, s);
-            add_compact_kernel<<<blocks_for((size_t)cnt * st), kT, 0, s>>>(me, ee, (size_t)cnt * st, l1, c.log_n,
-                                                                           c.d_primes);
+            LaunchScope _ls(c.prof, K_ELEMENTWISE, 8.0 * cnt * (n + st), s);
+            seeded_sample_kernel<<<dim3((n + kT - 1) / kT, cnt), kT, 0, s>>>(me, m_dev + (size_t)t0 * m_stride, m_stride, o,
+                                                                             c.seed, T, l1, c.log_n, c.d_primes);
             CK(cudaGetLastError());
         }
         std::vector<SeedRow> rows;
@@ -796,7 +961,6 @@ void encrypt_seeded_device(Ctx& c, const i64* m_dev, size_t m_stride, int count,
                                                                          (size_t)cnt * st, l1, c.log_n, c.d_primes);
             CK(cudaGetLastError());
         }
-        CK(cudaStreamSynchronize(s));  // `host` is refilled by the next chunk
     }
 }
 
@@ -806,37 +970,21 @@ void encrypt_coeffs_device(Ctx& c, const i64* m_dev, size_t m_stride, int count,
     if (level < 0 || level > c.L) fail(FHE_ERR_INVALID_ARG, "level out of range");
     const int n = c.n, l1 = level + 1;
     const GaussTable T = gauss_table(c.sigma);
-    const int chunk = 32;
-    std::vector<int8_t> host((size_t)chunk * 3 * n);
-    for (int t0 = 0; t0 < count; t0 += chunk) {
-        const int cnt = std::min(chunk, count - t0);
-        for (int t = 0; t < cnt; t++) {
-            u64 nonce = nonces[t0 + t];
-            int8_t* h = host.data() + (size_t)t * 3 * n;
-            sample_ternary(stream_key(c.seed, kEncV, nonce, 0, 0), h, n);
-            sample_gaussian(stream_key(c.seed, kEncE0, nonce, 0, 0), T, h + n, n);
-            sample_gaussian(stream_key(c.seed, kEncE1, nonce, 0, 0), T, h + 2 * n, n);
-        }
-        int8_t* d_small = (int8_t*)c.scratch_bytes("enc_small", (size_t)chunk * 3 * n);
-        u64* v = c.scratch_u64("enc_v", (size_t)chunk * l1 * n);
-        u64* c0 = c.scratch_u64("enc_c0", (size_t)chunk * l1 * n);
-        u64* c1 = c.scratch_u64("enc_c1", (size_t)chunk * l1 * n);
-        u64* mm = c.scratch_u64("enc_m", (size_t)chunk * l1 * n);
-        CK(cudaMemcpyAsync(d_small, host.data(), (size_t)cnt * 3 * n, cudaMemcpyHostToDevice, s));
+    const u64 z_rej = ternary_reject_state();
+    for (int t0 = 0; t0 < count; t0 += kEncChunk) {
+        const int cnt = std::min(kEncChunk, count - t0);
+        Objs o{};
+        for (int t = 0; t < cnt; t++) o.o[t] = nonces[t0 + t];
         const size_t st = (size_t)l1 * n;
-        k_int8_to_rns(c, v, st, d_small, (size_t)3 * n, cnt, l1, 1 << 30, 0, s);
-        k_int8_to_rns(c, c0, st, d_small + n, (size_t)3 * n, cnt, l1, 1 << 30, 0, s);
-        k_int8_to_rns(c, c1, st, d_small + 2 * n, (size_t)3 * n, cnt, l1, 1 << 30, 0, s);
-        k_int_to_rns(c, mm, st, m_dev + (size_t)t0 * m_stride, m_stride, cnt, l1, s);
+        u64* v = c.scratch_u64("enc_v", 3 * (size_t)cnt * st);  // v, c0, c1 of every message
+        u64 *c0 = v + cnt * st, *c1 = c0 + cnt * st;
         {
-            LaunchScope _ls(c.prof, K_ELEMENTWISE, 24.0 * cnt * st, s);
-            add_compact_kernel<<<blocks_for((size_t)cnt * st), kT, 0, s>>>(c0, mm, (size_t)cnt * st, l1,
-                                                                           c.log_n, c.d_primes);
+            LaunchScope _ls(c.prof, K_ELEMENTWISE, 8.0 * cnt * (n + 3 * st), s);
+            enc_sample_kernel<<<dim3((n + kT - 1) / kT, cnt), kT, 0, s>>>(v, m_dev + (size_t)t0 * m_stride, m_stride, o, c.seed, T,
+                                                                          z_rej, cnt, l1, c.log_n, c.d_primes);
             CK(cudaGetLastError());
         }
-        ntt_forward(c, poly_batch(v, st, 0, cnt, 1, 0, l1), s);
-        ntt_forward(c, poly_batch(c0, st, 0, cnt, 1, 0, l1), s);
-        ntt_forward(c, poly_batch(c1, st, 0, cnt, 1, 0, l1), s);
+        ntt_forward(c, poly_batch(v, st, 0, 3 * cnt, 1, 0, l1), s);
         {
             LaunchScope _ls(c.prof, K_ELEMENTWISE, 56.0 * cnt * st, s);
             enc_combine_kernel<<<blocks_for((size_t)cnt * st), kT, 0, s>>>(
@@ -844,7 +992,6 @@ void encrypt_coeffs_device(Ctx& c, const i64* m_dev, size_t m_stride, int count,
                 c.d_pk + (size_t)(c.L + 1) * n, cnt, l1, c.log_n, c.d_primes);
             CK(cudaGetLastError());
         }
-        CK(cudaStreamSynchronize(s));  // `host` is refilled by the next chunk
     }
 }
 
@@ -855,8 +1002,6 @@ void decrypt_to_slots(Ctx& c, const u64* ct, int level, double* host_slots, size
     if (n_slots > (size_t)c.slots) fail(FHE_ERR_INVALID_ARG, "more values than slots");
     const int n = c.n, nl = std::min(level, 1) + 1;
     u64* m = c.scratch_u64("dec_m", (size_t)nl * n);
-    double* md = (double*)c.scratch_bytes("dec_md", sizeof(double) * n);
-    double* z = (double*)c.scratch_bytes("dec_z", sizeof(double) * (n_slots + 1));
     {
         LaunchScope _ls(c.prof, K_ELEMENTWISE, 32.0 * nl * n, s);
         dec_kernel<<<blocks_for((size_t)nl * n), kT, 0, s>>>(m, ct, (size_t)(c.L + 1) * n, c.d_sk, nl, c.log_n,
@@ -864,18 +1009,26 @@ void decrypt_to_slots(Ctx& c, const u64* ct, int level, double* host_slots, size
         CK(cudaGetLastError());
     }
     ntt_inverse(c, poly_batch(m, (size_t)nl * n, 0, 1, 1, 0, nl), s);
-    u64 q0 = c.primes[0], q1 = c.primes[1 % (c.L + 1)];
-    u64 q0i = nl == 2 ? h_inv(q0 % q1, q1) : 0;
-    {
-        LaunchScope _ls(c.prof, K_ENCODE, 8.0 * (nl + 1) * n, s);
-        crt_kernel<<<blocks_for(n), kT, 0, s>>>(md, m, nl, c.log_n, q0, q1, q0i);
-        CK(cudaGetLastError());
-    }
     if (n_slots) {
+        const u64 q0 = c.primes[0], q1 = c.primes[1 % (c.L + 1)];
+        const Lift lift{q0, q1, nl == 2 ? h_inv(q0 % q1, q1) : 0, nl};
+        const int log_n1 = c.log_n / 2, n1 = 1 << log_n1, n2 = (n / 2) >> log_n1;
+        double2* y = (double2*)c.scratch_bytes("dec_y", sizeof(double2) * (n / 2));
+        double* re = (double*)c.scratch_bytes("dec_re", sizeof(double) * (n / 2));
+        double* z = (double*)c.scratch_bytes("dec_z", sizeof(double) * c.slots);
         {
-            LaunchScope _ls(c.prof, K_ENCODE, 8.0 * (n + n_slots), s);
-            decode_kernel<<<(unsigned)n_slots, 256, 0, s>>>(z, md, c.d_cos, c.d_pow5, c.log_n,
-                                                            std::ldexp(1.0, -c.log_scale), (int)n_slots);
+            LaunchScope _ls(c.prof, K_ENCODE, 8.0 * nl * n + 16.0 * (n / 2), s);
+            decode_columns<<<n2, n1 / 2, sizeof(double2) * n1, s>>>(y, m, lift, c.log_n, log_n1, c.d_cos, c.d_sin);
+            CK(cudaGetLastError());
+        }
+        {
+            LaunchScope _ls(c.prof, K_ENCODE, 24.0 * (n / 2), s);
+            decode_rows<<<n1, n2 / 2, sizeof(double2) * n2, s>>>(re, y, c.log_n, log_n1, c.d_cos, c.d_sin);
+            CK(cudaGetLastError());
+        }
+        {
+            LaunchScope _ls(c.prof, K_ENCODE, 20.0 * n_slots, s);
+            decode_slots<<<blocks_for(n_slots), kT, 0, s>>>(z, re, c.d_pow5, std::ldexp(1.0, -c.log_scale), (int)n_slots);
             CK(cudaGetLastError());
         }
         CK(cudaMemcpyAsync(host_slots, z, sizeof(double) * n_slots, cudaMemcpyDeviceToHost, s));

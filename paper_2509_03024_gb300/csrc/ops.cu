@@ -300,10 +300,12 @@ __global__ void sum_acc_kernel(const AccTarget* __restrict__ tg, const BinItem* 
     }
 }
 
-__device__ __forceinline__ u64 signed_mod(i64 v, u64 q) {
-    if (v >= 0) return (u64)v % q;
-    u64 m = (u64)(-(v + 1)) % q;  // -(v+1) >= 0 avoids overflow at INT64_MIN
-    return q - 1 - m;
+// v mod q: one Shoup product by 1 instead of a 64-bit division
+__device__ __forceinline__ u64 signed_mod(i64 v, const Prime& P) {
+    const u64 mag = v < 0 ? (u64)0 - (u64)v : (u64)v;
+    u64 r = mag - __umul64hi(mag, P.one_s) * P.q;
+    r = r >= P.q ? r - P.q : r;
+    return v < 0 && r ? P.q - r : r;
 }
 
 __global__ void int_to_rns_kernel(u64* out, size_t out_stride, const i64* __restrict__ in, size_t in_stride,
@@ -316,7 +318,7 @@ __global__ void int_to_rns_kernel(u64* out, size_t out_stride, const i64* __rest
         int limb = (int)(row % limbs);
         int item = (int)(row / limbs);
         out[(size_t)item * out_stride + ((size_t)limb << log_n) + k] =
-            signed_mod(in[(size_t)item * in_stride + k], pr[limb].q);
+            signed_mod(in[(size_t)item * in_stride + k], pr[limb]);
     }
 }
 

@@ -1,0 +1,83 @@
+"""Client side against the oracle: decoding of any number of slots on every size of ring, encryption whose
+ternary stream holds the one output the sampler rejects, and encodings of few and of many distinct values."""
+import numpy as np
+import pytest
+
+from oracle import ckks
+from paper_2509_03024_gb300 import capi
+from tests.gpu_common import assert_ct_equal, built, to_coeff, torch
+
+pytestmark = pytest.mark.gpu
+
+GAMMA, M64 = 0x9E3779B97F4A7C15, (1 << 64) - 1
+
+
+def _unmix64(y):
+    """Inverse of the SplitMix64 output function."""
+    def unshift(v, s):
+        x = v
+        for _ in range(0, 64, s):
+            x = v ^ (x >> s)
+        return x
+    z = unshift(y, 31) * pow(0x94D049BB133111EB, -1, 1 << 64) & M64
+    z = unshift(z, 27) * pow(0xBF58476D1CE4E5B9, -1, 1 << 64) & M64
+    return unshift(z, 30)
+
+
+@pytest.mark.parametrize("log_n", [9, 10, 13, 14, 15])
+def test_decode_matches_direct_sum(log_n):
+    """Slots of decrypted coefficients against the oracle's direct sum of N terms; both are float64 sums of
+    |m_j| / Delta with rounding below (N + 64) 2^-53 of the sum of magnitudes."""
+    built()
+    ctx = capi.Context(log_n, (60, 40), (60,), 40)
+    he = ckks.Ckks(ckks.Params(log_n, (60, 40), (60,), 40))
+    ctx.keygen(3)
+    he.keygen(3)
+    z = np.random.default_rng(log_n).normal(0, 2, 60)
+    for level in (1, 0):
+        ct = ctx.empty_ct()
+        ctx.encrypt(z, level, 17, ct)
+        m = he.decrypt_coeffs(he.encrypt(z, level, 17))
+        tol = (ctx.n + 64) * 2.0 ** -53 * float(sum(abs(int(v)) for v in m)) / 2.0 ** 40
+        for count in (1, 33, ctx.slots if log_n < 14 else 257):
+            got = ctx.decrypt(ct, level, count)
+            assert got.shape == (count,)
+            assert np.abs(got - he.enc.decode(m, count=count)).max() <= tol
+        full = ctx.decrypt(ct, level)
+        assert (full[:33] == ctx.decrypt(ct, level, 33)).all()
+
+
+@pytest.mark.parametrize("at", [1, 2, 700, 1024, 1025])
+def test_encryption_past_a_rejected_ternary_draw(at):
+    """A seed whose ternary stream of nonce 9 outputs 2^64 - 1 (rejected) at counter `at` of N = 1024."""
+    built()
+    h = (_unmix64(M64) - at * GAMMA) & M64               # state before the stream: mix64(h + at gamma) = 2^64 - 1
+    for f in (0, 0, 9, 6):                               # limb, poly, object, purpose
+        h = ((_unmix64(h) - GAMMA) & M64) ^ f
+    data, special = (60, 40, 40), (60,)
+    ctx = capi.Context(10, data, special, 40)
+    ctx.keygen(h)
+    he = ckks.Ckks(ckks.Params(10, data, special, 40))
+    he.keygen(h)
+    assert int(ckks.draws(ckks.stream_key(h, 6, 9), at - 1, 1)[0]) == M64
+    ct = ctx.empty_ct()
+    ctx.encrypt(np.ones(3), 2, 9, ct)
+    assert_ct_equal(to_coeff(ctx, ct, 2)[0], he.encrypt(np.ones(3), 2, 9), "encrypt")
+
+
+@pytest.mark.parametrize("log_n", [9, 11, 14])
+@pytest.mark.parametrize("distinct,count", [(1, 1), (1, 200), (7, 56), (7, 55), (32, 256), (33, 250)])
+def test_encode_few_and_many_distinct_values(log_n, distinct, count):
+    """Both forms of the encoding (products tabulated per distinct value, or formed per term) and the
+    rule between them give the oracle's integers."""
+    built()
+    ctx = capi.Context(log_n, (60, 40), (60,), 40)
+    he = ckks.Ckks(ckks.Params(log_n, (60, 40), (60,), 40))
+    rng = np.random.default_rng(distinct * 1000 + count)
+    vals = rng.normal(0, 3, distinct)
+    z = np.zeros(ctx.slots)
+    slots = np.sort(rng.choice(ctx.slots, count, replace=False))
+    z[slots] = vals[np.arange(count) % distinct]
+    out = torch.zeros(ctx.n, dtype=torch.int64, device="cuda")
+    ctx.encode(z, out)
+    assert np.array_equal(out.cpu().numpy(), he.enc.encode(z))
