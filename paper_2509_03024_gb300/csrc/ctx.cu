@@ -312,10 +312,10 @@ static void build_tables(Ctx& c) {
     }
     c.d_tw = dupload(tw);
     c.d_itw = dupload(itw);
-    // row-pass tables of the two-pass transform (N >= 2^14): row r of N2 entries; stage s of the row
+    // row-pass tables of the two-pass transform (N >= 2^12): row r of N2 entries; stage s of the row
     // transform in entries 2^s .. 2^(s+1) - 1, its group grp = t K + k (T = N2 / 16 threads per row, K =
     // 2^s / T sub-groups per thread) at 2^s + k T + t from stage 4 on, at 2^s + grp before
-    c.ntt_s1 = c.log_n >= 14 ? (c.log_n == 15 ? 7 : c.log_n / 2) : 0;
+    c.ntt_s1 = c.log_n >= 12 ? c.log_n / 2 : 0;
     if (c.ntt_s1) {
         const int S1 = c.ntt_s1, N1 = 1 << S1, N2 = n >> S1, T = N2 / 16;
         std::vector<ulonglong2> t2((size_t)ne * n, make_ulonglong2(0, 0)), it2(t2.size(), make_ulonglong2(0, 0));

@@ -425,7 +425,7 @@ void launch_ks_inner(const InnerArgs& a0, bool fanout, int variant, int max_data
     }
     // split at bit 25 needs data primes below 2^50 and at most 512 terms per sum (MacS25::reduce)
     a.split25 = a.keys_packed && max_data_prime_bits <= 50 && a.dn <= 512;
-    const bool two = (variant == INNER_S2 || variant == INNER_S2L) && !fanout && a.shared_key;
+    const bool two = (variant == INNER_S2 || variant == INNER_S2L) && !fanout && a.shared_key && a.items > 1;
 #define L2(MD, MS, I, F) inner2_kernel<MD, MS, I, F><<<grid2(a, I), 256, 0, s>>>(a)
     switch (variant) {
         case INNER_C1:
@@ -464,8 +464,14 @@ void launch_ks_hoist_inner(const InnerArgs& a0, int variant, int max_data_prime_
     switch (variant) {
         case INNER_C1: H2(MacC, MacC, 1); break;
         case INNER_P1: H2(MacP32, MacP32, 1); break;
-        case INNER_S2: H2(MacS25, MacP32, 2); break;
-        case INNER_S2L: H2(MacK25, MacP32, 2); break;
+        case INNER_S2:
+            if (a.items > 1) H2(MacS25, MacP32, 2);
+            else H2(MacS25, MacP32, 1);
+            break;
+        case INNER_S2L:
+            if (a.items > 1) H2(MacK25, MacP32, 2);
+            else H2(MacK25, MacP32, 1);
+            break;
         default: H2(MacS25, MacP32, 1); break;
     }
 #undef H2

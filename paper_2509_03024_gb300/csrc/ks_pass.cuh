@@ -84,38 +84,56 @@ __device__ __forceinline__ RowConst row_const(const KsRow& r, const Prime* __res
     return c;
 }
 
-// LD_CONV: the base conversion of residue k, sum_i src_i[k] c_i, over CNT sources (loads unconditional,
-// all issued before the products; constants in rc) or any number of them (CNT = 0).
+// LD_CONV: the base conversion of residue k, sum_i src_i[k] c_i: over CNT sources already loaded to x ...
 template <int AR, int CNT>
-__device__ __forceinline__ u64 conv_elem(const KsRow& r, size_t k, int log_n, const nttc::Mod<AR>& m, const RowConst& rc) {
-    if constexpr (CNT > 0) {
-        u64 x[CNT];
+__device__ __forceinline__ u64 conv_sum(const u64 (&x)[CNT], const nttc::Mod<AR>& m, const RowConst& rc) {
+    if constexpr (AR == nttc::AR_NEAR50) {
+        ConvSum s;
 #pragma unroll
-        for (int i = 0; i < CNT; i++) x[i] = r.src[((size_t)i << log_n) + k];
-        if constexpr (AR == nttc::AR_NEAR50) {
-            ConvSum s;
-#pragma unroll
-            for (int i = 0; i < CNT; i++) s.add(x[i], rc.w[i]);
-            return s.value(m.delta);
-        } else {
-            u64 acc = m.mul(x[0], rc.w[0]);
-#pragma unroll
-            for (int i = 1; i < CNT; i++) acc = m.fold(acc) + m.mul(x[i], rc.w[i]);
-            return acc;
-        }
+        for (int i = 0; i < CNT; i++) s.add(x[i], rc.w[i]);
+        return s.value(m.delta);
     } else {
-        u64 acc = 0;
-        for (int i0 = 0; i0 < r.src_cnt; i0 += kConvMax) {
-            ConvSum s;
-            for (int i = i0; i < min(i0 + kConvMax, r.src_cnt); i++) {
-                const u64 x = r.src[((size_t)i << log_n) + k];
-                const ulonglong2 w = words(r.cst + (size_t)i * r.cst_stride);
-                if constexpr (AR == nttc::AR_NEAR50) s.add(x, w);
-                else acc = m.fold(acc) + m.mul(x, w);
-            }
-            if constexpr (AR == nttc::AR_NEAR50) acc += m.fold(s.value(m.delta));
-        }
+        u64 acc = m.mul(x[0], rc.w[0]);
+#pragma unroll
+        for (int i = 1; i < CNT; i++) acc = m.fold(acc) + m.mul(x[i], rc.w[i]);
         return acc;
+    }
+}
+// ... or over any number of them.
+template <int AR>
+__device__ __forceinline__ u64 conv_any(const KsRow& r, size_t k, int log_n, const nttc::Mod<AR>& m) {
+    u64 acc = 0;
+    for (int i0 = 0; i0 < r.src_cnt; i0 += kConvMax) {
+        ConvSum s;
+        for (int i = i0; i < min(i0 + kConvMax, r.src_cnt); i++) {
+            const u64 x = r.src[((size_t)i << log_n) + k];
+            const ulonglong2 w = words(r.cst + (size_t)i * r.cst_stride);
+            if constexpr (AR == nttc::AR_NEAR50) s.add(x, w);
+            else acc = m.fold(acc) + m.mul(x, w);
+        }
+        if constexpr (AR == nttc::AR_NEAR50) acc += m.fold(s.value(m.delta));
+    }
+    return acc;
+}
+// Conversions of V residues, at(u) = conversion of residue addr(u). The loads of several residues are issued
+// together before anything is stored: a store to shared memory in between would order them (the compiler
+// cannot tell the source rows from it), one round trip to L2 per residue.
+template <int AR, int CNT, int V, class ADDR, class AT>
+__device__ __forceinline__ void conv_rows(const KsRow& r, int log_n, const nttc::Mod<AR>& m, const RowConst& rc, ADDR&& addr,
+                                          AT&& at) {
+    if constexpr (CNT == 0) {
+        for (int u = 0; u < V; u++) at(u) = conv_any(r, addr(u), log_n, m);
+    } else {
+        constexpr int G = CNT <= 2 ? 8 : 4;
+        for (int u0 = 0; u0 < V; u0 += G) {
+            u64 x[G][CNT];
+#pragma unroll
+            for (int u = 0; u < G; u++)
+#pragma unroll
+                for (int i = 0; i < CNT; i++) x[u][i] = r.src[((size_t)i << log_n) + addr(u0 + u)];
+#pragma unroll
+            for (int u = 0; u < G; u++) at(u0 + u) = conv_sum<AR, CNT>(x[u], m, rc);
+        }
     }
 }
 // f is called with the number of sources as a compile-time constant (0: more than kConvMax).
@@ -128,7 +146,7 @@ __device__ __forceinline__ void with_count(int cnt, F&& f) {
     else f(nttc::Tag<0>{});
 }
 
-// Residue k of the row as the transform takes it (LD_CONV: conv_elem): a congruent value, for a forward
+// Residue k of the row as the transform takes it (LD_CONV: conv_rows): a congruent value, for a forward
 // transform within 2^60.4 (NEAR50, signed), below 16 q (NEAR60) or 8 q (SHOUP); reduced for an inverse one.
 template <int LOAD, int AR>
 __device__ __forceinline__ u64 load_elem(const KsRow& r, size_t k, int log_n, const Prime& P, const nttc::Mod<AR>& m,
@@ -136,9 +154,7 @@ __device__ __forceinline__ u64 load_elem(const KsRow& r, size_t k, int log_n, co
     if constexpr (LOAD == LD_PLAIN) {
         return r.dst[k];
     } else if constexpr (LOAD == LD_GATHER) {
-        const u64 v = r.src[r.galois == 1 ? (int)k : auto_src((int)k, r.galois, log_n)];
-        if (r.out2) r.out2[k] = r.pack ? key_pack(v) : v;
-        return v;
+        return r.src[r.galois == 1 ? (int)k : auto_src((int)k, r.galois, log_n)];
     } else if constexpr (LOAD == LD_CENTRED) {  // the centred representative of src[k] (mod q_limb)
         const u64 ql = rc.ql, v = r.src[k];
         const bool neg = v > (ql >> 1);
@@ -158,42 +174,50 @@ __device__ __forceinline__ u64 load_elem(const KsRow& r, size_t k, int log_n, co
     }
 }
 
-// Residue k of the row from the transform's (unreduced) value v.
-template <bool INV, int STORE, int AR>
-__device__ __forceinline__ void store_elem(const KsRow& r, size_t k, u64 v, const Prime& P, const nttc::Mod<AR>& m,
-                                           const u64* __restrict__ ninv, const CombineArgs& ca, int log_n) {
-    const u64 q = m.q, one_s = P.one_s;
-    if (STORE == ST_LAZY) {
-        r.dst[k] = v;
-        return;
+// Residue k of the row from the transform's (unreduced) value v, in two steps so that the loads of several
+// residues go out before the first store (which the compiler cannot tell from them): store_operands, then
+// store_elem.
+struct StoreIn {
+    u64 a, b, c;
+};
+template <int STORE>
+__device__ __forceinline__ StoreIn store_operands(const KsRow& r, size_t k, const CombineArgs& ca, int log_n) {
+    StoreIn in{0, 0, 0};
+    if constexpr (STORE == ST_RESCALE) {
+        in.a = r.src2[k];
+        if (r.src3) in.b = r.src3[k];
+    } else if constexpr (STORE == ST_COMBINE || STORE == ST_COMBINE_RS) {
+        const KsItem& it = ca.items[r.item];
+        const size_t row_off = (size_t)r.limb << log_n;
+        in.a = ca.acc[((((size_t)r.item * 2 + r.half) * ca.next + r.limb) << log_n) + k];
+        const u64* add = r.half == 0 ? it.addI0 : it.addI1;
+        if (add) in.b = add[row_off + k];
+        if (STORE == ST_COMBINE && r.half == 0 && it.addP0)
+            in.c = it.addP0[row_off + (it.galois == 1 ? (int)k : auto_src((int)k, (int)it.galois, log_n))];
     }
-    if (STORE == ST_LAST || STORE == ST_SCALE) {  // inverse: times N^-1, or the row's constant in its place
+    return in;
+}
+template <bool INV, int STORE, int AR>
+__device__ __forceinline__ void store_elem(const KsRow& r, size_t k, u64 v, const StoreIn& in, const Prime& P,
+                                           const nttc::Mod<AR>& m, const u64* __restrict__ ninv, const CombineArgs& ca,
+                                           int log_n) {
+    const u64 q = m.q, one_s = P.one_s;
+    if constexpr (STORE == ST_LAZY) {
+        r.dst[k] = v;
+    } else if constexpr (STORE == ST_LAST || STORE == ST_SCALE) {  // inverse: times N^-1, or the row's constant in its place
         const u64 t = m.canon(INV ? m.mul(v, words(STORE == ST_SCALE ? r.cst : ninv + 2 * r.prime)) : v, one_s);
         r.dst[k] = !INV && r.pack ? key_pack(t) : t;
-        return;
-    }
-    const u64 t = m.canon(v, one_s);
-    if (STORE == ST_RESCALE) {  // forward: out = (x - [x_l]) q_l^-1 with the transformed [x_l] in v
-        const u64 x = r.src3 ? mul_mod(r.src2[k], r.src3[k], P) : r.src2[k];
-        r.out2[k] = m.canon(m.mul(x + q - t, words(r.cst2)), one_s);
-        return;
-    }
-    // out_h = (acc_h - v) P^-1 + add terms (Mod::mul's range and two reduced terms fit 64 bits)
-    const KsItem& it = ca.items[r.item];
-    const size_t row_off = (size_t)r.limb << log_n;
-    const u64 a = ca.acc[((((size_t)r.item * 2 + r.half) * ca.next + r.limb) << log_n) + k];
-    u64 s = m.mul(a + q - t, words(ca.pinv + 2 * r.limb));
-    if (STORE == ST_COMBINE_RS) {
-        // fused ModDown + rescale: out_h = (acc_h - conv) (P q_l)^-1 + c_h q_l^-1
-        const u64* c_h = r.half == 0 ? it.addI0 : it.addI1;
-        s += m.mul(c_h[row_off + k], words(ca.qlinv + 2 * r.limb));
-    } else if (r.half == 0) {
-        if (it.addP0) s += it.addP0[row_off + (it.galois == 1 ? (int)k : auto_src((int)k, (int)it.galois, log_n))];
-        if (it.addI0) s += it.addI0[row_off + k];
+    } else if constexpr (STORE == ST_RESCALE) {  // forward: out = (x - [x_l]) q_l^-1 with the transformed [x_l] in v
+        const u64 x = r.src3 ? mul_mod(in.a, in.b, P) : in.a;
+        r.out2[k] = m.canon(m.mul(x + q - m.canon(v, one_s), words(r.cst2)), one_s);
     } else {
-        if (it.addI1) s += it.addI1[row_off + k];
+        // out_h = (acc_h - v) P^-1 + add terms (Mod::mul's range and two reduced terms fit 64 bits); with the fused
+        // rescale (acc_h - v) (P q_l)^-1 + c_h q_l^-1
+        u64 s = m.mul(in.a + q - m.canon(v, one_s), words(ca.pinv + 2 * r.limb));
+        s += STORE == ST_COMBINE_RS ? m.mul(in.b, words(ca.qlinv + 2 * r.limb)) : in.b + in.c;
+        const KsItem& it = ca.items[r.item];
+        (r.half == 0 ? it.out0 : it.out1)[((size_t)r.limb << log_n) + k] = m.canon(s, one_s);
     }
-    (r.half == 0 ? it.out0 : it.out1)[row_off + k] = m.canon(s, one_s);
 }
 
 // ---------------------------------------------------------------- pass kernels
@@ -215,7 +239,7 @@ struct RowBatch {
     }
 };
 
-// Whole transform of one row per CTA (rings up to 2^13).
+// Whole transform of one row per CTA (rings up to 2^11).
 template <class ROWS, int LOGN, bool INV, int LOAD, int STORE>
 __global__ void __launch_bounds__((1 << LOGN) / 8, 1024 / ((1 << LOGN) / 8))
 single_pass_kernel(ROWS rows, const Prime* __restrict__ primes, const ulonglong2* __restrict__ tw,
@@ -225,22 +249,31 @@ single_pass_kernel(ROWS rows, const Prime* __restrict__ primes, const ulonglong2
     const KsRow r = rows.get(blockIdx.x, LOGN);
     const Prime& P = primes[r.prime];
     nttc::with_arith(P, [&](auto ar) {
-        const nttc::Mod<decltype(ar)::value> m(P);
+        constexpr int AR = decltype(ar)::value;
+        const nttc::Mod<AR> m(P);
         const RowConst rc = row_const<LOAD>(r, primes);
+        const int tid = threadIdx.x;
+        auto at = [&](int u) -> u64& { return sm[tid + u * T]; };
+        auto addr = [&](int u) -> size_t { return tid + u * T; };
         if constexpr (LOAD == LD_CONV) {
-            with_count(r.src_cnt, [&](auto cnt) {
-#pragma unroll 4
-                for (int e = threadIdx.x; e < N; e += T)
-                    sm[e] = conv_elem<decltype(ar)::value, decltype(cnt)::value>(r, e, LOGN, m, rc);
-            });
+            with_count(r.src_cnt, [&](auto cnt) { conv_rows<AR, decltype(cnt)::value, 8>(r, LOGN, m, rc, addr, at); });
         } else {
-#pragma unroll 4
-            for (int e = threadIdx.x; e < N; e += T) sm[e] = load_elem<LOAD>(r, e, LOGN, P, m, rc);
+            u64 v[8];
+#pragma unroll
+            for (int u = 0; u < 8; u++) v[u] = load_elem<LOAD>(r, addr(u), LOGN, P, m, rc);
+#pragma unroll
+            for (int u = 0; u < 8; u++) {
+                at(u) = v[u];
+                if (LOAD == LD_GATHER && r.out2) r.out2[addr(u)] = r.pack ? key_pack(v[u]) : v[u];
+            }
         }
         __syncthreads();
         nttc::single_blocks<LOGN, 0, INV>(sm, tw + ((size_t)r.prime << LOGN), m);
-#pragma unroll 2
-        for (int e = threadIdx.x; e < N; e += T) store_elem<INV, STORE>(r, e, sm[e], P, m, ninv, ca, LOGN);
+        StoreIn in[8];
+#pragma unroll
+        for (int u = 0; u < 8; u++) in[u] = store_operands<STORE>(r, addr(u), ca, LOGN);
+#pragma unroll
+        for (int u = 0; u < 8; u++) store_elem<INV, STORE>(r, addr(u), at(u), in[u], P, m, ninv, ca, LOGN);
     });
 }
 
@@ -261,7 +294,8 @@ single_pass_kernel(ROWS rows, const Prime* __restrict__ primes, const ulonglong2
 // What bounds it: the 32-bit multiply pipe (ntt_core.cuh) and, in passes whose loads convert, the latency
 // of their loads. Plain forward + inverse transform of 256 rows, N = 2^15 / 2^16 (ms): radix-8 tiles filled
 // from shared memory with Shoup products 0.205 / 0.424, the same with split products 0.176 / 0.372,
-// these passes 0.140 / 0.306; ModUp conversion pass set of 64 top-level inputs 1.032 / 4.66 -> 0.717 / 3.00.
+// these passes 0.140 / 0.306; ModUp conversion pass set of 64 top-level inputs 1.032 / 4.66 -> 0.717 / 3.00, and 0.595 / 2.64 with the loads of several residues
+// issued before the first store.
 template <class ROWS, int LOGN, int LOGM, int R, bool INV, int PASS, int LOAD, int STORE, int RB, int MINB>
 __global__ void __launch_bounds__(R * (1 << LOGM) / (1 << RB), MINB)
 pass_kernel(ROWS rows, int n_rows, int per_cta, const Prime* __restrict__ primes, const ulonglong2* __restrict__ tw,
@@ -318,20 +352,20 @@ pass_kernel(ROWS rows, int n_rows, int per_cta, const Prime* __restrict__ primes
             };
             // loads and stores with arithmetic of their own run in short loops over the thread's own
             // shared-memory elements: unrolled over the registers they overflow the instruction cache
+            const RowConst rc = row_const<LOAD>(r, primes);
             if constexpr (LOAD == LD_CONV) {
-                const RowConst rc = row_const<LOAD>(r, primes);
                 with_count(r.src_cnt, [&](auto cnt) {
-#pragma unroll 8
-                    for (int u = 0; u < V; u++)
-                        at(g + T * u) = conv_elem<AR, decltype(cnt)::value>(r, addr(g + T * u), LOGN, m, rc);
+                    conv_rows<AR, decltype(cnt)::value, V>(
+                        r, LOGN, m, rc, [&](int u) { return addr(g + T * u); }, [&](int u) -> u64& { return at(g + T * u); });
                 });
                 take(-1);
             } else {
-                const RowConst rc = row_const<LOAD>(r, primes);
 #pragma unroll
-                for (int u = 0; u < V; u++) {
-                    const int x = INV && PASS == 0 ? elem(NB - 1, u) : g + T * u;
-                    v[u] = load_elem<LOAD>(r, addr(x), LOGN, P, m, rc);
+                for (int u = 0; u < V; u++)
+                    v[u] = load_elem<LOAD>(r, addr(INV && PASS == 0 ? elem(NB - 1, u) : g + T * u), LOGN, P, m, rc);
+                if (LOAD == LD_GATHER && r.out2) {
+#pragma unroll
+                    for (int u = 0; u < V; u++) r.out2[addr(g + T * u)] = r.pack ? key_pack(v[u]) : v[u];
                 }
             }
             if constexpr (!INV) {
@@ -359,13 +393,20 @@ pass_kernel(ROWS rows, int n_rows, int per_cta, const Prime* __restrict__ primes
             if (!INV && PASS == 1) {
                 put(NB - 1);
                 sync();
-#pragma unroll 4
-                for (int u = 0; u < V; u++) store_elem<INV, STORE>(r, addr(g + T * u), at(g + T * u), P, m, ninv, ca, LOGN);
+                constexpr int G = STORE == ST_COMBINE || STORE == ST_RESCALE ? 4 : 8;
+                for (int u0 = 0; u0 < V; u0 += G) {
+                    StoreIn in[G];
+#pragma unroll
+                    for (int u = 0; u < G; u++) in[u] = store_operands<STORE>(r, addr(g + T * (u0 + u)), ca, LOGN);
+#pragma unroll
+                    for (int u = 0; u < G; u++)
+                        store_elem<INV, STORE>(r, addr(g + T * (u0 + u)), at(g + T * (u0 + u)), in[u], P, m, ninv, ca, LOGN);
+                }
                 sync();
             } else {
 #pragma unroll
                 for (int u = 0; u < V; u++)
-                    store_elem<INV, STORE>(r, addr(!INV ? elem(NB - 1, u) : g + T * u), v[u], P, m, ninv, ca, LOGN);
+                    store_elem<INV, STORE>(r, addr(!INV ? elem(NB - 1, u) : g + T * u), v[u], StoreIn{}, P, m, ninv, ca, LOGN);
             }
         });
     }
@@ -399,8 +440,10 @@ void launch_single(const Ctx& c, const ROWS& rows, int n_rows, const CombineArgs
 }
 
 // A full forward (INV = false) or inverse transform over the rows: the first pass applies LOAD, the
-// last pass applies STORE (rings up to 2^13 do both in one kernel). The column passes of a ring of 2^15
-// have 2^7 points, its row passes 2^8. TPS: threads per SM the register cap of the kernels leaves room for.
+// last pass applies STORE (rings up to 2^11 do both in one kernel). The column passes of a ring of 2^15
+// have 2^7 points, its row passes 2^8. Rings of 2^12 and 2^13 in two passes: a row spreads over several SMs
+// and the kernels are the register-direct ones (two polynomials of three limbs at 2^13, forward and inverse with
+// their copies: 51 -> 35 us). TPS: threads per SM the register cap of the kernels leaves room for.
 template <class ROWS, bool INV, int LOAD, int STORE, int R, int RB, int TPS>
 void transform_t(const Ctx& c, const ROWS& rows, int n_rows, const CombineArgs& ca, int cls, double bytes, cudaStream_t s) {
     if (n_rows == 0) return;
@@ -409,8 +452,6 @@ void transform_t(const Ctx& c, const ROWS& rows, int n_rows, const CombineArgs& 
             case 9: launch_single<ROWS, 9, INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s); return;
             case 10: launch_single<ROWS, 10, INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s); return;
             case 11: launch_single<ROWS, 11, INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s); return;
-            case 12: launch_single<ROWS, 12, INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s); return;
-            case 13: launch_single<ROWS, 13, INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s); return;
             default: break;
         }
     }
@@ -420,6 +461,8 @@ void transform_t(const Ctx& c, const ROWS& rows, int n_rows, const CombineArgs& 
         launch_pass<ROWS, LG, INV ? LC : LG - LC, R, INV, INV ? 0 : 1, LD_PLAIN, STORE, RB, TPS>(c, rows, n_rows, ca, cls, bytes, s); \
         return;
     switch (c.log_n) {
+        TWO(12, 6)
+        TWO(13, 6)
         TWO(14, 7)
         TWO(15, 7)
         TWO(16, 8)
@@ -462,8 +505,9 @@ void ks_transform_r8x(const Ctx& c, const KsRow* rows, int n_rows, const Combine
 template <bool INV, int LOAD, int STORE>
 void ks_transform(const Ctx& c, const KsRow* rows, int n_rows, const CombineArgs& ca, int cls, double bytes,
                   cudaStream_t s) {
-    if (c.log_n < 14) ks_transform_r16<INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s);
-    else if (c.tune.ks == KS_R8) ks_transform_r8<INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s);
+    // (the rings below 2^14 are not tuned: small tiles, for the CTAs)
+    if (c.log_n < 12) ks_transform_r16<INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s);
+    else if (c.log_n < 14 || c.tune.ks == KS_R8) ks_transform_r8<INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s);
     else if (c.tune.ks == KS_R8X) ks_transform_r8x<INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s);
     else ks_transform_r16<INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s);
 }

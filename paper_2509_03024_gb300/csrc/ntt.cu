@@ -7,7 +7,7 @@
 // Decomposition. A ring of N = N1 * N2 coefficients is viewed as N1 rows of
 // N2: the first log2(N1) stages couple elements N2 apart (independent
 // N1-point transforms on columns), the remaining stages couple elements inside
-// one row (N2-point transforms with row-dependent twiddles). Rings up to 2^13
+// one row (N2-point transforms with row-dependent twiddles). Rings up to 2^11
 // run in one pass (one CTA per limb); larger rings in two passes, one kernel
 // each (pass_kernel in ks_pass.cuh). Values stay unreduced between stages
 // wherever 64 bits allow it (ntt_core.cuh); the last pass reduces to [0, q).
@@ -26,7 +26,7 @@ using namespace ntt_tile;
 template <bool INV>
 void run_ntt(const Ctx& c, const PolyBatch& pb, cudaStream_t s) {
     const double bytes = 16.0 * pb.rows() * ((size_t)1 << c.log_n);
-    switch (c.log_n < 14 ? NTT_R16B4 : c.tune.ntt) {
+    switch (c.log_n < 12 ? NTT_R16B4 : c.log_n < 14 ? NTT_R8B4 : c.tune.ntt) {
         case NTT_R8B4: transform_r8b4(c, pb, INV, s, bytes); return;
         case NTT_R32B4: transform_r32b4(c, pb, INV, s, bytes); return;
         case NTT_R16B3: transform_r16b3(c, pb, INV, s, bytes); return;
