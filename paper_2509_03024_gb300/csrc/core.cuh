@@ -178,13 +178,27 @@ struct Arena {
     };
     Half halves[2];
     int h = 0;
+    // between gather() and upload(s) pushes only stage their data: upload enqueues one copy for all of them
+    // (per block), which must precede the work that reads them
+    bool gathering = false;
+    size_t from = 0;  // first byte of the current block not yet uploaded
     void reset(cudaStream_t s);
     void* push(const void* data, size_t bytes, cudaStream_t s);
+    void gather();
+    void upload(cudaStream_t s);
+    void upload_block(cudaStream_t s);
     template <typename T>
     T* push_vec(const std::vector<T>& v, cudaStream_t s) {
         return (T*)push(v.data(), v.size() * sizeof(T), s);
     }
     ~Arena();
+};
+// Scope of one gather: an exception between gather() and upload() leaves no half-open state.
+struct ArenaGather {
+    Arena& a;
+    explicit ArenaGather(Arena& arena) : a(arena) { a.gather(); }
+    void upload(cudaStream_t s) { a.upload(s); }
+    ~ArenaGather() { a.gathering = false; }
 };
 
 // ----------------------------------------------------------------------------- launch accounting

@@ -95,8 +95,13 @@ __global__ void fanin_sum_kernel(const FanRow* __restrict__ rows, const FanSrc* 
     }
 }
 
-void moddown_run(Ctx& c, const std::vector<KsItem>& it, const KsItem* d_items, const u64* acc, int level,
-                 cudaStream_t s);
+// K4 and K5 row tables of a ModDown, uploaded.
+struct DownRows {
+    const KsRow *r4, *r5;
+    int n4, n5;
+};
+DownRows moddown_rows(Ctx& c, int items, const u64* acc, int level, cudaStream_t s);
+void moddown_run(Ctx& c, const DownRows& d, const KsItem* d_items, const u64* acc, int level, cudaStream_t s);
 
 void ks_run(Ctx& c, const std::vector<KsItem>& all, int level, const HoistKeys* hk, cudaStream_t s,
             bool fused_rescale = false, const std::vector<int>* fanout_src = nullptr, const FanIn* fi = nullptr) {
@@ -130,8 +135,6 @@ void ks_run(Ctx& c, const std::vector<KsItem>& all, int level, const HoistKeys* 
         }
         b0 += items;
         const int n_sources = (int)src_first.size();
-        const KsItem* d_items = c.arena.push_vec(it, s);
-        const int* d_src_of = fan ? c.arena.push_vec(src_of, s) : nullptr;
         size_t nkeys = 0;
         {
             std::vector<const u64*> ks;
@@ -142,10 +145,13 @@ void ks_run(Ctx& c, const std::vector<KsItem>& all, int level, const HoistKeys* 
         u64* y = c.scratch_u64("ks_y", (size_t)n_sources * l1 * n);
         u64* ext = c.scratch_u64("ks_ext", (size_t)n_sources * dn * next * n);
         u64* acc = c.scratch_u64("ks_acc", (size_t)items * 2 * next * n);
-        u64* yP = fi ? nullptr : c.scratch_u64("ks_yp", (size_t)items * 2 * SP * n);
-        u64* conv = fi ? nullptr : c.scratch_u64("ks_conv", (size_t)items * 2 * l1 * n);
-        CombineArgs ca{d_items, acc, c.d_pinv, next, nullptr};
+        u64* c0sum = hk ? c.scratch_u64("ks_c0sum", (size_t)items * l1 * n) : nullptr;
         const CombineArgs none{nullptr, nullptr, nullptr, 0, nullptr};
+
+        // every table of the sub-batch goes up in one copy before its first kernel
+        ArenaGather tables(c.arena);
+        const KsItem* d_items = c.arena.push_vec(it, s);
+        const int* d_src_of = fan ? c.arena.push_vec(src_of, s) : nullptr;
 
         // K1: y_i = INTT(perm(d_i)) * qhat_i^-1 (fan-out: once per source, no permutation); its loads also
         // store perm(d_i) as limb i of its own raised digit
@@ -165,7 +171,6 @@ void ks_run(Ctx& c, const std::vector<KsItem>& all, int level, const HoistKeys* 
                 r1.push_back(r);
             }
         const KsRow* d_r1 = c.arena.push_vec(r1, s);
-        ks_transform<true, LD_GATHER, ST_SCALE>(c, d_r1, (int)r1.size(), none, K_NTT_INV, 16.0 * r1.size() * n, s);
 
         // K2: ModUp_j(d)_x for x outside D_j
         std::vector<KsRow> r2;
@@ -189,6 +194,67 @@ void ks_run(Ctx& c, const std::vector<KsItem>& all, int level, const HoistKeys* 
                 }
             }
         const KsRow* d_r2 = c.arena.push_vec(r2, s);
+
+        const HoistStep* d_steps = nullptr;
+        const KsItem* d_items5 = d_items;
+        if (hk) {
+            std::vector<HoistStep> hs;
+            for (int r = 0; r < hk->count; r++) hs.push_back({hk->key[r], (long long)hk->galois[r]});
+            d_steps = c.arena.push_vec(hs, s);
+            // the combine adds c0sum to component 0 and c1 to component 1
+            std::vector<KsItem> it5(it);
+            for (int t = 0; t < items; t++) {
+                it5[t].addP0 = nullptr;
+                it5[t].addI0 = c0sum + (size_t)t * l1 * n;
+                it5[t].addI1 = it[t].d;
+            }
+            d_items5 = c.arena.push_vec(it5, s);
+        }
+        DownRows down{};
+        if (fused_rescale) {
+            u64* yP = c.scratch_u64("ks_yp", (size_t)items * 2 * SP * n);
+            u64* conv = c.scratch_u64("ks_conv", (size_t)items * 2 * l1 * n);
+            // K4: y_s = INTT(source s) * N^-1 (M'/m_s)^-1 for m_s = p_0.., p_{alpha-1}, q_l, where the q_l
+            // source is acc_h + (P mod q_l) c_h
+            std::vector<KsRow> r4, r5;
+            for (int t = 0; t < items; t++)
+                for (int h = 0; h < 2; h++)
+                    for (int sx = 0; sx < SP; sx++) {
+                        KsRow r{};
+                        r.dst = yP + (((size_t)t * 2 + h) * SP + sx) * n;
+                        const bool ql = sx == A;
+                        r.src = acc + (((size_t)t * 2 + h) * next + (ql ? level : l1 + sx)) * n;
+                        r.src2 = ql ? (h == 0 ? it[t].addI0 : it[t].addI1) + (size_t)level * n : nullptr;
+                        r.cst2 = c.d_fd_pq + 2 * (size_t)level;
+                        r.cst = c.d_fd_ninv + 2 * ((size_t)level * SP + sx);
+                        r.prime = ql ? level : L + 1 + sx;
+                        r.galois = 1;
+                        r4.push_back(r);
+                    }
+            // K5: out_h = (acc_h - NTT(Conv(y))) (P q_l)^-1 + c_h q_l^-1 for limbs i < level
+            for (int t = 0; t < items; t++)
+                for (int h = 0; h < 2; h++)
+                    for (int i = 0; i < level; i++) {
+                        KsRow r{};
+                        r.dst = conv + (((size_t)t * 2 + h) * l1 + i) * n;
+                        r.src = yP + ((size_t)t * 2 + h) * SP * n;
+                        r.cst = c.d_fd_hat + 2 * ((size_t)level * SP * (L + 1) + i);
+                        r.cst_stride = 2 * (L + 1);
+                        r.src_cnt = SP;
+                        r.prime = i;
+                        r.galois = 1;
+                        r.item = t;
+                        r.half = h;
+                        r.limb = i;
+                        r5.push_back(r);
+                    }
+            down = {c.arena.push_vec(r4, s), c.arena.push_vec(r5, s), (int)r4.size(), (int)r5.size()};
+        } else if (!fi) {
+            down = moddown_rows(c, items, acc, level, s);
+        }
+        tables.upload(s);
+
+        ks_transform<true, LD_GATHER, ST_SCALE>(c, d_r1, (int)r1.size(), none, K_NTT_INV, 16.0 * r1.size() * n, s);
         ks_transform<false, LD_CONV, ST_LAST>(c, d_r2, (int)r2.size(), none, K_NTT_FWD, 16.0 * r2.size() * n, s);
 
         // K3: key inner product
@@ -217,69 +283,21 @@ void ks_run(Ctx& c, const std::vector<KsItem>& all, int level, const HoistKeys* 
             launch_ks_inner(ia, fan, c.tune.inner, c.max_data_prime_bits, s);
         } else {
             // reads: the raised digits and c0 once per item, every key once; writes acc and c0sum
-            u64* c0sum = c.scratch_u64("ks_c0sum", (size_t)items * l1 * n);
             LaunchScope _ls(c.prof, K_KS_INNER,
                             8.0 * n * ((double)items * (dn * next + l1) + (double)hk->count * dn * 2 * next +
                                        (double)items * (2 * next + l1)),
                             s, 2.0 * items * next * n * dn * hk->count);
-            std::vector<HoistStep> hs;
-            for (int r = 0; r < hk->count; r++) hs.push_back({hk->key[r], (long long)hk->galois[r]});
-            ia.steps = c.arena.push_vec(hs, s);
+            ia.steps = d_steps;
             ia.n_steps = hk->count;
             ia.c0sum = c0sum;
             launch_ks_hoist_inner(ia, c.tune.hoist, c.max_data_prime_bits, s);
-            // the combine adds c0sum to component 0 and c1 to component 1
-            std::vector<KsItem> it5(it);
-            for (int t = 0; t < items; t++) {
-                it5[t].addP0 = nullptr;
-                it5[t].addI0 = c0sum + (size_t)t * l1 * n;
-                it5[t].addI1 = it[t].d;
-            }
-            ca.items = c.arena.push_vec(it5, s);
         }
 
         if (fused_rescale) {
-            // K4: y_s = INTT(source s) * N^-1 (M'/m_s)^-1 for m_s = p_0.., p_{alpha-1}, q_l, where the q_l
-            // source is acc_h + (P mod q_l) c_h
-            std::vector<KsRow> r4;
-            for (int t = 0; t < items; t++)
-                for (int h = 0; h < 2; h++)
-                    for (int sx = 0; sx < SP; sx++) {
-                        KsRow r{};
-                        r.dst = yP + (((size_t)t * 2 + h) * SP + sx) * n;
-                        const bool ql = sx == A;
-                        r.src = acc + (((size_t)t * 2 + h) * next + (ql ? level : l1 + sx)) * n;
-                        r.src2 = ql ? (h == 0 ? it[t].addI0 : it[t].addI1) + (size_t)level * n : nullptr;
-                        r.cst2 = c.d_fd_pq + 2 * (size_t)level;
-                        r.cst = c.d_fd_ninv + 2 * ((size_t)level * SP + sx);
-                        r.prime = ql ? level : L + 1 + sx;
-                        r.galois = 1;
-                        r4.push_back(r);
-                    }
-            const KsRow* d_r4 = c.arena.push_vec(r4, s);
-            ks_transform<true, LD_AXPY, ST_SCALE>(c, d_r4, (int)r4.size(), none, K_NTT_INV, 16.0 * r4.size() * n, s);
-            // K5: out_h = (acc_h - NTT(Conv(y))) (P q_l)^-1 + c_h q_l^-1 for limbs i < level
-            std::vector<KsRow> r5;
-            for (int t = 0; t < items; t++)
-                for (int h = 0; h < 2; h++)
-                    for (int i = 0; i < level; i++) {
-                        KsRow r{};
-                        r.dst = conv + (((size_t)t * 2 + h) * l1 + i) * n;
-                        r.src = yP + ((size_t)t * 2 + h) * SP * n;
-                        r.cst = c.d_fd_hat + 2 * ((size_t)level * SP * (L + 1) + i);
-                        r.cst_stride = 2 * (L + 1);
-                        r.src_cnt = SP;
-                        r.prime = i;
-                        r.galois = 1;
-                        r.item = t;
-                        r.half = h;
-                        r.limb = i;
-                        r5.push_back(r);
-                    }
             CombineArgs cr{d_items, acc, c.d_fd_minv + 2 * (size_t)level * (L + 1), next,
                            c.d_resc_w + 2 * (size_t)level * (L + 1)};
-            const KsRow* d_r5 = c.arena.push_vec(r5, s);
-            ks_transform<false, LD_CONV, ST_COMBINE_RS>(c, d_r5, (int)r5.size(), cr, K_NTT_FWD, 16.0 * r5.size() * n, s);
+            ks_transform<true, LD_AXPY, ST_SCALE>(c, down.r4, down.n4, none, K_NTT_INV, 16.0 * down.n4 * n, s);
+            ks_transform<false, LD_CONV, ST_COMBINE_RS>(c, down.r5, down.n5, cr, K_NTT_FWD, 16.0 * down.n5 * n, s);
             continue;
         }
         if (fi) {
@@ -304,66 +322,64 @@ void ks_run(Ctx& c, const std::vector<KsItem>& all, int level, const HoistKeys* 
                 }
                 t0 = t1;
             }
+            ArenaGather sums(c.arena);
             const FanRow* d_fr = c.arena.push_vec(fr, s);
             const FanSrc* d_fs = c.arena.push_vec(fs, s);
+            sums.upload(s);
             LaunchScope _ls(c.prof, K_ELEMENTWISE, 8.0 * n * (fs.size() + 2.0 * fr.size()), s);
             const size_t total = fr.size() * (size_t)n;
             fanin_sum_kernel<<<grid1(total), 256, 0, s>>>(d_fr, d_fs, (int)fr.size(), c.log_n, c.d_primes);
             CK(cudaGetLastError());
             continue;
         }
-        moddown_run(c, it, ca.items, acc, level, s);
+        moddown_run(c, down, d_items5, acc, level, s);
     }
 }
 
 // K4/K5 of a plain key switch over the items' accumulators acc ([item][2][next][N]): out_h =
 // (acc_h - Conv_{P->Q}(acc_h)) P^-1 + the item's add terms.
-void moddown_run(Ctx& c, const std::vector<KsItem>& it, const KsItem* d_items, const u64* acc, int level,
-                 cudaStream_t s) {
+DownRows moddown_rows(Ctx& c, int items, const u64* acc, int level, cudaStream_t s) {
     const int n = c.n, L = c.L, A = c.alpha, l1 = level + 1, next = l1 + A;
-    const int items = (int)it.size();
     u64* yP = c.scratch_u64("ks_yp", (size_t)items * 2 * A * n);
     u64* conv = c.scratch_u64("ks_conv", (size_t)items * 2 * l1 * n);
-    const CombineArgs ca{d_items, acc, c.d_pinv, next, nullptr};
-    const CombineArgs none{nullptr, nullptr, nullptr, 0, nullptr};
-    {
-        // K4: y_k = INTT(acc_h special limb k) * Phat_k^-1
-        std::vector<KsRow> r4;
-        for (int t = 0; t < items; t++)
-            for (int h = 0; h < 2; h++)
-                for (int kk = 0; kk < A; kk++) {
-                    KsRow r{};
-                    r.dst = yP + (((size_t)t * 2 + h) * A + kk) * n;
-                    r.src = acc + (((size_t)t * 2 + h) * next + l1 + kk) * n;
-                    r.cst = c.d_down_ninv + 2 * kk;
-                    r.prime = L + 1 + kk;
-                    r.galois = 1;
-                    r4.push_back(r);
-                }
-        const KsRow* d_r4 = c.arena.push_vec(r4, s);
-        ks_transform<true, LD_GATHER, ST_SCALE>(c, d_r4, (int)r4.size(), none, K_NTT_INV, 16.0 * r4.size() * n, s);
+    // K4: y_k = INTT(acc_h special limb k) * Phat_k^-1
+    std::vector<KsRow> r4, r5;
+    for (int t = 0; t < items; t++)
+        for (int h = 0; h < 2; h++)
+            for (int kk = 0; kk < A; kk++) {
+                KsRow r{};
+                r.dst = yP + (((size_t)t * 2 + h) * A + kk) * n;
+                r.src = acc + (((size_t)t * 2 + h) * next + l1 + kk) * n;
+                r.cst = c.d_down_ninv + 2 * kk;
+                r.prime = L + 1 + kk;
+                r.galois = 1;
+                r4.push_back(r);
+            }
+    // K5: out_h = (acc_h - NTT(Conv_{P->Q}(y))) * P^-1 + add terms
+    for (int t = 0; t < items; t++)
+        for (int h = 0; h < 2; h++)
+            for (int i = 0; i < l1; i++) {
+                KsRow r{};
+                r.dst = conv + (((size_t)t * 2 + h) * l1 + i) * n;
+                r.src = yP + ((size_t)t * 2 + h) * A * n;
+                r.cst = c.d_down_hat + 2 * (size_t)i;
+                r.cst_stride = 2 * (L + 1);
+                r.src_cnt = A;
+                r.prime = i;
+                r.galois = 1;
+                r.item = t;
+                r.half = h;
+                r.limb = i;
+                r5.push_back(r);
+            }
+    return {c.arena.push_vec(r4, s), c.arena.push_vec(r5, s), (int)r4.size(), (int)r5.size()};
+}
 
-        // K5: out_h = (acc_h - NTT(Conv_{P->Q}(y))) * P^-1 + add terms
-        std::vector<KsRow> r5;
-        for (int t = 0; t < items; t++)
-            for (int h = 0; h < 2; h++)
-                for (int i = 0; i < l1; i++) {
-                    KsRow r{};
-                    r.dst = conv + (((size_t)t * 2 + h) * l1 + i) * n;
-                    r.src = yP + ((size_t)t * 2 + h) * A * n;
-                    r.cst = c.d_down_hat + 2 * (size_t)i;
-                    r.cst_stride = 2 * (L + 1);
-                    r.src_cnt = A;
-                    r.prime = i;
-                    r.galois = 1;
-                    r.item = t;
-                    r.half = h;
-                    r.limb = i;
-                    r5.push_back(r);
-                }
-        const KsRow* d_r5 = c.arena.push_vec(r5, s);
-        ks_transform<false, LD_CONV, ST_COMBINE>(c, d_r5, (int)r5.size(), ca, K_NTT_FWD, 16.0 * r5.size() * n, s);
-    }
+void moddown_run(Ctx& c, const DownRows& d, const KsItem* d_items, const u64* acc, int level, cudaStream_t s) {
+    const CombineArgs ca{d_items, acc, c.d_pinv, level + 1 + c.alpha, nullptr};
+    const CombineArgs none{nullptr, nullptr, nullptr, 0, nullptr};
+    ks_transform<true, LD_GATHER, ST_SCALE>(c, d.r4, d.n4, none, K_NTT_INV, 16.0 * d.n4 * c.n, s);
+    ks_transform<false, LD_CONV, ST_COMBINE>(c, d.r5, d.n5, ca, K_NTT_FWD, 16.0 * d.n5 * c.n, s);
 }
 
 }  // namespace
@@ -418,12 +434,13 @@ void rescale_run(Ctx& c, const std::vector<const u64*>& in, const std::vector<co
                     rb.push_back(q);
                 }
             }
-        const KsRow* d_ra = c.arena.push_vec(ra, s);
+        ArenaGather tables(c.arena);
+        const KsRow *d_ra = c.arena.push_vec(ra, s), *d_rb = c.arena.push_vec(rb, s);
+        tables.upload(s);
         if (prod)
             ks_transform<true, LD_MUL, ST_SCALE>(c, d_ra, (int)ra.size(), none, K_NTT_INV, 16.0 * ra.size() * n, s);
         else
             ks_transform<true, LD_GATHER, ST_SCALE>(c, d_ra, (int)ra.size(), none, K_NTT_INV, 16.0 * ra.size() * n, s);
-        const KsRow* d_rb = c.arena.push_vec(rb, s);
         ks_transform<false, LD_CENTRED, ST_RESCALE>(c, d_rb, (int)rb.size(), none, K_NTT_FWD, 16.0 * rb.size() * n, s);
     }
 }
@@ -515,7 +532,11 @@ void rotate_fanin_items(Ctx& c, const std::vector<u64*>& acc, const std::vector<
             u64* a = acc[gs[g0 + g]];
             gi.push_back({nullptr, nullptr, gc0 + (size_t)g * l1 * n, a, a + lw, a, a + lw, 1});
         }
-        moddown_run(c, gi, c.arena.push_vec(gi, s), gacc, level, s);
+        ArenaGather tables(c.arena);
+        const KsItem* d_gi = c.arena.push_vec(gi, s);
+        const DownRows down = moddown_rows(c, groups, gacc, level, s);
+        tables.upload(s);
+        moddown_run(c, down, d_gi, gacc, level, s);
     }
 }
 

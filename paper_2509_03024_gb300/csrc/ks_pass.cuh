@@ -497,8 +497,17 @@ template <bool INV, int LOAD, int STORE>
 void ks_transform_r8(const Ctx& c, const KsRow* rows, int n_rows, const CombineArgs& ca, int cls, double bytes,
                      cudaStream_t s);
 template <bool INV, int LOAD, int STORE>
+void ks_transform_few(const Ctx& c, const KsRow* rows, int n_rows, const CombineArgs& ca, int cls, double bytes,
+                      cudaStream_t s);
+template <bool INV, int LOAD, int STORE>
 void ks_transform_r8x(const Ctx& c, const KsRow* rows, int n_rows, const CombineArgs& ca, int cls, double bytes,
                       cudaStream_t s);
+
+// Launches of few rows leave an SM with a handful of warps, each a serial chain of 16-residue register
+// blocks; with 8 residues per thread (ks_pass_few.cu, 16 rows or columns per tile) the chain is half as long and
+// the warps twice as many. The line: less than 16 warps per SM at 16 residues per thread. One rotation at N = 2^16 with
+// it and with one table upload per key switch 214 -> 170 us, one product at N = 2^13 111 -> 72 us.
+inline bool few_rows(const Ctx& c, int n_rows) { return ((size_t)n_rows << (c.log_n - 4)) < (size_t)152 * 512; }
 
 // A full forward (INV = false) or inverse transform over a row table with the context's tile shape:
 // the first pass applies LOAD, the last pass applies STORE (single-pass rings do both in one kernel).
@@ -507,6 +516,7 @@ void ks_transform(const Ctx& c, const KsRow* rows, int n_rows, const CombineArgs
                   cudaStream_t s) {
     // (the rings below 2^14 are not tuned: small tiles, for the CTAs)
     if (c.log_n < 12) ks_transform_r16<INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s);
+    else if (few_rows(c, n_rows)) ks_transform_few<INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s);
     else if (c.log_n < 14 || c.tune.ks == KS_R8) ks_transform_r8<INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s);
     else if (c.tune.ks == KS_R8X) ks_transform_r8x<INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s);
     else ks_transform_r16<INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s);

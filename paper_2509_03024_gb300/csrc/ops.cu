@@ -34,7 +34,11 @@ void Arena::reset(cudaStream_t s) {
 void* Arena::push(const void* data, size_t bytes, cudaStream_t s) {
     Half& hf = halves[h];
     const size_t span = std::max<size_t>((bytes + 255) & ~(size_t)255, 256);
-    while (hf.cur < hf.blocks.size() && hf.blocks[hf.cur].used + span > hf.blocks[hf.cur].cap) hf.cur++;
+    while (hf.cur < hf.blocks.size() && hf.blocks[hf.cur].used + span > hf.blocks[hf.cur].cap) {
+        if (gathering) upload_block(s);
+        hf.cur++;
+        from = hf.cur < hf.blocks.size() ? hf.blocks[hf.cur].used : 0;
+    }
     if (hf.cur == hf.blocks.size()) {
         Block b;
         b.cap = std::max<size_t>(span, (size_t)4 << 20);
@@ -48,9 +52,28 @@ void* Arena::push(const void* data, size_t bytes, cudaStream_t s) {
     b.used += span;
     if (bytes) {
         std::memcpy(hp, data, bytes);
-        CK(cudaMemcpyAsync(d, hp, bytes, cudaMemcpyHostToDevice, s));
+        if (!gathering) CK(cudaMemcpyAsync(d, hp, bytes, cudaMemcpyHostToDevice, s));
     }
     return d;
+}
+
+void Arena::upload_block(cudaStream_t s) {
+    Half& hf = halves[h];
+    if (hf.cur >= hf.blocks.size()) return;
+    Block& b = hf.blocks[hf.cur];
+    if (b.used > from) CK(cudaMemcpyAsync(b.dev + from, b.host + from, b.used - from, cudaMemcpyHostToDevice, s));
+    from = b.used;
+}
+
+void Arena::gather() {
+    const Half& hf = halves[h];
+    gathering = true;
+    from = hf.cur < hf.blocks.size() ? hf.blocks[hf.cur].used : 0;
+}
+
+void Arena::upload(cudaStream_t s) {
+    gathering = false;
+    upload_block(s);
 }
 
 Arena::~Arena() {
@@ -426,8 +449,10 @@ void items_tensor(Ctx& c, const std::vector<BinItem>& it, int limbs, cudaStream_
 void items_tensor_acc(Ctx& c, const std::vector<AccTarget>& tg, const std::vector<BinItem>& contrib, int limbs,
                       cudaStream_t s) {
     if (tg.empty()) return;
+    ArenaGather tables(c.arena);
     const AccTarget* dt = upload(c, tg, s);
     const BinItem* dc = upload(c, contrib, s);
+    tables.upload(s);
     size_t per = (size_t)limbs * c.n / 2;
     {
         LaunchScope _ls(c.prof, K_TENSOR, 8.0 * per * 2 * (4.0 * contrib.size() + 6.0 * tg.size()), s);
@@ -440,8 +465,10 @@ void items_tensor_acc(Ctx& c, const std::vector<AccTarget>& tg, const std::vecto
 void items_sum_acc(Ctx& c, const std::vector<AccTarget>& tg, const std::vector<BinItem>& contrib, int parts,
                    int limbs, cudaStream_t s) {
     if (tg.empty()) return;
+    ArenaGather tables(c.arena);
     const AccTarget* dt = upload(c, tg, s);
     const BinItem* dc = upload(c, contrib, s);
+    tables.upload(s);
     size_t per = (size_t)parts * limbs * c.n / 2;
     {
         LaunchScope _ls(c.prof, K_ELEMENTWISE, 8.0 * per * 2 * (contrib.size() + 2.0 * tg.size()), s);
