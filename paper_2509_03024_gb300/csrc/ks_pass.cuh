@@ -166,7 +166,7 @@ __device__ __forceinline__ u64 load_elem(const KsRow& r, size_t k, int log_n, co
             return neg ? (t ? P.q - t : 0) : t;
         }
     } else if constexpr (LOAD == LD_MUL) {
-        return mul_mod(r.src[k], r.src2[k], P);
+        return nttc::product(r.src[k], r.src2[k], m, P);
     } else {  // LD_AXPY: src + cst2 * src2
         static_assert(LOAD == LD_AXPY, "load mode");
         const u64 v = r.src[k];
@@ -208,7 +208,7 @@ __device__ __forceinline__ void store_elem(const KsRow& r, size_t k, u64 v, cons
         const u64 t = m.canon(INV ? m.mul(v, words(STORE == ST_SCALE ? r.cst : ninv + 2 * r.prime)) : v, one_s);
         r.dst[k] = !INV && r.pack ? key_pack(t) : t;
     } else if constexpr (STORE == ST_RESCALE) {  // forward: out = (x - [x_l]) q_l^-1 with the transformed [x_l] in v
-        const u64 x = r.src3 ? mul_mod(in.a, in.b, P) : in.a;
+        const u64 x = r.src3 ? nttc::product(in.a, in.b, m, P) : in.a;
         r.out2[k] = m.canon(m.mul(x + q - m.canon(v, one_s), words(r.cst2)), one_s);
     } else {
         // out_h = (acc_h - v) P^-1 + add terms (Mod::mul's range and two reduced terms fit 64 bits); with the fused

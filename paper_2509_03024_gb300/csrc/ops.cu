@@ -10,7 +10,7 @@
 #include <algorithm>
 #include <cstring>
 
-#include "core.cuh"
+#include "ntt_core.cuh"
 
 namespace fhe {
 
@@ -217,10 +217,11 @@ __global__ void mul_plain_items_kernel(const BinItem* __restrict__ tab, int item
         const Prime P = pr[x.limb];
         ulonglong2 va = reinterpret_cast<const ulonglong2*>(t.a + o)[x.k2];
         ulonglong2 vb = reinterpret_cast<const ulonglong2*>(t.b + ((size_t)x.limb << log_n))[x.k2];
-        ulonglong2 r;
-        r.x = mul_mod(va.x, vb.x, P);
-        r.y = mul_mod(va.y, vb.y, P);
-        reinterpret_cast<ulonglong2*>(t.out + o)[x.k2] = r;
+        nttc::with_arith(P, [&](auto ar) {
+            const nttc::Mod<decltype(ar)::value> m(P);
+            reinterpret_cast<ulonglong2*>(t.out + o)[x.k2] =
+                make_ulonglong2(nttc::product(va.x, vb.x, m, P), nttc::product(va.y, vb.y, m, P));
+        });
     }
 }
 
@@ -247,19 +248,38 @@ __global__ void mul_const_items_kernel(const ConstItem* __restrict__ tab, int it
     }
 }
 
-__device__ __forceinline__ void tensor_pair(const u64* a, const u64* b, size_t o, size_t pw, int k2,
-                                            const Prime& P, ulonglong2& d0, ulonglong2& d1, ulonglong2& d2) {
-    ulonglong2 a0 = reinterpret_cast<const ulonglong2*>(a + o)[k2];
-    ulonglong2 a1 = reinterpret_cast<const ulonglong2*>(a + pw + o)[k2];
-    ulonglong2 b0 = reinterpret_cast<const ulonglong2*>(b + o)[k2];
-    ulonglong2 b1 = reinterpret_cast<const ulonglong2*>(b + pw + o)[k2];
-    d0.x = mul_mod(a0.x, b0.x, P);
-    d0.y = mul_mod(a0.y, b0.y, P);
-    d1.x = add_mod(mul_mod(a0.x, b1.x, P), mul_mod(a1.x, b0.x, P), P.q);
-    d1.y = add_mod(mul_mod(a0.y, b1.y, P), mul_mod(a1.y, b0.y, P), P.q);
-    d2.x = mul_mod(a1.x, b1.x, P);
-    d2.y = mul_mod(a1.y, b1.y, P);
-}
+// The three components of a (x) b at one slot pair, summed over several a, b before one reduction.
+template <int AR>
+struct TensorSum {
+    nttc::Products<AR> x[3], y[3];
+    __device__ __forceinline__ void add(const u64* a, const u64* b, size_t o, size_t pw, int k2, const Prime& P) {
+        const ulonglong2 a0 = reinterpret_cast<const ulonglong2*>(a + o)[k2];
+        const ulonglong2 a1 = reinterpret_cast<const ulonglong2*>(a + pw + o)[k2];
+        const ulonglong2 b0 = reinterpret_cast<const ulonglong2*>(b + o)[k2];
+        const ulonglong2 b1 = reinterpret_cast<const ulonglong2*>(b + pw + o)[k2];
+        x[0].add(a0.x, b0.x, P);
+        y[0].add(a0.y, b0.y, P);
+        x[1].add(a0.x, b1.x, P);
+        x[1].add(a1.x, b0.x, P);
+        y[1].add(a0.y, b1.y, P);
+        y[1].add(a1.y, b0.y, P);
+        x[2].add(a1.x, b1.x, P);
+        y[2].add(a1.y, b1.y, P);
+    }
+    __device__ __forceinline__ void add_stored(const u64* out, size_t o, size_t pw, int k2, const Prime& P) {
+#pragma unroll
+        for (int i = 0; i < 3; i++) {
+            const ulonglong2 v = reinterpret_cast<const ulonglong2*>(out + i * pw + o)[k2];
+            x[i].add_residue(v.x, P);
+            y[i].add_residue(v.y, P);
+        }
+    }
+    __device__ __forceinline__ void store(u64* out, size_t o, size_t pw, int k2, const nttc::Mod<AR>& m, const Prime& P) const {
+#pragma unroll
+        for (int i = 0; i < 3; i++)
+            reinterpret_cast<ulonglong2*>(out + i * pw + o)[k2] = make_ulonglong2(x[i].reduce(m, P), y[i].reduce(m, P));
+    }
+};
 
 __global__ void tensor_items_kernel(const BinItem* __restrict__ tab, int items, int limbs, int log_n,
                                     size_t pw, const Prime* __restrict__ pr) {
@@ -268,40 +288,36 @@ __global__ void tensor_items_kernel(const BinItem* __restrict__ tab, int items, 
         const BinItem t = tab[it];
         PIdx x = pidx(e, log_n - 1, limbs);
         size_t o = (size_t)x.limb << log_n;
-        const Prime P = pr[x.limb];
-        ulonglong2 d0, d1, d2;
-        tensor_pair(t.a, t.b, o, pw, x.k2, P, d0, d1, d2);
-        reinterpret_cast<ulonglong2*>(t.out + o)[x.k2] = d0;
-        reinterpret_cast<ulonglong2*>(t.out + pw + o)[x.k2] = d1;
-        reinterpret_cast<ulonglong2*>(t.out + 2 * pw + o)[x.k2] = d2;
+        const Prime& P = pr[x.limb];
+        nttc::with_arith(P, [&](auto ar) {
+            constexpr int AR = decltype(ar)::value;
+            TensorSum<AR> s;
+            s.add(t.a, t.b, o, pw, x.k2, P);
+            s.store(t.out, o, pw, x.k2, nttc::Mod<AR>(P), P);
+        });
     }
 }
 
-__global__ void tensor_acc_kernel(const AccTarget* __restrict__ tg, const BinItem* __restrict__ cb, int targets,
+__global__ void __launch_bounds__(kThreads, 2) tensor_acc_kernel(const AccTarget* __restrict__ tg, const BinItem* __restrict__ cb, int targets,
                                   int limbs, int log_n, size_t pw, const Prime* __restrict__ pr) {
     const size_t per = (size_t)limbs << (log_n - 1);
     ITEM_LOOP(targets) {
         const AccTarget t = tg[it];
         PIdx x = pidx(e, log_n - 1, limbs);
         size_t o = (size_t)x.limb << log_n;
-        const Prime P = pr[x.limb];
-        ulonglong2 s0 = reinterpret_cast<const ulonglong2*>(t.out + o)[x.k2];
-        ulonglong2 s1 = reinterpret_cast<const ulonglong2*>(t.out + pw + o)[x.k2];
-        ulonglong2 s2 = reinterpret_cast<const ulonglong2*>(t.out + 2 * pw + o)[x.k2];
-        for (int j = 0; j < t.cnt; j++) {
-            const BinItem c = cb[t.off + j];
-            ulonglong2 d0, d1, d2;
-            tensor_pair(c.a, c.b, o, pw, x.k2, P, d0, d1, d2);
-            s0.x = add_mod(s0.x, d0.x, P.q);
-            s0.y = add_mod(s0.y, d0.y, P.q);
-            s1.x = add_mod(s1.x, d1.x, P.q);
-            s1.y = add_mod(s1.y, d1.y, P.q);
-            s2.x = add_mod(s2.x, d2.x, P.q);
-            s2.y = add_mod(s2.y, d2.y, P.q);
-        }
-        reinterpret_cast<ulonglong2*>(t.out + o)[x.k2] = s0;
-        reinterpret_cast<ulonglong2*>(t.out + pw + o)[x.k2] = s1;
-        reinterpret_cast<ulonglong2*>(t.out + 2 * pw + o)[x.k2] = s2;
+        const Prime& P = pr[x.limb];
+        nttc::with_arith(P, [&](auto ar) {
+            constexpr int AR = decltype(ar)::value;
+            const nttc::Mod<AR> m(P);
+            // two products per contributor enter the middle component, and the stored value counts as one
+            constexpr int kBatch = nttc::Products<AR>::kTerms / 2 - 1;
+            for (int j0 = 0; j0 < t.cnt; j0 += kBatch) {
+                TensorSum<AR> s;
+                s.add_stored(t.out, o, pw, x.k2, P);
+                for (int j = j0; j < min(j0 + kBatch, t.cnt); j++) s.add(cb[t.off + j].a, cb[t.off + j].b, o, pw, x.k2, P);
+                s.store(t.out, o, pw, x.k2, m, P);
+            }
+        });
     }
 }
 
