@@ -863,7 +863,8 @@ CLASS_BOUND = {"ntt_forward": "alu", "ntt_inverse": "alu", "ks_inner": "alu", "t
 # the integer multiply pipe) of one lazy Shoup butterfly on 64-bit residues: the high half of y ws (four
 # partial products), the low halves of y w and of qhat q (one wide and two low products each) = 10; and
 # of one 64 x 64 -> 128-bit multiply-accumulate: four partial products. Additions and carries run on the
-# ALU pipe alongside.
+# ALU pipe alongside. (The transforms of near primes take six wide multiplies, ntt_core.cuh; the count of the
+# general form stays the fixed reference.)
 BFLY_MIN_IMAD = 10
 MAC_MIN_IMAD = 4
 

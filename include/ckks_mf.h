@@ -220,7 +220,7 @@ int fhe_rotate_fanin(fhe_ctx* ctx, uint64_t* acc, int32_t n_groups, const int32_
 /* ------------------------------------------------------------------ launch accounting */
 
 /* Measurement helper (no counterpart in the paper): the rate, in 10^9 butterflies per second,
- * at which this GPU runs the forward NTT's butterfly arithmetic (lazy Shoup Cooley-Tukey
+ * at which this GPU runs the forward NTT's butterfly arithmetic for the first data prime (Cooley-Tukey
  * butterflies, three stages per radix-8 block, a reduction every 15 stages) on values held in
  * registers, with no memory traffic inside the loop. It is the integer-pipe ceiling of the
  * NTT passes. reps: loop trips (each thread does 60 butterflies per trip; ~2000 takes tens of

@@ -993,6 +993,7 @@ void encrypt_coeffs_device(Ctx& c, const i64* m_dev, size_t m_stride, int count,
             CK(cudaGetLastError());
         }
     }
+    CK(cudaStreamSynchronize(s));  // the ciphertexts are complete when the call returns, whatever stream reads them
 }
 
 void decrypt_to_slots(Ctx& c, const u64* ct, int level, double* host_slots, size_t n_slots,

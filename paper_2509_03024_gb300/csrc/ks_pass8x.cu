@@ -1,5 +1,5 @@
 // ks_pass8x.cu — the fused key-switch / rescale transforms with 8 rows or columns per tile and the
-// register cap of LOOSE launch bounds, in a translation unit of their own so that the library builds
+// looser register cap, in a translation unit of their own so that the library builds
 // in parallel (see ks_pass.cuh).
 #include "ks_pass.cuh"
 
