@@ -605,8 +605,9 @@ __device__ __forceinline__ int gaussian_dev(u64 h, u64 k, const GaussTable& T) {
 constexpr u64 kGammaInv = 0xF1DE83E19937733DULL;  // 0x9E3779B97F4A7C15^-1 mod 2^64
 static_assert(kGammaInv * 0x9E3779B97F4A7C15ULL == 1, "inverse of gamma");
 __device__ __forceinline__ int ternary_dev(u64 h, u64 k, u64 z_rej) {
+    // counters start at 1, so a stream key equal to z_rej (counter 0) rejects nothing: 0 - 1 is above every c - 1
     u64 c = k + 1;
-    if (c >= (z_rej - h) * kGammaInv) c++;
+    if (c - 1 >= (z_rej - h) * kGammaInv - 1) c++;
     return (int)(mix64_dev(h + c * 0x9E3779B97F4A7C15ULL) % 3) - 1;
 }
 // m mod q for a signed m; e mod q for a small e

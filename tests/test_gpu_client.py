@@ -65,6 +65,24 @@ def test_encryption_past_a_rejected_ternary_draw(at):
     assert_ct_equal(to_coeff(ctx, ct, 2)[0], he.encrypt(np.ones(3), 2, 9), "encrypt")
 
 
+def test_encryption_with_the_rejected_state_as_stream_key():
+    """The ternary stream of nonce 9 starts in the one state the sampler rejects: counters start at 1, so the
+    stream holds no rejected output and nothing is skipped."""
+    built()
+    h = _unmix64(M64)
+    for f in (0, 0, 9, 6):
+        h = ((_unmix64(h) - GAMMA) & M64) ^ f
+    data, special = (60, 40, 40), (60,)
+    ctx = capi.Context(10, data, special, 40)
+    ctx.keygen(h)
+    he = ckks.Ckks(ckks.Params(10, data, special, 40))
+    he.keygen(h)
+    assert ckks.stream_key(h, 6, 9) == _unmix64(M64)
+    ct = ctx.empty_ct()
+    ctx.encrypt(np.ones(3), 2, 9, ct)
+    assert_ct_equal(to_coeff(ctx, ct, 2)[0], he.encrypt(np.ones(3), 2, 9), "encrypt")
+
+
 @pytest.mark.parametrize("log_n", [9, 11, 14])
 @pytest.mark.parametrize("distinct,count", [(1, 1), (1, 200), (7, 56), (7, 55), (32, 256), (33, 250)])
 def test_encode_few_and_many_distinct_values(log_n, distinct, count):
