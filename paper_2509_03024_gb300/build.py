@@ -8,6 +8,7 @@ tables) is plain IEEE double arithmetic.
 from __future__ import annotations
 
 import concurrent.futures as cf
+import hashlib
 import os
 import shutil
 import subprocess
@@ -35,6 +36,15 @@ def _headers():
     hs = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cuh", ".h"))]
     hs.append(os.path.join(os.path.dirname(HERE), "include", "ckks_mf.h"))
     return hs
+
+
+def kernel_version(csrc: str = CSRC) -> str:
+    """Digest of the CUDA sources: what a timing of the library's kernels was measured on."""
+    h = hashlib.sha256()
+    for name in sorted(f for f in os.listdir(csrc) if f.endswith((".cu", ".cuh"))):
+        with open(os.path.join(csrc, name), "rb") as f:
+            h.update(name.encode() + b"\0" + hashlib.sha256(f.read()).digest())
+    return h.hexdigest()[:16]
 
 
 def _stale(target: str, deps) -> bool:

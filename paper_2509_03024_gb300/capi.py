@@ -14,6 +14,8 @@ from typing import Optional, Sequence
 
 import numpy as np
 
+from paper_2509_03024_gb300 import build
+
 HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(HERE, "_lib", "libckks_mf.so")
 
@@ -69,8 +71,10 @@ class IntPipeRates(ctypes.Structure):
 
 
 def tune_cache_key(device_name: str, n: int, primes: Sequence[int], level: int) -> str:
-    """Key of a stored autotuner choice: the GPU model, and the ring and level it was timed on."""
-    return f"{device_name}|N={n}|q={','.join(str(int(p)) for p in primes)}|level={level}"
+    """Key of a stored autotuner choice: the GPU model, the ring and level it was timed on, and the kernels
+    timed (the variants' names stay when the code behind them changes)."""
+    return (f"{device_name}|N={n}|q={','.join(str(int(p)) for p in primes)}|level={level}"
+            f"|kernels={build.kernel_version()}")
 
 
 def load_tune_cache(path: str) -> dict:
@@ -414,8 +418,8 @@ class Context:
         """Time every launch variant of each tunable kernel family at `level` (default: one below the
         top, the level of an epoch's per-group products) and keep the fastest. Returns
         [{family, variant, chosen, ms}]. With `cache` (a JSON file path), choices are stored under the
-        GPU model and the ring (degree, primes, level), and a later call that finds its key sets the
-        stored choices without timing (records then carry ms None and cached True)."""
+        GPU model, the ring (degree, primes, level) and the kernels' version, and a later call that finds its
+        key sets the stored choices without timing (records then carry ms None and cached True)."""
         level = self.top - 1 if level is None else level
         key = None
         if cache:

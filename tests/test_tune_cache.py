@@ -4,7 +4,7 @@ import json
 
 import pytest
 
-from paper_2509_03024_gb300 import capi
+from paper_2509_03024_gb300 import build, capi
 
 
 def test_keys_separate_device_ring_and_level():
@@ -35,3 +35,18 @@ def test_rejects_a_file_that_is_not_a_cache(tmp_path):
     path.write_text("[1, 2]")
     with pytest.raises(ValueError):
         capi.load_tune_cache(str(path))
+
+
+def test_keys_separate_kernel_versions(tmp_path, monkeypatch):
+    """A choice timed on other kernels is not found again, though ring and variant names are the same."""
+    old = capi.tune_cache_key("GB300", 1 << 15, [97], 6)
+    (tmp_path / "a.cu").write_text("one")
+    (tmp_path / "b.cuh").write_text("two")
+    (tmp_path / "notes.txt").write_text("three")
+    v = build.kernel_version(str(tmp_path))
+    (tmp_path / "notes.txt").write_text("four")
+    assert build.kernel_version(str(tmp_path)) == v
+    (tmp_path / "b.cuh").write_text("five")
+    assert build.kernel_version(str(tmp_path)) != v
+    monkeypatch.setattr(build, "kernel_version", lambda: v)
+    assert capi.tune_cache_key("GB300", 1 << 15, [97], 6) != old
