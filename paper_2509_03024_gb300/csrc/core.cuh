@@ -179,8 +179,9 @@ struct Arena {
     Half halves[2];
     int h = 0;
     // between gather() and upload(s) pushes only stage their data: upload enqueues one copy for all of them
-    // (per block), which must precede the work that reads them
-    bool gathering = false;
+    // (per block), which must precede the work that reads them. Scopes may nest: an inner upload copies what
+    // the outer scope has staged so far along with its own, and the outer scope goes on gathering
+    int gathering = 0;
     size_t from = 0;  // first byte of the current block not yet uploaded
     void reset(cudaStream_t s);
     void* push(const void* data, size_t bytes, cudaStream_t s);
@@ -193,12 +194,18 @@ struct Arena {
     }
     ~Arena();
 };
-// Scope of one gather: an exception between gather() and upload() leaves no half-open state.
+// Scope of one gather, from here to upload(); an exception before it leaves no half-open state.
 struct ArenaGather {
     Arena& a;
+    bool open = true;
     explicit ArenaGather(Arena& arena) : a(arena) { a.gather(); }
-    void upload(cudaStream_t s) { a.upload(s); }
-    ~ArenaGather() { a.gathering = false; }
+    void upload(cudaStream_t s) {
+        open = false;
+        a.upload(s);
+    }
+    ~ArenaGather() {
+        if (open) a.gathering--;
+    }
 };
 
 // ----------------------------------------------------------------------------- launch accounting
