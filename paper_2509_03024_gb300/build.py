@@ -41,7 +41,7 @@ def _headers():
 def kernel_version(csrc: str = CSRC) -> str:
     """Digest of the CUDA sources: what a timing of the library's kernels was measured on."""
     h = hashlib.sha256()
-    for name in sorted(f for f in os.listdir(csrc) if f.endswith((".cu", ".cuh"))):
+    for name in sorted(f for f in os.listdir(csrc) if f.endswith((".cu", ".cuh", ".h"))):
         with open(os.path.join(csrc, name), "rb") as f:
             h.update(name.encode() + b"\0" + hashlib.sha256(f.read()).digest())
     return h.hexdigest()[:16]

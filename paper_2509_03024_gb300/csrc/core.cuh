@@ -269,6 +269,7 @@ struct DeviceBuf {
 
 struct Ctx {
     int device = 0;
+    int n_sm = 0;    // SMs of the device
     int log_n = 0, n = 0, slots = 0;
     int L = 0;       // top level
     int alpha = 0;   // special primes

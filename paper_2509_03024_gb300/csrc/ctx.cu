@@ -1229,6 +1229,7 @@ int fhe_ctx_create(const fhe_params* p, fhe_ctx** out) {
         if (p->log_scale < 1 || p->log_scale > 60) fail(FHE_ERR_INVALID_ARG, "bad log_scale");
         c.device = p->device;
         CK(cudaSetDevice(c.device));
+        CK(cudaDeviceGetAttribute(&c.n_sm, cudaDevAttrMultiProcessorCount, c.device));
         c.log_n = p->log_n;
         c.n = 1 << p->log_n;
         c.slots = c.n / 2;

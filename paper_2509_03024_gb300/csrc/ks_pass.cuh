@@ -3,9 +3,8 @@
 // last pass of a transform, the pass kernel and its launchers. See ks.cu for the algorithm.
 #pragma once
 
-#include <algorithm>
-
 #include "ks_inner.cuh"
+#include "launch_rules.h"
 #include "ntt_core.cuh"
 
 namespace fhe {
@@ -420,9 +419,7 @@ void launch_pass(const Ctx& c, const ROWS& rows, int n_rows, const CombineArgs& 
     const ulonglong2* tw = PASS == 1 && RB == 4 ? (INV ? c.d_itw2 : c.d_tw2) : (INV ? c.d_itw : c.d_tw);
     auto kernel = pass_kernel<ROWS, LOGN, LOGM, R, INV, PASS, LOAD, STORE, RB, MINB>;
     if (smem > 48 * 1024) CK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    // a row pass takes several rows per CTA while at least eight waves of CTAs remain
-    int per_cta = 1;
-    if (PASS == 1) per_cta = (int)std::min<long long>(4, std::max<long long>(1, (long long)n_rows * tiles / (152 * MINB * 8)));
+    const int per_cta = PASS == 1 ? rules::rows_per_cta(c.n_sm, MINB, n_rows, tiles) : 1;
     LaunchScope _ls(c.prof, cls, bytes, s, (double)n_rows * ((size_t)1 << (c.log_n - 1)) * LOGM);
     kernel<<<dim3((n_rows + per_cta - 1) / per_cta, tiles), threads, smem, s>>>(rows, n_rows, per_cta, c.d_primes, tw,
                                                                              c.d_ninv, ca);
@@ -503,12 +500,6 @@ template <bool INV, int LOAD, int STORE>
 void ks_transform_r8x(const Ctx& c, const KsRow* rows, int n_rows, const CombineArgs& ca, int cls, double bytes,
                       cudaStream_t s);
 
-// Launches of few rows leave an SM with a handful of warps, each a serial chain of 16-residue register
-// blocks; with 8 residues per thread (ks_pass_few.cu, 16 rows or columns per tile) the chain is half as long and
-// the warps twice as many. The line: less than 16 warps per SM at 16 residues per thread. One rotation at N = 2^16 with
-// it and with one table upload per key switch 214 -> 170 us, one product at N = 2^13 111 -> 72 us.
-inline bool few_rows(const Ctx& c, int n_rows) { return ((size_t)n_rows << (c.log_n - 4)) < (size_t)152 * 512; }
-
 // A full forward (INV = false) or inverse transform over a row table with the context's tile shape:
 // the first pass applies LOAD, the last pass applies STORE (single-pass rings do both in one kernel).
 template <bool INV, int LOAD, int STORE>
@@ -516,7 +507,7 @@ void ks_transform(const Ctx& c, const KsRow* rows, int n_rows, const CombineArgs
                   cudaStream_t s) {
     // (the rings below 2^14 are not tuned: small tiles, for the CTAs)
     if (c.log_n < 12) ks_transform_r16<INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s);
-    else if (few_rows(c, n_rows)) ks_transform_few<INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s);
+    else if (rules::few_rows(c.n_sm, c.log_n, n_rows)) ks_transform_few<INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s);
     else if (c.log_n < 14 || c.tune.ks == KS_R8) ks_transform_r8<INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s);
     else if (c.tune.ks == KS_R8X) ks_transform_r8x<INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s);
     else ks_transform_r16<INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s);

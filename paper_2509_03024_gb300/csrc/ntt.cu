@@ -26,7 +26,7 @@ using namespace ntt_tile;
 template <bool INV>
 void run_ntt(const Ctx& c, const PolyBatch& pb, cudaStream_t s) {
     const double bytes = 16.0 * pb.rows() * ((size_t)1 << c.log_n);
-    switch (c.log_n < 12 ? NTT_R16B4 : ksp::few_rows(c, pb.rows()) ? NTT_R16B3 : c.log_n < 14 ? NTT_R8B4 : c.tune.ntt) {
+    switch (c.log_n < 12 ? NTT_R16B4 : rules::few_rows(c.n_sm, c.log_n, pb.rows()) ? NTT_R16B3 : c.log_n < 14 ? NTT_R8B4 : c.tune.ntt) {
         case NTT_R8B4: transform_r8b4(c, pb, INV, s, bytes); return;
         case NTT_R32B4: transform_r32b4(c, pb, INV, s, bytes); return;
         case NTT_R16B3: transform_r16b3(c, pb, INV, s, bytes); return;
