@@ -3,6 +3,8 @@
 // last pass of a transform, the pass kernel and its launchers. See ks.cu for the algorithm.
 #pragma once
 
+#include <type_traits>
+
 #include "ks_inner.cuh"
 #include "launch_rules.h"
 #include "ntt_core.cuh"
@@ -238,7 +240,7 @@ struct RowBatch {
     }
 };
 
-// Whole transform of one row per CTA (rings up to 2^11).
+// Whole transform of one row per CTA (rings up to 2^12, see rules::single_pass).
 template <class ROWS, int LOGN, bool INV, int LOAD, int STORE>
 __global__ void __launch_bounds__((1 << LOGN) / 8, 1024 / ((1 << LOGN) / 8))
 single_pass_kernel(ROWS rows, const Prime* __restrict__ primes, const ulonglong2* __restrict__ tw,
@@ -437,35 +439,49 @@ void launch_single(const Ctx& c, const ROWS& rows, int n_rows, const CombineArgs
 }
 
 // A full forward (INV = false) or inverse transform over the rows: the first pass applies LOAD, the
-// last pass applies STORE (rings up to 2^11 do both in one kernel). The column passes of a ring of 2^15
-// have 2^7 points, its row passes 2^8. Rings of 2^12 and 2^13 in two passes: a row spreads over several SMs
-// and the kernels are the register-direct ones (two polynomials of three limbs at 2^13, forward and inverse with
-// their copies: 51 -> 35 us). TPS: threads per SM the register cap of the kernels leaves room for.
+// last pass applies STORE (single-pass rings do both in one kernel). The column passes of a ring of 2^15
+// have 2^7 points, its row passes 2^8. Rings of 2^13 in two passes: a row spreads over several SMs and the
+// kernels are the register-direct ones. The shapes R = 16 with RB = 4 hold the single-pass kernels; rings of 2^12
+// and 2^13 are otherwise transformed by the small tiles only. TPS: threads per SM the register cap of the
+// kernels leaves room for.
 template <class ROWS, bool INV, int LOAD, int STORE, int R, int RB, int TPS>
 void transform_t(const Ctx& c, const ROWS& rows, int n_rows, const CombineArgs& ca, int cls, double bytes, cudaStream_t s) {
     if (n_rows == 0) return;
-    if constexpr (R == 16 && RB == 4) {  // single-pass rings: one shape, instantiated with the first one
+    constexpr bool single = R == 16 && RB == 4, small = R == 8 || RB == 3, plain = std::is_same<ROWS, RowBatch>::value;
+#define ONE(LG)                                                                                    \
+    case LG:                                                                                       \
+        if constexpr (single) {                                                                    \
+            launch_single<ROWS, LG, INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s);         \
+            return;                                                                                \
+        }                                                                                          \
+        break;
+#define TWO(LG, LC, BUILT)                                                                                       \
+    case LG:                                                                                                     \
+        if constexpr (BUILT) {                                                                                   \
+            launch_pass<ROWS, LG, INV ? LG - LC : LC, R, INV, INV ? 1 : 0, LOAD, ST_LAZY, RB, TPS>(c, rows, n_rows, ca, cls, bytes, s); \
+            launch_pass<ROWS, LG, INV ? LC : LG - LC, R, INV, INV ? 0 : 1, LD_PLAIN, STORE, RB, TPS>(c, rows, n_rows, ca, cls, bytes, s); \
+            return;                                                                                              \
+        }                                                                                                        \
+        break;
+    if (rules::single_pass(c.n_sm, c.log_n, !plain, INV, n_rows)) {
         switch (c.log_n) {
-            case 9: launch_single<ROWS, 9, INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s); return;
-            case 10: launch_single<ROWS, 10, INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s); return;
-            case 11: launch_single<ROWS, 11, INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s); return;
-            default: break;
+            ONE(9)
+            ONE(10)
+            ONE(11)
+            ONE(12)
+        }
+    } else {
+        switch (c.log_n) {
+            TWO(12, 6, small && plain)
+            TWO(13, 6, small)
+            TWO(14, 7, true)
+            TWO(15, 7, true)
+            TWO(16, 8, true)
         }
     }
-#define TWO(LG, LC)                                                                                              \
-    case LG:                                                                                                     \
-        launch_pass<ROWS, LG, INV ? LG - LC : LC, R, INV, INV ? 1 : 0, LOAD, ST_LAZY, RB, TPS>(c, rows, n_rows, ca, cls, bytes, s); \
-        launch_pass<ROWS, LG, INV ? LC : LG - LC, R, INV, INV ? 0 : 1, LD_PLAIN, STORE, RB, TPS>(c, rows, n_rows, ca, cls, bytes, s); \
-        return;
-    switch (c.log_n) {
-        TWO(12, 6)
-        TWO(13, 6)
-        TWO(14, 7)
-        TWO(15, 7)
-        TWO(16, 8)
-        default: fail(FHE_ERR_INVALID_ARG, "unsupported ring degree");
-    }
+#undef ONE
 #undef TWO
+    fail(FHE_ERR_INVALID_ARG, "no transform of this ring in this shape");
 }
 
 // The tile shapes of the fused passes the autotuner chooses between (family "ks_pass"): rows or
@@ -505,8 +521,8 @@ void ks_transform_r8x(const Ctx& c, const KsRow* rows, int n_rows, const Combine
 template <bool INV, int LOAD, int STORE>
 void ks_transform(const Ctx& c, const KsRow* rows, int n_rows, const CombineArgs& ca, int cls, double bytes,
                   cudaStream_t s) {
-    // (the rings below 2^14 are not tuned: small tiles, for the CTAs)
-    if (c.log_n < 12) ks_transform_r16<INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s);
+    // (rings below 2^14 are not tuned: 2^13 takes the small tiles, for the CTAs)
+    if (rules::single_pass(c.n_sm, c.log_n, true, INV, n_rows)) ks_transform_r16<INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s);
     else if (rules::few_rows(c.n_sm, c.log_n, n_rows)) ks_transform_few<INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s);
     else if (c.log_n < 14 || c.tune.ks == KS_R8) ks_transform_r8<INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s);
     else if (c.tune.ks == KS_R8X) ks_transform_r8x<INV, LOAD, STORE>(c, rows, n_rows, ca, cls, bytes, s);

@@ -8,8 +8,8 @@
 // N2: the first log2(N1) stages couple elements N2 apart (independent
 // N1-point transforms on columns), the remaining stages couple elements inside
 // one row (N2-point transforms with row-dependent twiddles). Rings up to 2^11
-// run in one pass (one CTA per limb); larger rings in two passes, one kernel
-// each (pass_kernel in ks_pass.cuh). Values stay unreduced between stages
+// run in one pass (one CTA per limb), rings from 2^13 on in two passes, one kernel each
+// (pass_kernel in ks_pass.cuh), 2^12 in either (rules::single_pass). Values stay unreduced between stages
 // wherever 64 bits allow it (ntt_core.cuh); the last pass reduces to [0, q).
 #include "ntt_tile.cuh"
 
@@ -26,7 +26,11 @@ using namespace ntt_tile;
 template <bool INV>
 void run_ntt(const Ctx& c, const PolyBatch& pb, cudaStream_t s) {
     const double bytes = 16.0 * pb.rows() * ((size_t)1 << c.log_n);
-    switch (c.log_n < 12 ? NTT_R16B4 : rules::few_rows(c.n_sm, c.log_n, pb.rows()) ? NTT_R16B3 : c.log_n < 14 ? NTT_R8B4 : c.tune.ntt) {
+    const int shape = rules::single_pass(c.n_sm, c.log_n, false, INV, pb.rows()) ? NTT_R16B4
+                      : rules::few_rows(c.n_sm, c.log_n, pb.rows())              ? NTT_R16B3
+                      : c.log_n < 14                                            ? NTT_R8B4
+                                                                                : c.tune.ntt;
+    switch (shape) {
         case NTT_R8B4: transform_r8b4(c, pb, INV, s, bytes); return;
         case NTT_R32B4: transform_r32b4(c, pb, INV, s, bytes); return;
         case NTT_R16B3: transform_r16b3(c, pb, INV, s, bytes); return;
