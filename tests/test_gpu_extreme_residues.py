@@ -11,7 +11,9 @@ from tests.gpu_common import assert_ct_equal, built, ct_slice, to_coeff, torch
 
 pytestmark = pytest.mark.gpu
 
-DATA, SPECIAL, SCALE = (50, 60, 61, 45), (60, 61), 40
+RINGS = {"mixed": ((50, 60, 61, 45), (60, 61)), "unreduced57": ((57, 57, 58, 57), (57, 57))}
+SCALE = 40
+rings = pytest.mark.parametrize("ring", sorted(RINGS))
 
 
 def _line(ctx):
@@ -36,10 +38,11 @@ def _patterns(ctx, polys):
     return torch.from_numpy(a.view(np.int64).reshape(-1)).cuda()
 
 
+@rings
 @pytest.mark.parametrize("log_n", [14, 15, 16])
-def test_plain_tile_shapes(log_n):
+def test_plain_tile_shapes(log_n, ring):
     built()
-    ctx = capi.Context(log_n, DATA, SPECIAL, SCALE)
+    ctx = capi.Context(log_n, *RINGS[ring], SCALE)
     limbs = ctx.top + 1
     polys = -(-_line(ctx) // limbs) + 7
     w = limbs * ctx.n
@@ -65,10 +68,11 @@ def test_plain_tile_shapes(log_n):
         assert torch.equal(x, base), v
 
 
+@rings
 @pytest.mark.parametrize("log_n", [14, 15, 16])
-def test_fused_tile_shapes(log_n):
+def test_fused_tile_shapes(log_n, ring):
     built()
-    ctx = capi.Context(log_n, DATA, SPECIAL, SCALE)
+    ctx = capi.Context(log_n, *RINGS[ring], SCALE)
     ctx.keygen(6, [3])
     count, level = -(-_line(ctx) // 2) + 3, ctx.top          # the smallest launch has two rows per ciphertext
     a = _patterns(ctx, 2 * count)
@@ -90,7 +94,7 @@ def test_fused_tile_shapes(log_n):
             for t in picks:
                 assert torch.equal(ct_slice(ctx, out, t), ref[name, t]), (name, v, t)
     if log_n == 14:
-        he = ckks.Ckks(ckks.Params(log_n, DATA, SPECIAL, SCALE))
+        he = ckks.Ckks(ckks.Params(log_n, *RINGS[ring], SCALE))
         he.keygen(6, [3])
         for t in picks[:3]:
             oa, ob = (ckks.Ciphertext(to_coeff(ctx, ct_slice(ctx, x, t), level)[0], level) for x in (a, b))
