@@ -40,7 +40,7 @@ void cuda_check(cudaError_t e, const char* what);
 
 // One RNS prime with its Barrett constant (HAC Alg. 14.42, base 2):
 // mu = floor(2^(2b) / q), b = bit length of q, q < 2^62.
-struct Prime {
+struct alignas(16) Prime {
     u64 q;
     u64 mu;
     u64 one_s;  // floor(2^64 / q): Shoup companion of 1, for lazy reduction of any 64-bit value

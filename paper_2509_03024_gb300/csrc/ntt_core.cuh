@@ -141,6 +141,11 @@ template <int AR>
 struct Products {
     static constexpr int kTerms = 512;
     u64 c0 = 0, c1 = 0, c2 = 0;
+    // the first product (the sum's start, which the Barrett form need not add to)
+    __device__ __forceinline__ void start(u64 a, u64 b, const Prime& P) {
+        if constexpr (AR == AR_NEAR50) add(a, b, P);
+        else c0 = mul_mod(a, b, P);
+    }
     __device__ __forceinline__ void add(u64 a, u64 b, const Prime& P) {
         if constexpr (AR == AR_NEAR50) {
             constexpr u32 m25 = (1u << 25) - 1;
@@ -168,7 +173,7 @@ struct Products {
 template <int AR>
 __device__ __forceinline__ u64 product(u64 a, u64 b, const Mod<AR>& m, const Prime& P) {
     Products<AR> s;
-    s.add(a, b, P);
+    s.start(a, b, P);
     return s.reduce(m, P);
 }
 

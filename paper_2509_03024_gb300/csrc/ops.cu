@@ -133,6 +133,22 @@ __global__ void copy_items_kernel(const UnItem* __restrict__ tab, int items, int
     }
 }
 
+// Products of two residues modulo near 50-bit primes go to column sums (Products in ntt_core.cuh); N50 = false is
+// the kernel of launches whose primes are all others. With the column sums' code beside it the Barrett form needs 80
+// to 128 registers instead of 60 to 78: the tensor of 64 ciphertexts at N = 2^14, four 45-bit limbs, 65 us alone, 69 so;
+// 64 plaintext products 66 and 69.
+template <bool N50, class F>
+__device__ __forceinline__ void with_products(const Prime& P, F&& f) {
+    if (N50 && P.cls == nttc::AR_NEAR50) f(nttc::Tag<nttc::AR_NEAR50>{});
+    else f(nttc::Tag<nttc::AR_SHOUP>{});
+}
+inline bool any_near50(const Ctx& c, int limbs) {
+    for (int i = 0; i < limbs; i++)
+        if (c.hprimes[i].cls == nttc::AR_NEAR50) return true;
+    return false;
+}
+
+template <bool N50>
 __global__ void mul_plain_items_kernel(const BinItem* __restrict__ tab, int items, int parts, int limbs,
                                        int log_n, size_t part_words, const Prime* __restrict__ pr) {
     const size_t per = (size_t)parts * limbs << (log_n - 1);
@@ -143,7 +159,7 @@ __global__ void mul_plain_items_kernel(const BinItem* __restrict__ tab, int item
         const Prime P = pr[x.limb];
         ulonglong2 va = reinterpret_cast<const ulonglong2*>(t.a + o)[x.k2];
         ulonglong2 vb = reinterpret_cast<const ulonglong2*>(t.b + ((size_t)x.limb << log_n))[x.k2];
-        nttc::with_arith(P, [&](auto ar) {
+        with_products<N50>(P, [&](auto ar) {
             const nttc::Mod<decltype(ar)::value> m(P);
             reinterpret_cast<ulonglong2*>(t.out + o)[x.k2] =
                 make_ulonglong2(nttc::product(va.x, vb.x, m, P), nttc::product(va.y, vb.y, m, P));
@@ -178,19 +194,25 @@ __global__ void mul_const_items_kernel(const ConstItem* __restrict__ tab, int it
 template <int AR>
 struct TensorSum {
     nttc::Products<AR> x[3], y[3];
+    template <bool START>
+    __device__ __forceinline__ static void enter(nttc::Products<AR>& s, u64 a, u64 b, const Prime& P) {
+        if (START) s.start(a, b, P);
+        else s.add(a, b, P);
+    }
+    template <bool START>
     __device__ __forceinline__ void add(const u64* a, const u64* b, size_t o, size_t pw, int k2, const Prime& P) {
         const ulonglong2 a0 = reinterpret_cast<const ulonglong2*>(a + o)[k2];
         const ulonglong2 a1 = reinterpret_cast<const ulonglong2*>(a + pw + o)[k2];
         const ulonglong2 b0 = reinterpret_cast<const ulonglong2*>(b + o)[k2];
         const ulonglong2 b1 = reinterpret_cast<const ulonglong2*>(b + pw + o)[k2];
-        x[0].add(a0.x, b0.x, P);
-        y[0].add(a0.y, b0.y, P);
-        x[1].add(a0.x, b1.x, P);
+        enter<START>(x[0], a0.x, b0.x, P);
+        enter<START>(y[0], a0.y, b0.y, P);
+        enter<START>(x[1], a0.x, b1.x, P);
         x[1].add(a1.x, b0.x, P);
-        y[1].add(a0.y, b1.y, P);
+        enter<START>(y[1], a0.y, b1.y, P);
         y[1].add(a1.y, b0.y, P);
-        x[2].add(a1.x, b1.x, P);
-        y[2].add(a1.y, b1.y, P);
+        enter<START>(x[2], a1.x, b1.x, P);
+        enter<START>(y[2], a1.y, b1.y, P);
     }
     __device__ __forceinline__ void add_stored(const u64* out, size_t o, size_t pw, int k2, const Prime& P) {
 #pragma unroll
@@ -207,6 +229,7 @@ struct TensorSum {
     }
 };
 
+template <bool N50>
 __global__ void tensor_items_kernel(const BinItem* __restrict__ tab, int items, int limbs, int log_n,
                                     size_t pw, const Prime* __restrict__ pr) {
     const size_t per = (size_t)limbs << (log_n - 1);
@@ -214,17 +237,18 @@ __global__ void tensor_items_kernel(const BinItem* __restrict__ tab, int items, 
         const BinItem t = tab[it];
         PIdx x = pidx(e, log_n - 1, limbs);
         size_t o = (size_t)x.limb << log_n;
-        const Prime& P = pr[x.limb];
-        nttc::with_arith(P, [&](auto ar) {
+        const Prime P = pr[x.limb];
+        with_products<N50>(P, [&](auto ar) {
             constexpr int AR = decltype(ar)::value;
             TensorSum<AR> s;
-            s.add(t.a, t.b, o, pw, x.k2, P);
+            s.template add<true>(t.a, t.b, o, pw, x.k2, P);
             s.store(t.out, o, pw, x.k2, nttc::Mod<AR>(P), P);
         });
     }
 }
 
-__global__ void __launch_bounds__(kThreads, 2) tensor_acc_kernel(const AccTarget* __restrict__ tg, const BinItem* __restrict__ cb, int targets,
+template <bool N50>
+__global__ void __launch_bounds__(kThreads, N50 ? 2 : 3) tensor_acc_kernel(const AccTarget* __restrict__ tg, const BinItem* __restrict__ cb, int targets,
                                   int limbs, int log_n, size_t pw, const Prime* __restrict__ pr) {
     const size_t per = (size_t)limbs << (log_n - 1);
     ITEM_LOOP(targets) {
@@ -232,7 +256,7 @@ __global__ void __launch_bounds__(kThreads, 2) tensor_acc_kernel(const AccTarget
         PIdx x = pidx(e, log_n - 1, limbs);
         size_t o = (size_t)x.limb << log_n;
         const Prime& P = pr[x.limb];
-        nttc::with_arith(P, [&](auto ar) {
+        with_products<N50>(P, [&](auto ar) {
             constexpr int AR = decltype(ar)::value;
             const nttc::Mod<AR> m(P);
             // two products per contributor enter the middle component, and the stored value counts as one
@@ -240,7 +264,7 @@ __global__ void __launch_bounds__(kThreads, 2) tensor_acc_kernel(const AccTarget
             for (int j0 = 0; j0 < t.cnt; j0 += kBatch) {
                 TensorSum<AR> s;
                 s.add_stored(t.out, o, pw, x.k2, P);
-                for (int j = j0; j < min(j0 + kBatch, t.cnt); j++) s.add(cb[t.off + j].a, cb[t.off + j].b, o, pw, x.k2, P);
+                for (int j = j0; j < min(j0 + kBatch, t.cnt); j++) s.template add<false>(cb[t.off + j].a, cb[t.off + j].b, o, pw, x.k2, P);
                 s.store(t.out, o, pw, x.k2, m, P);
             }
         });
@@ -357,7 +381,8 @@ void items_mul_plain(Ctx& c, const std::vector<BinItem>& it, int parts, int limb
     size_t per = (size_t)parts * limbs * c.n / 2;
     {
         LaunchScope _ls(c.prof, K_ELEMENTWISE, 2.5 * 8 * per * 2 * it.size(), s);
-        mul_plain_items_kernel<<<grid2(per, (int)it.size()), kThreads, 0, s>>>(d, (int)it.size(), parts, limbs,
+        auto kernel = any_near50(c, limbs) ? mul_plain_items_kernel<true> : mul_plain_items_kernel<false>;
+        kernel<<<grid2(per, (int)it.size()), kThreads, 0, s>>>(d, (int)it.size(), parts, limbs,
                                                                            c.log_n, (size_t)(c.L + 1) * c.n,
                                                                            c.d_primes);
     CK(cudaGetLastError());
@@ -382,7 +407,8 @@ void items_tensor(Ctx& c, const std::vector<BinItem>& it, int limbs, cudaStream_
     size_t per = (size_t)limbs * c.n / 2;
     {
         LaunchScope _ls(c.prof, K_TENSOR, 7.0 * 8 * per * 2 * it.size(), s);
-        tensor_items_kernel<<<grid2(per, (int)it.size()), kThreads, 0, s>>>(d, (int)it.size(), limbs, c.log_n,
+        auto kernel = any_near50(c, limbs) ? tensor_items_kernel<true> : tensor_items_kernel<false>;
+        kernel<<<grid2(per, (int)it.size()), kThreads, 0, s>>>(d, (int)it.size(), limbs, c.log_n,
                                                                         (size_t)(c.L + 1) * c.n, c.d_primes);
     CK(cudaGetLastError());
     }
@@ -398,7 +424,8 @@ void items_tensor_acc(Ctx& c, const std::vector<AccTarget>& tg, const std::vecto
     size_t per = (size_t)limbs * c.n / 2;
     {
         LaunchScope _ls(c.prof, K_TENSOR, 8.0 * per * 2 * (4.0 * contrib.size() + 6.0 * tg.size()), s);
-        tensor_acc_kernel<<<grid2(per, (int)tg.size()), kThreads, 0, s>>>(dt, dc, (int)tg.size(), limbs, c.log_n,
+        auto kernel = any_near50(c, limbs) ? tensor_acc_kernel<true> : tensor_acc_kernel<false>;
+        kernel<<<grid2(per, (int)tg.size()), kThreads, 0, s>>>(dt, dc, (int)tg.size(), limbs, c.log_n,
                                                                       (size_t)(c.L + 1) * c.n, c.d_primes);
     CK(cudaGetLastError());
     }
