@@ -147,17 +147,24 @@ __device__ __forceinline__ void with_count(int cnt, F&& f) {
     else f(nttc::Tag<0>{});
 }
 
-// Residue k of the row as the transform takes it (LD_CONV: conv_rows): a congruent value, for a forward
-// transform within 2^60.4 (NEAR50, signed), below 16 q (NEAR60) or 8 q (SHOUP); reduced for an inverse one.
+// Residue k of the row as it stands in memory (LD_CONV: conv_rows). The kernels of few or short rows load it before
+// anything of the row's prime is known: behind the branch on the prime's arithmetic the loads wait for the prime,
+// one more trip to L2 in a launch that is a handful of them.
+template <int LOAD>
+__device__ __forceinline__ u64 load_raw(const KsRow& r, size_t k, int log_n) {
+    if constexpr (LOAD == LD_PLAIN) return r.dst[k];
+    else if constexpr (LOAD == LD_GATHER) return r.src[r.galois == 1 ? (int)k : auto_src((int)k, r.galois, log_n)];
+    else return r.src[k];
+}
+// The same as the transform takes it: a congruent value, for a forward transform within 2^60.4 (NEAR50, signed),
+// below 16 q (NEAR60) or 8 q (SHOUP); reduced for an inverse one.
 template <int LOAD, int AR>
-__device__ __forceinline__ u64 load_elem(const KsRow& r, size_t k, int log_n, const Prime& P, const nttc::Mod<AR>& m,
+__device__ __forceinline__ u64 load_elem(const KsRow& r, u64 v, size_t k, const Prime& P, const nttc::Mod<AR>& m,
                                          const RowConst& rc) {
-    if constexpr (LOAD == LD_PLAIN) {
-        return r.dst[k];
-    } else if constexpr (LOAD == LD_GATHER) {
-        return r.src[r.galois == 1 ? (int)k : auto_src((int)k, r.galois, log_n)];
+    if constexpr (LOAD == LD_PLAIN || LOAD == LD_GATHER) {
+        return v;
     } else if constexpr (LOAD == LD_CENTRED) {  // the centred representative of src[k] (mod q_limb)
-        const u64 ql = rc.ql, v = r.src[k];
+        const u64 ql = rc.ql;
         const bool neg = v > (ql >> 1);
         if constexpr (AR == nttc::AR_NEAR50) {
             return neg ? v - ql : v;  // signed, magnitude at most 2^60
@@ -167,10 +174,9 @@ __device__ __forceinline__ u64 load_elem(const KsRow& r, size_t k, int log_n, co
             return neg ? (t ? P.q - t : 0) : t;
         }
     } else if constexpr (LOAD == LD_MUL) {
-        return nttc::product(r.src[k], r.src2[k], m, P);
+        return nttc::product(v, r.src2[k], m, P);
     } else {  // LD_AXPY: src + cst2 * src2
         static_assert(LOAD == LD_AXPY, "load mode");
-        const u64 v = r.src[k];
         return r.src2 ? m.canon(v + m.mul(r.src2[k], words(r.cst2)), P.one_s) : v;
     }
 }
@@ -249,19 +255,24 @@ single_pass_kernel(ROWS rows, const Prime* __restrict__ primes, const ulonglong2
     extern __shared__ u64 sm[];
     const KsRow r = rows.get(blockIdx.x, LOGN);
     const Prime& P = primes[r.prime];
+    const int tid = threadIdx.x;
+    auto at = [&](int u) -> u64& { return sm[tid + u * T]; };
+    auto addr = [&](int u) -> size_t { return tid + u * T; };
+    u64 raw[LOAD == LD_CONV ? 1 : 8];
+    if constexpr (LOAD != LD_CONV) {
+#pragma unroll
+        for (int u = 0; u < 8; u++) raw[u] = load_raw<LOAD>(r, addr(u), LOGN);
+    }
     nttc::with_arith(P, [&](auto ar) {
         constexpr int AR = decltype(ar)::value;
         const nttc::Mod<AR> m(P);
         const RowConst rc = row_const<LOAD>(r, primes);
-        const int tid = threadIdx.x;
-        auto at = [&](int u) -> u64& { return sm[tid + u * T]; };
-        auto addr = [&](int u) -> size_t { return tid + u * T; };
         if constexpr (LOAD == LD_CONV) {
             with_count(r.src_cnt, [&](auto cnt) { conv_rows<AR, decltype(cnt)::value, 8>(r, LOGN, m, rc, addr, at); });
         } else {
             u64 v[8];
 #pragma unroll
-            for (int u = 0; u < 8; u++) v[u] = load_elem<LOAD>(r, addr(u), LOGN, P, m, rc);
+            for (int u = 0; u < 8; u++) v[u] = load_elem<LOAD>(r, raw[u], addr(u), P, m, rc);
 #pragma unroll
             for (int u = 0; u < 8; u++) {
                 at(u) = v[u];
@@ -320,13 +331,19 @@ pass_kernel(ROWS rows, int n_rows, int per_cta, const Prime* __restrict__ primes
         const KsRow r = rows.get(i, LOGN);
         const Prime& P = primes[r.prime];
         const ulonglong2* const W = tw + ((size_t)r.prime << LOGN) + (PASS == 1 && RB == 4 ? (size_t)t0 << LOGM : 0);
+        // register u holds element g + T u before block 0 and outside the blocks of a row pass (arrangement
+        // -1), block_elem(k, g, u) in block k
+        auto elem = [&](int blk, int u) { return blk < 0 ? g + T * u : nttc::block_elem<LOGM, RB>(blk, g, u); };
+        auto load_addr = [&](int u) { return addr(INV && PASS == 0 ? elem(NB - 1, u) : g + T * u); };
+        u64 v[V];
+        constexpr bool early = LOAD != LD_CONV && RB == 3;  // (16 residues a thread: spills instead)
+        if constexpr (early) {
+#pragma unroll
+            for (int u = 0; u < V; u++) v[u] = load_raw<LOAD>(r, load_addr(u), LOGN);
+        }
         nttc::with_arith(P, [&](auto ar) {
             constexpr int AR = decltype(ar)::value;
             const nttc::Mod<AR> m(P);
-            u64 v[V];
-            // register u holds element g + T u before block 0 and outside the blocks of a row pass (arrangement
-            // -1), block_elem(k, g, u) in block k
-            auto elem = [&](int blk, int u) { return blk < 0 ? g + T * u : nttc::block_elem<LOGM, RB>(blk, g, u); };
             auto put = [&](int blk) {
 #pragma unroll
                 for (int u = 0; u < V; u++) at(elem(blk, u)) = v[u];
@@ -363,7 +380,7 @@ pass_kernel(ROWS rows, int n_rows, int per_cta, const Prime* __restrict__ primes
             } else {
 #pragma unroll
                 for (int u = 0; u < V; u++)
-                    v[u] = load_elem<LOAD>(r, addr(INV && PASS == 0 ? elem(NB - 1, u) : g + T * u), LOGN, P, m, rc);
+                    v[u] = load_elem<LOAD>(r, early ? v[u] : load_raw<LOAD>(r, load_addr(u), LOGN), load_addr(u), P, m, rc);
                 if (LOAD == LD_GATHER && r.out2) {
 #pragma unroll
                     for (int u = 0; u < V; u++) r.out2[addr(g + T * u)] = r.pack ? key_pack(v[u]) : v[u];
