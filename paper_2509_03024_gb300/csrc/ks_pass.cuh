@@ -464,6 +464,10 @@ void launch_single(const Ctx& c, const ROWS& rows, int n_rows, const CombineArgs
 template <class ROWS, bool INV, int LOAD, int STORE, int R, int RB, int TPS>
 void transform_t(const Ctx& c, const ROWS& rows, int n_rows, const CombineArgs& ca, int cls, double bytes, cudaStream_t s) {
     if (n_rows == 0) return;
+    // rows or columns per tile: with 8 residues per thread, 256-point sub-transforms take half as many, so that no CTA
+    // has more than 256 threads. The ten rows of a rescale at N = 2^16 were 160 CTAs of 512 threads on 152 SMs: one
+    // ciphertext, five 45-bit limbs left, 50.2 us, by rescale_noalloc 55.6; with 320 CTAs of half the size 40.6 and 45.4
+    constexpr auto tile = [](int log_m) { return RB == 3 && log_m == 8 ? R / 2 : R; };
     constexpr bool single = R == 16 && RB == 4, small = R == 8 || RB == 3, plain = std::is_same<ROWS, RowBatch>::value;
 #define ONE(LG)                                                                                    \
     case LG:                                                                                       \
@@ -475,8 +479,9 @@ void transform_t(const Ctx& c, const ROWS& rows, int n_rows, const CombineArgs& 
 #define TWO(LG, LC, BUILT)                                                                                       \
     case LG:                                                                                                     \
         if constexpr (BUILT) {                                                                                   \
-            launch_pass<ROWS, LG, INV ? LG - LC : LC, R, INV, INV ? 1 : 0, LOAD, ST_LAZY, RB, TPS>(c, rows, n_rows, ca, cls, bytes, s); \
-            launch_pass<ROWS, LG, INV ? LC : LG - LC, R, INV, INV ? 0 : 1, LD_PLAIN, STORE, RB, TPS>(c, rows, n_rows, ca, cls, bytes, s); \
+            constexpr int first = INV ? LG - LC : LC, last = LG - first;                                         \
+            launch_pass<ROWS, LG, first, tile(first), INV, INV ? 1 : 0, LOAD, ST_LAZY, RB, TPS>(c, rows, n_rows, ca, cls, bytes, s); \
+            launch_pass<ROWS, LG, last, tile(last), INV, INV ? 0 : 1, LD_PLAIN, STORE, RB, TPS>(c, rows, n_rows, ca, cls, bytes, s); \
             return;                                                                                              \
         }                                                                                                        \
         break;

@@ -24,7 +24,7 @@ inline bool single_pass(int n_sm, int log_n, bool fused, bool inverse, size_t n_
 }
 
 // Launches of few rows leave an SM with a handful of warps, each a serial chain of 16-residue register
-// blocks; with 8 residues per thread (ks_pass_few.cu, 16 rows or columns per tile) the chain is half as long and
+// blocks; with 8 residues per thread (ks_pass_few.cu, 16 rows or columns per tile, 8 of 256 points) the chain is half as long and
 // the warps twice as many. The line: less than 16 warps per SM at 16 residues per thread. One rotation at N = 2^16 with
 // it and with one table upload per key switch 214 -> 170 us, one product at N = 2^13 111 -> 72 us.
 inline bool few_rows(int n_sm, int log_n, size_t n_rows) { return (n_rows << (log_n - 4)) < (size_t)n_sm * 512; }
