@@ -846,10 +846,17 @@ void encode_many_device(Ctx& c, const std::vector<int>& idx, const std::vector<d
     }
     CK(cudaMemcpyAsync(d_off, offsets.data(), sizeof(int) * offsets.size(), cudaMemcpyHostToDevice, s));
     const double factor = std::ldexp(1.0, c.log_scale + 1 - c.log_n);  // 2 Delta / N
-    // few distinct values over many terms: tabulate their products, when that is an eighth of the terms' work
+    // Few distinct values over many terms: tabulate their products. That costs two more copies, a launch and 2N products
+    // per value, about 7 us and 0.3 per value; it saves 0.125 us a term at N = 2^16, 0.0625 at 2^15 and 0.036 on rings
+    // up to 2^14, whose terms wait for latency. us with : without it, N = 2^15: 60 terms of one value 31 : 29, 128 of one
+    // 38 : 40, 128 of 16 43 : 39, 256 of 16 56 : 61; 2^13: 60 of one 29 : 26, 256 of 16 48 : 44, 512 of 16 65 : 69; 2^12:
+    // 256 of one 41 : 43, 512 of 16 60 : 68; 2^16: 60 of one 34 : 36, 128 of 16 50 : 55.
+    const auto worth = [&](size_t values) {
+        return nz * std::max<size_t>(c.n, 18 << 10) >= ((size_t)7 << 19) + values * ((size_t)5 << 15);
+    };
     std::vector<double> distinct;
     std::vector<int> which;
-    bool pre = nz >= 8;
+    bool pre = worth(1);
     if (pre) {
         which.resize(nz);
         int last = -1;
@@ -859,7 +866,7 @@ void encode_many_device(Ctx& c, const std::vector<int>& idx, const std::vector<d
                     if (std::memcmp(&distinct[last], &val[t], sizeof(double)) == 0) break;
                 if (last == (int)distinct.size()) {
                     distinct.push_back(val[t]);
-                    pre = (int)distinct.size() <= kEncDistinct && distinct.size() * 8 <= nz;
+                    pre = (int)distinct.size() <= kEncDistinct && distinct.size() * 8 <= nz && worth(distinct.size());
                 }
             }
             which[t] = last;

@@ -99,3 +99,23 @@ def test_encode_few_and_many_distinct_values(log_n, distinct, count):
     out = torch.zeros(ctx.n, dtype=torch.int64, device="cuda")
     ctx.encode(z, out)
     assert np.array_equal(out.cpu().numpy(), he.enc.encode(z))
+
+
+@pytest.mark.parametrize("log_n,distinct,count,tabulated", [
+    (9, 1, 256, True), (10, 1, 207, False), (10, 1, 208, True), (10, 5, 512, True), (12, 5, 243, False), (12, 5,
+    244, True), (12, 16, 340, False), (12, 16, 342, True), (13, 1, 60, False), (14, 32, 512, True), (15, 1, 116,
+    False), (15, 1, 117, True), (15, 16, 128, False), (15, 16, 192, True), (16, 1, 58, False), (16, 1, 59, True),
+    (16, 33, 600, False)])
+def test_products_are_tabulated_where_it_pays(log_n, distinct, count, tabulated):
+    """Both sides of the rule's line: the launches it chooses, and the oracle's integers."""
+    built()
+    ctx = capi.Context(log_n, (60, 40), (60,), 40)
+    he = ckks.Ckks(ckks.Params(log_n, (60, 40), (60,), 40))
+    rng = np.random.default_rng(count)
+    z = np.zeros(ctx.slots)
+    z[np.sort(rng.choice(ctx.slots, count, replace=False))] = rng.normal(0, 3, distinct)[np.arange(count) % distinct]
+    out = torch.zeros(ctx.n, dtype=torch.int64, device="cuda")
+    ctx.profile_begin()
+    ctx.encode(z, out)
+    assert ctx.profile_end()["encode"][0] == (2 if tabulated else 1)
+    assert np.array_equal(out.cpu().numpy(), he.enc.encode(z))
