@@ -312,6 +312,7 @@ struct Ctx {
     double* d_cos_t = nullptr;        // [N/32][64] the same for the encoding, entry e at [e mod N/32][e / (N/32)]
     double* d_sin = nullptr;          // [2N] sin(pi e / N)
     u32* d_pow5 = nullptr;            // [N/2] 5^t mod 2N
+    u32* d_slot_of = nullptr;         // [N/2] the slot t with 5^t = 4 k + 1 mod 2N, entry k
 
     // keys
     bool have_keys = false;

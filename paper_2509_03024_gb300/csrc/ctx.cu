@@ -70,7 +70,7 @@ Ctx::~Ctx() {
     cudaSetDevice(device);
     cudaDeviceSynchronize();
     void* bufs[] = {d_primes, d_ninv, d_tw, d_itw, d_tw2, d_itw2, d_up_ninv, d_down_ninv, d_resc, d_resc_w, d_up_hat,
-                    d_down_hat, d_pinv, d_pmod, d_fd_ninv, d_fd_hat, d_fd_minv, d_fd_pq, d_cos, d_cos_t, d_sin, d_pow5, d_sk, d_pk, rlk.d};
+                    d_down_hat, d_pinv, d_pmod, d_fd_ninv, d_fd_hat, d_fd_minv, d_fd_pq, d_cos, d_cos_t, d_sin, d_pow5, d_slot_of, d_sk, d_pk, rlk.d};
     for (void* p : bufs)
         if (p) cudaFree(p);
     for (auto& kv : rot)
@@ -462,13 +462,15 @@ static void build_tables(Ctx& c) {
     for (int e = 0; e < 2 * n; e++) cs_t[(size_t)(e % (n / 32)) * 64 + e / (n / 32)] = cs[e];
     c.d_cos_t = dupload(cs_t);
     c.d_sin = dupload(sn);
-    std::vector<u32> p5(c.slots);
+    std::vector<u32> p5(c.slots), slot_of(c.slots);
     u64 x = 1;
     for (int t = 0; t < c.slots; t++) {
         p5[t] = (u32)x;
+        slot_of[(x - 1) >> 2] = (u32)t;
         x = x * 5 % (2 * (u64)n);
     }
     c.d_pow5 = dupload(p5);
+    c.d_slot_of = dupload(slot_of);
 }
 
 // ============================================================================ kernels local to this file
@@ -724,14 +726,12 @@ __global__ void dec_kernel(u64* m, const u64* __restrict__ ct, size_t part_strid
 
 // The integer coefficient of residues x0 mod q0 (nl = 1) or x0, x1 mod q0, q1 (nl = 2), centred, as a double.
 struct Lift {
-    u64 q0, q1, q0inv;  // q0inv: q0^-1 mod q1
+    u64 q0, q1, one1, q0inv, q0inv_s;  // q0inv: q0^-1 mod q1; one1, q0inv_s: Shoup companions of 1 and q0inv
     int nl;
 };
 __device__ __forceinline__ double centred_lift(u64 x0, u64 x1, const Lift& l) {
     if (l.nl == 1) return x0 > l.q0 / 2 ? -(double)(l.q0 - x0) : (double)x0;
-    const u64 r = x0 % l.q1;
-    const u64 d = x1 >= r ? x1 - r : x1 + l.q1 - r;
-    const u64 k = (u64)(((u128)d * l.q0inv) % l.q1);
+    const u64 k = mul_shoup(sub_mod(x1, nttc::reduce_any(x0, l.q1, l.one1), l.q1), l.q0inv, l.q0inv_s, l.q1);
     const u128 v = (u128)k * l.q0 + x0, Q = (u128)l.q0 * l.q1;
     return v > Q / 2 ? -(double)(Q - v) : (double)v;
 }
@@ -764,9 +764,35 @@ __global__ void crt_int64_kernel(i64* out, const u64* __restrict__ m, int nl, in
 
 // Decoding: z_t = Re m(zeta^(5^t)) / Delta with zeta = exp(i pi / N). 5^t = 4 k + 1, and zeta^(N/2 (4k+1)) = i,
 // so m(zeta^(4k+1)) = sum_{j < n} (m_j + i m_(j+n)) zeta^j exp(2 pi i j k / n) for n = N/2: one complex
-// transform of n points gives every slot, where a sum of N terms per slot read N scattered cosines each
+// transform of n points gives every slot, where a sum of N terms per slot reads N scattered cosines each
 // (6.9 ms for the 2^15 slots of N = 2^16, one ciphertext). Four-step form n = n1 n2, one small transform
-// per CTA; j = j1 n2 + j2, k = k1 + n1 k2.
+// per CTA; j = j1 n2 + j2, k = k1 + n1 k2. Rings up to 2^11 take the direct sums, because the transform's stages wait
+// for their table entries one after another. Decryption of two limbs, us for one slot : all of them, direct against
+// transform: N = 2^9 35.6 : 35.7 against 37.8 : 38.2, 2^10 34.9 : 37.6 against 38.7 : 39.1, 2^11 35.9 : 50.0 against
+// 39.7 : 41.2, 2^12 37.8 : 64.4 against 41.6 : 43.0. The rule is the ring's alone, so that every prefix of the slots
+// has the same bits.
+inline bool decode_direct(int log_n) { return log_n <= 11; }
+
+__global__ void lift_kernel(double* out, const u64* __restrict__ m, Lift lift, int log_n) {
+    const int n = 1 << log_n, j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j < n) out[j] = centred_lift(m[j], lift.nl == 2 ? m[n + j] : 0, lift);
+}
+
+// Slot t = blockIdx.x: kT strided partial sums of m_j cos(pi (j 5^t mod 2N) / N), added in a tree.
+__global__ void __launch_bounds__(kT) decode_sums(double* z, const double* __restrict__ m, const double* __restrict__ cs,
+                                                  const u32* __restrict__ pow5, int log_n, double inv_scale) {
+    __shared__ double part[kT];
+    const u32 mask = (2u << log_n) - 1, p = pow5[blockIdx.x];
+    double acc = 0.0;
+    for (int j = threadIdx.x; j < 1 << log_n; j += kT) acc += m[j] * cs[(u32)j * p & mask];
+    part[threadIdx.x] = acc;
+    __syncthreads();
+    for (int h = kT / 2; h; h >>= 1) {
+        if (threadIdx.x < h) part[threadIdx.x] += part[threadIdx.x + h];
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) z[blockIdx.x] = part[0] * inv_scale;
+}
 
 // In-place decimation-in-frequency transform of M = blockDim.x * 2 points in shared memory; entry i holds
 // output brev(i) after it. tab_step: 2N / M, the table step of exp(2 pi i / M).
@@ -803,22 +829,18 @@ __global__ void decode_columns(double2* y, const u64* __restrict__ m, Lift lift,
     }
 }
 
-// Rows k1 (blockIdx.x): n2-point transform over j2, the real parts of outputs k1 + n1 k2.
-__global__ void decode_rows(double* re, const double2* __restrict__ y, int log_n, int log_n1, const double* __restrict__ cs,
-                            const double* __restrict__ sn) {
+// Rows k1 (blockIdx.x): n2-point transform over j2; the real part of output k = k1 + n1 k2 is slot slot_of[k].
+__global__ void decode_rows(double* z, const double2* __restrict__ y, int log_n, int log_n1, const double* __restrict__ cs,
+                            const double* __restrict__ sn, const u32* __restrict__ slot_of, double inv_scale, int n_slots) {
     extern __shared__ double2 fx[];
     const int log_n2 = log_n - 1 - log_n1, n2 = 1 << log_n2, k1 = blockIdx.x;
     for (int j = threadIdx.x; j < n2; j += blockDim.x) fx[j] = y[(size_t)k1 * n2 + j];
     __syncthreads();
     fft_block(fx, log_n2, 1 << (log_n + 1 - log_n2), cs, sn);
-    for (int i = threadIdx.x; i < n2; i += blockDim.x)
-        re[((size_t)(__brev((unsigned)i) >> (32 - log_n2)) << log_n1) + k1] = fx[i].x;
-}
-
-__global__ void decode_slots(double* z, const double* __restrict__ re, const u32* __restrict__ pow5, double inv_scale,
-                             int n_slots) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t < n_slots) z[t] = re[(pow5[t] - 1) >> 2] * inv_scale;
+    for (int i = threadIdx.x; i < n2; i += blockDim.x) {
+        const u32 t = slot_of[((__brev((unsigned)i) >> (32 - log_n2)) << log_n1) + k1];
+        if (t < (u32)n_slots) z[t] = fx[i].x * inv_scale;
+    }
 }
 
 }  // namespace
@@ -1020,24 +1042,31 @@ void decrypt_to_slots(Ctx& c, const u64* ct, int level, double* host_slots, size
     ntt_inverse(c, poly_batch(m, (size_t)nl * n, 0, 1, 1, 0, nl), s);
     if (n_slots) {
         const u64 q0 = c.primes[0], q1 = c.primes[1 % (c.L + 1)];
-        const Lift lift{q0, q1, nl == 2 ? h_inv(q0 % q1, q1) : 0, nl};
-        const int log_n1 = c.log_n / 2, n1 = 1 << log_n1, n2 = (n / 2) >> log_n1;
-        double2* y = (double2*)c.scratch_bytes("dec_y", sizeof(double2) * (n / 2));
-        double* re = (double*)c.scratch_bytes("dec_re", sizeof(double) * (n / 2));
+        const u64 q0inv = nl == 2 ? h_inv(q0 % q1, q1) : 0;
+        const Lift lift{q0, q1, h_shoup(1, q1), q0inv, h_shoup(q0inv, q1), nl};
+        const double inv_scale = std::ldexp(1.0, -c.log_scale);
         double* z = (double*)c.scratch_bytes("dec_z", sizeof(double) * c.slots);
-        {
-            LaunchScope _ls(c.prof, K_ENCODE, 8.0 * nl * n + 16.0 * (n / 2), s);
-            decode_columns<<<n2, n1 / 2, sizeof(double2) * n1, s>>>(y, m, lift, c.log_n, log_n1, c.d_cos, c.d_sin);
+        if (decode_direct(c.log_n)) {
+            double* md = (double*)c.scratch_bytes("dec_y", sizeof(double) * n);
+            {
+                LaunchScope _ls(c.prof, K_ENCODE, 8.0 * (nl + 1) * n, s);
+                lift_kernel<<<blocks_for(n), kT, 0, s>>>(md, m, lift, c.log_n);
+                CK(cudaGetLastError());
+            }
+            LaunchScope _ls(c.prof, K_ENCODE, 8.0 * (n + n_slots), s);
+            decode_sums<<<(unsigned)n_slots, kT, 0, s>>>(z, md, c.d_cos, c.d_pow5, c.log_n, inv_scale);
             CK(cudaGetLastError());
-        }
-        {
-            LaunchScope _ls(c.prof, K_ENCODE, 24.0 * (n / 2), s);
-            decode_rows<<<n1, n2 / 2, sizeof(double2) * n2, s>>>(re, y, c.log_n, log_n1, c.d_cos, c.d_sin);
-            CK(cudaGetLastError());
-        }
-        {
-            LaunchScope _ls(c.prof, K_ENCODE, 20.0 * n_slots, s);
-            decode_slots<<<blocks_for(n_slots), kT, 0, s>>>(z, re, c.d_pow5, std::ldexp(1.0, -c.log_scale), (int)n_slots);
+        } else {
+            const int log_n1 = c.log_n / 2, n1 = 1 << log_n1, n2 = (n / 2) >> log_n1;
+            double2* y = (double2*)c.scratch_bytes("dec_y", sizeof(double2) * (n / 2));
+            {
+                LaunchScope _ls(c.prof, K_ENCODE, 8.0 * nl * n + 16.0 * (n / 2), s);
+                decode_columns<<<n2, n1 / 2, sizeof(double2) * n1, s>>>(y, m, lift, c.log_n, log_n1, c.d_cos, c.d_sin);
+                CK(cudaGetLastError());
+            }
+            LaunchScope _ls(c.prof, K_ENCODE, 20.0 * (n / 2) + 8.0 * n_slots, s);
+            decode_rows<<<n1, n2 / 2, sizeof(double2) * n2, s>>>(z, y, c.log_n, log_n1, c.d_cos, c.d_sin, c.d_slot_of, inv_scale,
+                                                                 (int)n_slots);
             CK(cudaGetLastError());
         }
         CK(cudaMemcpyAsync(host_slots, z, sizeof(double) * n_slots, cudaMemcpyDeviceToHost, s));

@@ -47,6 +47,32 @@ def test_decode_matches_direct_sum(log_n):
         assert (full[:33] == ctx.decrypt(ct, level, 33)).all()
 
 
+@pytest.mark.parametrize("bits", [(60, 40), (61, 61), (20, 50)])
+@pytest.mark.parametrize("log_n", [11, 12, 16])
+def test_decode_by_direct_sums_and_by_transform(log_n, bits):
+    """The last ring decoded by direct sums, the first by a transform and the largest: two launches each, any number of
+    slots a prefix of all, within the rounding of float64 sums of the oracle's, for extreme pairs of primes."""
+    built()
+    scale = min(bits[0] - 8, 40)
+    ctx = capi.Context(log_n, bits, (61,), scale)
+    he = ckks.Ckks(ckks.Params(log_n, bits, (61,), scale))
+    ctx.keygen(3)
+    he.keygen(3)
+    z = np.random.default_rng(log_n).normal(0, 2, 40)
+    for level in (1, 0):
+        ct = ctx.empty_ct()
+        ctx.encrypt(z, level, 17, ct)
+        m = he.decrypt_coeffs(he.encrypt(z, level, 17))
+        tol = (ctx.n + 64) * 2.0 ** -53 * float(sum(abs(int(v)) for v in m)) / 2.0 ** scale
+        ctx.profile_begin()
+        full = ctx.decrypt(ct, level)
+        assert ctx.profile_end()["encode"][0] == 2
+        count = 2048 if log_n < 16 else 97
+        assert np.abs(full[:count] - he.enc.decode(m, count=min(count, ctx.slots))).max() <= tol
+        for count in (1, 33, 700):
+            assert (full[:count] == ctx.decrypt(ct, level, count)).all()
+
+
 @pytest.mark.parametrize("at", [1, 2, 700, 1024, 1025])
 def test_encryption_past_a_rejected_ternary_draw(at):
     """A seed whose ternary stream of nonce 9 outputs 2^64 - 1 (rejected) at counter `at` of N = 1024."""
