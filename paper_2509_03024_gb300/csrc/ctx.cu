@@ -1134,6 +1134,9 @@ static void make_evk(Ctx& c, EvalKey& key, const u64* d_s2, u64 obj, cudaStream_
             evk_kernel<<<blocks_for((size_t)ne * n), kT, 0, s>>>(kb, ka, c.d_sk, d_e, d_s2, ne, c.L, lo, hi,
                                                                  c.log_n, c.d_primes, c.d_pmod);
             CK(cudaGetLastError());
+        }
+        {
+            LaunchScope _ls(c.prof, K_OTHER, 32.0 * ne * n, s);
             key_store_kernel<<<blocks_for((size_t)ne * n), kT, 0, s>>>(
                 reinterpret_cast<ulonglong2*>(key.d) + (size_t)j * ne * n, kb, ka, (size_t)ne * n, c.L, c.log_n, c.keys_packed);
             CK(cudaGetLastError());
