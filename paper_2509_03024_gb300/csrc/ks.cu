@@ -255,6 +255,7 @@ void ks_run(Ctx& c, const std::vector<KsItem>& all, int level, const HoistKeys* 
         tables.upload(s);
 
         ks_transform<true, LD_GATHER, ST_SCALE>(c, d_r1, (int)r1.size(), none, K_NTT_INV, 16.0 * r1.size() * n, s);
+        c.prof.bytes[K_NTT_INV] += 8.0 * r1.size() * n;  // the second copy of every row
         ks_transform<false, LD_CONV, ST_LAST>(c, d_r2, (int)r2.size(), none, K_NTT_FWD, 16.0 * r2.size() * n, s);
 
         // K3: key inner product
