@@ -356,8 +356,6 @@ struct Ctx {
 
 // ----------------------------------------------------------------------------- kernels (ntt.cu)
 
-// Kernel attributes (dynamic shared memory limits); called once per device.
-void ntt_init();
 // In-place negacyclic NTT / inverse NTT of every row of the batch.
 void ntt_forward(const Ctx& c, const PolyBatch& pb, cudaStream_t s);
 void ntt_inverse(const Ctx& c, const PolyBatch& pb, cudaStream_t s);

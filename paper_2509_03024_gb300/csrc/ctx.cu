@@ -612,13 +612,7 @@ __device__ __forceinline__ int ternary_dev(u64 h, u64 k, u64 z_rej) {
     if (c - 1 >= (z_rej - h) * kGammaInv - 1) c++;
     return (int)(mix64_dev(h + c * 0x9E3779B97F4A7C15ULL) % 3) - 1;
 }
-// m mod q for a signed m; e mod q for a small e
-__device__ __forceinline__ u64 signed_residue(i64 m, const Prime& P) {
-    const u64 mag = m < 0 ? (u64)0 - (u64)m : (u64)m;
-    u64 r = mag - __umul64hi(mag, P.one_s) * P.q;
-    r = r >= P.q ? r - P.q : r;
-    return m < 0 && r ? P.q - r : r;
-}
+// e mod q for a small e
 __device__ __forceinline__ u64 small_residue(int e, u64 q) { return e >= 0 ? (u64)e : q - (u64)(-e); }
 
 constexpr int kEncChunk = 32;  // messages per launch
@@ -641,7 +635,7 @@ __global__ void enc_sample_kernel(u64* out, const i64* __restrict__ m, size_t m_
     for (int i = 0; i < l1; i++, o += (size_t)1 << log_n) {
         const Prime P = pr[i];
         o[0] = small_residue(v, P.q);
-        o[part] = add_mod(small_residue(e0, P.q), signed_residue(mk, P), P.q);
+        o[part] = add_mod(small_residue(e0, P.q), nttc::signed_residue(mk, P), P.q);
         o[2 * part] = small_residue(e1, P.q);
     }
 }
@@ -655,7 +649,7 @@ __global__ void seeded_sample_kernel(u64* me, const i64* __restrict__ m, size_t 
     u64* o = me + (((size_t)t * l1) << log_n) + k;
     for (int i = 0; i < l1; i++, o += (size_t)1 << log_n) {
         const Prime P = pr[i];
-        o[0] = add_mod(small_residue(e, P.q), signed_residue(mk, P), P.q);
+        o[0] = add_mod(small_residue(e, P.q), nttc::signed_residue(mk, P), P.q);
     }
 }
 
@@ -1283,7 +1277,6 @@ int fhe_ctx_create(const fhe_params* p, fhe_ctx** out) {
         for (int i = 0; i <= c.L; i++) c.max_data_prime_bits = std::max(c.max_data_prime_bits, (int)c.hprimes[i].b);
         c.keys_packed = c.max_data_prime_bits <= 50;
         c.d_primes = dupload(c.hprimes);
-        ntt_init();
         build_tables(c);
         CK(cudaDeviceSynchronize());
     });

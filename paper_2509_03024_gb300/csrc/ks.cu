@@ -266,7 +266,6 @@ void ks_run(Ctx& c, const std::vector<KsItem>& all, int level, const HoistKeys* 
         ia.src_of = d_src_of;
         ia.items = items;
         ia.dn = dn;
-        ia.alpha = A;
         ia.next = next;
         ia.level = level;
         ia.L = L;

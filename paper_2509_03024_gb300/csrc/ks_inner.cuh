@@ -31,7 +31,7 @@ struct InnerArgs {
     const int* src_of;        // fan-out: source of each item
     const HoistStep* steps;   // hoisted: device table of the rotations
     int n_steps;
-    int items, dn, alpha, next, level, L, n_ext, log_n;
+    int items, dn, next, level, L, n_ext, log_n;
     const Prime* pr;
     const u64* shared_key;    // plain: non-null when every item uses this key (then several items per thread may run)
     int split25;              // set by the launchers: data limbs use the split-at-bit-25 sums

@@ -40,8 +40,6 @@ void run_ntt(const Ctx& c, const PolyBatch& pb, cudaStream_t s) {
 
 }  // namespace
 
-void ntt_init() {}
-
 void ntt_forward(const Ctx& c, const PolyBatch& pb, cudaStream_t s) { run_ntt<false>(c, pb, s); }
 void ntt_inverse(const Ctx& c, const PolyBatch& pb, cudaStream_t s) { run_ntt<true>(c, pb, s); }
 

@@ -177,16 +177,16 @@ __device__ __forceinline__ u64 product(u64 a, u64 b, const Mod<AR>& m, const Pri
     return s.reduce(m, P);
 }
 
-// Shoup product without the final correction: a * w mod q in [0, 2q) for any a < 2^64.
-__device__ __forceinline__ u64 shoup_lazy(u64 a, u64 w, u64 ws, u64 q) {
-    u64 qh = __umul64hi(a, ws);
-    return a * w - qh * q;
-}
-
 // Any 64-bit value reduced to [0, q): a lazy Shoup product by 1, then one correction.
 __device__ __forceinline__ u64 reduce_any(u64 x, u64 q, u64 one_s) {
     u64 t = x - __umul64hi(x, one_s) * q;
     return t >= q ? t - q : t;
+}
+
+// m mod q for a signed m.
+__device__ __forceinline__ u64 signed_residue(i64 m, const Prime& P) {
+    const u64 r = reduce_any(m < 0 ? (u64)0 - (u64)m : (u64)m, P.q, P.one_s);
+    return m < 0 && r ? P.q - r : r;
 }
 
 // Element x (within its sub-transform) that register u of the 2^RB-element group g holds in

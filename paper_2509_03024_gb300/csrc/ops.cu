@@ -9,6 +9,7 @@
 // context's pinned descriptor arena.
 #include <algorithm>
 
+#include "ks_inner.cuh"
 #include "ntt_core.cuh"
 
 namespace fhe {
@@ -289,14 +290,6 @@ __global__ void sum_acc_kernel(const AccTarget* __restrict__ tg, const BinItem* 
     }
 }
 
-// v mod q: one Shoup product by 1 instead of a 64-bit division
-__device__ __forceinline__ u64 signed_mod(i64 v, const Prime& P) {
-    const u64 mag = v < 0 ? (u64)0 - (u64)v : (u64)v;
-    u64 r = mag - __umul64hi(mag, P.one_s) * P.q;
-    r = r >= P.q ? r - P.q : r;
-    return v < 0 && r ? P.q - r : r;
-}
-
 __global__ void int_to_rns_kernel(u64* out, size_t out_stride, const i64* __restrict__ in, size_t in_stride,
                                   int items, int limbs, int log_n, const Prime* __restrict__ pr) {
     const size_t total = (size_t)items * limbs << log_n;
@@ -307,7 +300,7 @@ __global__ void int_to_rns_kernel(u64* out, size_t out_stride, const i64* __rest
         int limb = (int)(row % limbs);
         int item = (int)(row / limbs);
         out[(size_t)item * out_stride + ((size_t)limb << log_n) + k] =
-            signed_mod(in[(size_t)item * in_stride + k], pr[limb]);
+            nttc::signed_residue(in[(size_t)item * in_stride + k], pr[limb]);
     }
 }
 
@@ -328,16 +321,7 @@ __global__ void int8_to_rns_kernel(u64* out, size_t out_stride, const int8_t* __
     }
 }
 
-// Evaluation slot k holds a(psi^(2 brev(k) + 1)); X -> X^g maps it to the slot k'
-// with 2 brev(k') + 1 = g (2 brev(k) + 1) mod 2N.
-__device__ __forceinline__ int auto_src(int k, long long g, int log_n) {
-    const unsigned sh = 32 - log_n;
-    unsigned bk = __brev((unsigned)k) >> sh;
-    unsigned e = (unsigned)(((unsigned long long)g * (2ull * bk + 1ull)) & ((2ull << log_n) - 1ull));
-    return (int)(__brev((e - 1u) >> 1) >> sh);
-}
-
-__global__ void automorphism_kernel(u64* out, const u64* __restrict__ in, int limbs, int log_n, long long g) {
+__global__ void automorphism_kernel(u64* out, const u64* __restrict__ in, int limbs, int log_n, int g) {
     const size_t total = (size_t)limbs << log_n;
     for (size_t e = blockIdx.x * (size_t)blockDim.x + threadIdx.x; e < total;
          e += (size_t)gridDim.x * blockDim.x) {

@@ -81,23 +81,21 @@ void tune_inner(Ctx& c, int level, std::vector<fhe_tune_result>& out) {
     const int n = c.n, A = c.alpha, l1 = level + 1, next = l1 + A, dn = c.dnum(level);
     const int items = c.log_n >= 16 ? 32 : 64, steps = 15;
     DevTmp tmp;
-    // ext: [items][dn][next][N]; keys: [steps][dnum_top][2][n_ext][N]; inputs [items][L+1][N]; acc, c0sum
+    // ext [items][dn][next][N], keys [steps][digit][n_ext][N][2], c0 [items][L+1][N]; acc, c0sum
     const size_t key_words = c.key_words();
     u64* ext = tmp.get((size_t)items * dn * next * n);
     u64* keys = tmp.get((size_t)steps * key_words);
-    u64* din = tmp.get((size_t)items * (c.L + 1) * n);
     u64* c0 = tmp.get((size_t)items * (c.L + 1) * n);
     u64* acc = tmp.get((size_t)items * 2 * next * n);
     u64* c0sum = tmp.get((size_t)items * l1 * n);
-    // the key rows are laid out [digit][n_ext][N][2]; residues below the smallest prime serve every row
+    // residues below the smallest prime serve every row
     fill_residues<<<1024, 256>>>(ext, (size_t)items * dn * next * n, c.log_n, 1, c.d_primes, 1);
     fill_residues<<<1024, 256>>>(keys, (size_t)steps * key_words, c.log_n, 1, c.d_primes, 2);
-    fill_residues<<<1024, 256>>>(din, (size_t)items * (c.L + 1) * n, c.log_n, 1, c.d_primes, 3);
     fill_residues<<<1024, 256>>>(c0, (size_t)items * (c.L + 1) * n, c.log_n, 1, c.d_primes, 4);
     CK(cudaGetLastError());
     std::vector<KsItem> it(items);
     for (int t = 0; t < items; t++) {
-        it[t] = KsItem{din + (size_t)t * (c.L + 1) * n, keys, c0 + (size_t)t * (c.L + 1) * n, nullptr, nullptr,
+        it[t] = KsItem{nullptr, keys, c0 + (size_t)t * (c.L + 1) * n, nullptr, nullptr,
                        nullptr, nullptr, 1};
     }
     std::vector<HoistStep> hs(steps);
@@ -117,7 +115,6 @@ void tune_inner(Ctx& c, int level, std::vector<fhe_tune_result>& out) {
     ia.tab = d_it;
     ia.items = items;
     ia.dn = dn;
-    ia.alpha = A;
     ia.next = next;
     ia.level = level;
     ia.L = c.L;
@@ -166,7 +163,6 @@ void tune_ntt(Ctx& c, std::vector<fhe_tune_result>& out) {
     fill_residues<<<1024, 256>>>(buf, (size_t)polys * L1 * c.n, c.log_n, 1, c.d_primes, 5);
     CK(cudaGetLastError());
     const PolyBatch pb = poly_batch(buf, (size_t)L1 * c.n, 0, polys, 1, 0, L1);
-    const int saved = c.tune.ntt;
     double best = 1e30;
     int best_v = 0;
     const size_t first = out.size();
@@ -182,7 +178,6 @@ void tune_ntt(Ctx& c, std::vector<fhe_tune_result>& out) {
             best_v = v;
         }
     }
-    (void)saved;
     out[first + best_v].chosen = 1;
     c.tune.ntt = best_v;
     CK(cudaDeviceSynchronize());
