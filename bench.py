@@ -46,13 +46,14 @@ sys.path.insert(0, HERE)
 
 METRIC = "encrypted MF ratings/sec, served vs one-by-one on 1 GB300; p50/p99 latency"
 # DRAM bytes per limb row of a forward NTT pass at N = 2^15, from the ncu capture (dram__bytes_read
-# + write) of the fused ModUp passes of the current kernels (the hoisted rotate-and-sum of 64
-# ciphertexts at level 6, 1856 rows per pass): (552.8 MB + 917.4 MB) / 2 passes / 1856 rows
-NCU_FWD_DRAM_BYTES_PER_ROW = (552.8e6 + 917.4e6) / 2 / 1856
+# + write, profiles/ks_passes_paper_N2e15.md) of the fused ModUp passes (the hoisted rotate-and-sum of 64
+# ciphertexts at level 6, 1856 rows per pass): (558.6 MB + 914.9 MB) / 2 passes / 1856 rows
+NCU_FWD_DRAM_BYTES_PER_ROW = (558.6e6 + 914.9e6) / 2 / 1856
 # the same for the served ring's forward passes (N = 2^16, 13 + 3 primes): ncu dram__bytes_read + write
 # of the four forward passes (ModUp conversion and second pass, ModDown conversion and combine) of a
-# key switch of 8 top-level ciphertexts, 1240 MB over 1488 limb-row passes (0.79 x the algorithmic 16 N)
-NCU_SERVED_FWD_DRAM_BYTES_PER_ROW = 1239.7e6 / 1488
+# key switch of 8 top-level ciphertexts, 1241 MB over 1488 limb-row passes (0.80 x the algorithmic 16 N;
+# profiles/served_fwd_traffic_N2e16.md)
+NCU_SERVED_FWD_DRAM_BYTES_PER_ROW = 1241.2e6 / 1488
 UNIT = "ratings/s"
 SEED = 20250903
 LR, LAM, K_RANK = 0.005, 0.02, 10
@@ -932,7 +933,7 @@ def roofline_of(stats, ceil, hbm_peak, measured, traffic_per_row, log_n):
                                   "scaled by the rows of the average launch" if traffic else None,
                 "peak_source": ceil["source"],
                 "probe_peak": {"value": ceil["probe_butterfly_gbfly"], "frac": achieved / ceil["probe_butterfly_gbfly"],
-                               "source": "fhe_probe_butterfly_rate: this library's lazy Shoup butterfly code on "
+                               "source": "fhe_probe_butterfly_rate: this library's butterfly code for the first data prime on "
                                          "register-resident values (no memory traffic)"},
                 "butterflies_per_launch": work / launches, "hbm_view": hbm_view, **base}
     if name == "ks_inner" and work > 0:

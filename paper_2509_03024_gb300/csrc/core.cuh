@@ -470,6 +470,7 @@ void encode_sparse_device(Ctx& c, const std::vector<std::pair<int, double>>& nz,
 // Encode many sparse slot vectors at once: nz lists concatenated with offsets (host), out [count][N].
 void encode_many_device(Ctx& c, const std::vector<int>& idx, const std::vector<double>& val,
                         const std::vector<int>& offsets, i64* out_dev, cudaStream_t s);
+// The ciphertexts are complete when the call returns (it synchronises s).
 void encrypt_coeffs_device(Ctx& c, const i64* m_dev, size_t m_stride, int count, int level,
                            const std::vector<u64>& nonces, u64* ct, cudaStream_t s);
 
@@ -486,7 +487,8 @@ struct SeedRow {
 u64 seeded_key(const Ctx& c, u64 obj, int limb);
 // Fill each row with its uniform coefficients (coefficient form).
 void seeded_uniform_device(Ctx& c, const std::vector<SeedRow>& rows, cudaStream_t s);
-// c0 only, evaluation domain, compact [count][level+1][N] at c0_out.
+// c0 only, evaluation domain, compact [count][level+1][N] at c0_out, in the order of s: a caller that reads it
+// on the host or from another stream waits for s.
 void encrypt_seeded_device(Ctx& c, const i64* m_dev, size_t m_stride, int count, int level,
                            const std::vector<u64>& objs, u64* c0_out, cudaStream_t s);
 // plaintext materialisation: int64 coefficients -> evaluation domain limbs [0, limbs)

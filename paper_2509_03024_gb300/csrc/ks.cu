@@ -3,12 +3,13 @@
 // For one polynomial d at level l (l1 = l+1 limbs, evaluation domain) and a key
 // of dnum digits of alpha limbs, with ext = Q_l u P (next = l1 + alpha limbs):
 //
-//   K1  inverse NTT of d (read through the automorphism of the item); the last
-//       pass stores y_i = c_i * N^-1 * qhat_i^-1 mod q_i (ModUp's first factor),
+//   K1  inverse NTT of d (read through the automorphism of the item); the first
+//       pass also stores the rows it reads as their digits' own limbs, the last
+//       stores y_i = c_i * N^-1 * qhat_i^-1 mod q_i (ModUp's first factor),
 //   K2  for every digit j and every target limb x outside D_j: the first pass
 //       of a forward NTT loads sum_{i in D_j} y_i * qhat_i mod p_x (fast base
-//       conversion, Bajard et al. 2016) and the transform yields ModUp_j(d)_x;
-//       the limbs of D_j are d itself and are read from d in K3,
+//       conversion, Bajard et al. 2016) and the transform yields ModUp_j(d)_x
+//       beside the limbs of D_j that K1 stored, so K3 reads every limb alike,
 //   K3  acc_h = sum_j ModUp_j(d) * evk_j[h] over ext (key inner product),
 //   K4  inverse NTT of the alpha special limbs of acc_h; the last pass stores
 //       y_k = c_k * N^-1 * Phat_k^-1 mod p_k,
@@ -16,9 +17,9 @@
 //       sum_k y_k * Phat_k mod q_i (Conv_{P->Q}); the last pass stores
 //       out_h = (acc_h - conv) * P^-1 + the item's add terms (ModDown).
 //
-// K1, K2, K4, K5 run the register-blocked NTT tiles of ntt_core.cuh over row
-// tables (one descriptor per limb row), so the conversions happen while the
-// tiles are loaded and the combinations while they are stored.
+// K1, K2, K4, K5 run the pass kernels of ks_pass.cuh over row tables (one
+// descriptor per limb row), so the conversions happen while a pass loads its
+// residues and the combinations while it stores them.
 //
 // The exact rescale uses the same machinery: an inverse transform of the last limb, then forward
 // transforms whose load forms the centred last limb modulo each q_i and whose store writes
@@ -336,8 +337,7 @@ void ks_run(Ctx& c, const std::vector<KsItem>& all, int level, const HoistKeys* 
     }
 }
 
-// K4/K5 of a plain key switch over the items' accumulators acc ([item][2][next][N]): out_h =
-// (acc_h - Conv_{P->Q}(acc_h)) P^-1 + the item's add terms.
+// The tables of K4/K5 of a plain key switch over the items' accumulators acc ([item][2][next][N]).
 DownRows moddown_rows(Ctx& c, int items, const u64* acc, int level, cudaStream_t s) {
     const int n = c.n, L = c.L, A = c.alpha, l1 = level + 1, next = l1 + A;
     u64* yP = c.scratch_u64("ks_yp", (size_t)items * 2 * A * n);
@@ -375,6 +375,7 @@ DownRows moddown_rows(Ctx& c, int items, const u64* acc, int level, cudaStream_t
     return {c.arena.push_vec(r4, s), c.arena.push_vec(r5, s), (int)r4.size(), (int)r5.size()};
 }
 
+// K4/K5 over those tables: out_h = (acc_h - Conv_{P->Q}(acc_h)) P^-1 + the item's add terms.
 void moddown_run(Ctx& c, const DownRows& d, const KsItem* d_items, const u64* acc, int level, cudaStream_t s) {
     const CombineArgs ca{d_items, acc, c.d_pinv, level + 1 + c.alpha, nullptr};
     const CombineArgs none{nullptr, nullptr, nullptr, 0, nullptr};

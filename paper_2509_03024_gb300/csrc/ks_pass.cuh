@@ -306,8 +306,8 @@ single_pass_kernel(ROWS rows, const Prime* __restrict__ primes, const ulonglong2
 // What bounds it: the 32-bit multiply pipe (ntt_core.cuh) and, in passes whose loads convert, the latency
 // of their loads. Plain forward + inverse transform of 256 rows, N = 2^15 / 2^16 (ms): radix-8 tiles filled
 // from shared memory with Shoup products 0.205 / 0.424, the same with split products 0.176 / 0.372,
-// these passes 0.140 / 0.306; ModUp conversion pass set of 64 top-level inputs 1.032 / 4.66 -> 0.717 / 3.00, and 0.595 / 2.64 with the loads of several residues
-// issued before the first store.
+// these passes 0.141 / 0.305; ModUp conversion pass set of 64 top-level inputs 1.032 / 4.66 -> 0.717 / 3.00, and
+// 0.590 / 2.60 with the loads of several residues issued before the first store.
 template <class ROWS, int LOGN, int LOGM, int R, bool INV, int PASS, int LOAD, int STORE, int RB, int MINB>
 __global__ void __launch_bounds__(R * (1 << LOGM) / (1 << RB), MINB)
 pass_kernel(ROWS rows, int n_rows, int per_cta, const Prime* __restrict__ primes, const ulonglong2* __restrict__ tw,
@@ -509,9 +509,9 @@ void transform_t(const Ctx& c, const ROWS& rows, int n_rows, const CombineArgs& 
 // The tile shapes of the fused passes the autotuner chooses between (family "ks_pass"): rows or
 // columns per tile of the two-pass rings, 16 residues per thread under a cap of 64 registers (r8x: 8 rows
 // with 80 registers: fewer spills, a quarter fewer threads per SM); every shape computes the same bits.
-// The exact rescale of 64 ciphertexts at N = 2^15 / 2^16 (ms): r16 0.355 / 1.12, r8 0.355 / 1.10, r8x
-// 0.394 / 1.25; under 80 registers r16 took 0.396 / 1.25 (the loads' latency needs the warps). Each shape's instantiations live in a translation unit of their own
-// (ks_pass16.cu, ks_pass8.cu, ks_pass8x.cu).
+// The exact rescale of 64 ciphertexts at N = 2^15 / 2^16 (ms): r16 0.306 / 0.969, r8 0.294 / 0.951, r8x
+// 0.322 / 1.016 (the loads' latency needs the warps). Each shape's instantiations live in a translation
+// unit of their own (ks_pass16.cu, ks_pass8.cu, ks_pass8x.cu).
 enum KsTile { KS_R16 = 0, KS_R8, KS_R8X, KS_N_TILES };
 extern const char* const kKsTileNames[KS_N_TILES];
 

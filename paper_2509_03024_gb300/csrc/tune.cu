@@ -6,6 +6,10 @@
 //   ks_hoist_inner  K3 of the hoisted rotate-and-sum (kp - 1 = 15 rotations, the epoch's per-group
 //                   rotate-and-sum), variants of ks_inner.cuh
 //   ks_inner        K3 of a relinearisation (every item shares the key), variants of ks_inner.cuh
+//   ntt             the plain two-pass transforms of rings of 2^14 and more, tile shapes of ntt_tile.cuh
+//   ks_pass         the fused key-switch and rescale passes of the same rings, tile shapes of ks_pass.cuh
+// The tile shapes hold for launches of many rows; launches of few (rules::few_rows) and smaller rings have shapes
+// of their own.
 // The synthetic operands are uniform residues below each prime; the kernels' work does not depend
 // on the values.
 #include <cstring>
