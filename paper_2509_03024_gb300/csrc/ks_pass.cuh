@@ -147,9 +147,9 @@ __device__ __forceinline__ void with_count(int cnt, F&& f) {
     else f(nttc::Tag<0>{});
 }
 
-// Residue k of the row as it stands in memory (LD_CONV: conv_rows). The kernels of few or short rows load it before
-// anything of the row's prime is known: behind the branch on the prime's arithmetic the loads wait for the prime,
-// one more trip to L2 in a launch that is a handful of them.
+// Residue k of the row as it stands in memory (LD_CONV: conv_rows). The single-pass kernel loads it before anything
+// of the row's prime is known: behind the branch on the prime's arithmetic the loads wait for the prime, one more
+// trip to L2 in a launch that may be a handful of them (two launches of three rows at N = 2^9 10.5 -> 9.1 us).
 template <int LOAD>
 __device__ __forceinline__ u64 load_raw(const KsRow& r, size_t k, int log_n) {
     if constexpr (LOAD == LD_PLAIN) return r.dst[k];
@@ -263,7 +263,7 @@ single_pass_kernel(ROWS rows, const Prime* __restrict__ primes, const ulonglong2
 #pragma unroll
         for (int u = 0; u < 8; u++) raw[u] = load_raw<LOAD>(r, addr(u), LOGN);
     }
-    nttc::with_arith(P, [&](auto ar) {
+    nttc::with_arith<INV>(P, [&](auto ar) {
         constexpr int AR = decltype(ar)::value;
         const nttc::Mod<AR> m(P);
         const RowConst rc = row_const<LOAD>(r, primes);
@@ -336,12 +336,7 @@ pass_kernel(ROWS rows, int n_rows, int per_cta, const Prime* __restrict__ primes
         auto elem = [&](int blk, int u) { return blk < 0 ? g + T * u : nttc::block_elem<LOGM, RB>(blk, g, u); };
         auto load_addr = [&](int u) { return addr(INV && PASS == 0 ? elem(NB - 1, u) : g + T * u); };
         u64 v[V];
-        constexpr bool early = LOAD != LD_CONV && RB == 3;  // (16 residues a thread: spills instead)
-        if constexpr (early) {
-#pragma unroll
-            for (int u = 0; u < V; u++) v[u] = load_raw<LOAD>(r, load_addr(u), LOGN);
-        }
-        nttc::with_arith(P, [&](auto ar) {
+        nttc::with_arith<INV>(P, [&](auto ar) {
             constexpr int AR = decltype(ar)::value;
             const nttc::Mod<AR> m(P);
             auto put = [&](int blk) {
@@ -380,7 +375,7 @@ pass_kernel(ROWS rows, int n_rows, int per_cta, const Prime* __restrict__ primes
             } else {
 #pragma unroll
                 for (int u = 0; u < V; u++)
-                    v[u] = load_elem<LOAD>(r, early ? v[u] : load_raw<LOAD>(r, load_addr(u), LOGN), load_addr(u), P, m, rc);
+                    v[u] = load_elem<LOAD>(r, load_raw<LOAD>(r, load_addr(u), LOGN), load_addr(u), P, m, rc);
                 if (LOAD == LD_GATHER && r.out2) {
 #pragma unroll
                     for (int u = 0; u < V; u++) r.out2[addr(g + T * u)] = r.pack ? key_pack(v[u]) : v[u];

@@ -28,14 +28,15 @@ namespace nttc {
 //              first operand folded in every other forward stage, the sum in every inverse one
 //   AR_SHOUP   any prime up to 61 bits: Shoup products with a quotient from the three upper partial
 //              products (at most two below the true one), y w < 4 q; values below 8 q, the first
-//              operand of each butterfly brought below 4 q. Below 2^57 (Mod::lazy) a forward transform
-//              leaves it as it is: 8 q and 4 q more per stage are below 72 q < 2^64 after 16 stages
-//              (1024 polynomials of four 40-bit limbs at N = 2^12 217 -> 205 us, 84 of six 45-bit limbs
-//              at 2^16 477 -> 421)
+//              operand of each butterfly brought below 4 q
+//   AR_LAZY    the same for the forward transforms of primes below 2^57, which leave the first operand as it
+//              is: 8 q and 4 q more per stage are below 72 q < 2^64 after 16 stages (1024 polynomials of four 40-bit limbs at N = 2^12 217 -> 197 us, 84 of six 45-bit limbs
+//              at 2^16 477 -> 420)
 // Register-only rate of the forward butterfly (GB300, 10^9 per second, unrolled radix-8 blocks): Shoup
 // with the exact quotient 998, NEAR50 1420 (13 instructions); the same with B's low word shifted by
 // shift and add 1290, with unsigned values and a multiple of q in the difference 1120.
-enum Arith { AR_SHOUP = 0, AR_NEAR50 = 1, AR_NEAR60 = 2 };
+// Prime::cls holds one of the first three; with_arith makes AR_SHOUP of a small prime AR_LAZY.
+enum Arith { AR_SHOUP = 0, AR_NEAR50 = 1, AR_NEAR60 = 2, AR_LAZY = 3 };
 __host__ __device__ constexpr int split_at(int ar) { return ar == AR_NEAR50 ? 20 : 29; }
 
 __device__ __forceinline__ u64 mul_wide(u32 a, u32 b) {
@@ -61,8 +62,8 @@ struct Mod {
     u64 q;
     u64 K;      // multiple of q: 2^13 q (NEAR50: makes any signed value non-negative), 7 q (NEAR60), 4 q (SHOUP)
     u32 delta;  // near primes
-    bool lazy;  // SHOUP: forward transforms run unreduced
-    __device__ __forceinline__ explicit Mod(const Prime& p) : q(p.q), lazy(AR == AR_SHOUP && p.b <= 57) {
+    static constexpr bool shoup = AR == AR_SHOUP || AR == AR_LAZY;
+    __device__ __forceinline__ explicit Mod(const Prime& p) : q(p.q) {
         K = AR == AR_NEAR50 ? p.q << 13 : AR == AR_NEAR60 ? p.q * 7 : p.q << 2;
         delta = p.delta;
     }
@@ -70,7 +71,7 @@ struct Mod {
     __device__ __forceinline__ u64 mul(u64 y, const ulonglong2& w) const {
         const u32 y0 = (u32)y, y1 = (u32)(y >> 32);
         const u32 a0 = (u32)w.x, a1 = (u32)(w.x >> 32), b0 = (u32)w.y, b1 = (u32)(w.y >> 32);
-        if constexpr (AR == AR_SHOUP) {
+        if constexpr (shoup) {
             const u64 c0 = mul_wide(y0, b1), c1 = mul_wide(y1, b0);
             const u64 qh = mad_wide(y1, b1, (c0 >> 32) + (c1 >> 32));
             return y * w.x - qh * q;
@@ -87,13 +88,13 @@ struct Mod {
     // a congruent value: NEAR50 any signed v to (-2^39, 2^50 + 2^39), NEAR60 any v below 2^60 + 2^30,
     // SHOUP v < 8 q below 4 q
     __device__ __forceinline__ u64 fold(u64 v) const {
-        if constexpr (AR == AR_SHOUP) return v >= K ? v - K : v;
+        if constexpr (shoup) return v >= K ? v - K : v;
         else if constexpr (AR == AR_NEAR50) return mad_wide_s((u32)((i64)v >> 50), delta, v & (((u64)1 << 50) - 1));
         else return mad_wide((u32)(v >> 60), delta, v & (((u64)1 << 60) - 1));
     }
     // any v in the ranges above reduced to [0, q) (SHOUP: any v at all)
     __device__ __forceinline__ u64 canon(u64 v, u64 one_s) const {
-        if constexpr (AR == AR_SHOUP) {
+        if constexpr (shoup) {
             v -= __umul64hi(v, one_s) * q;
         } else if constexpr (AR == AR_NEAR50) {
             v += K;  // in [0, 2^64)
@@ -104,16 +105,14 @@ struct Mod {
         const u64 d = v - q;  // v < 2 q < 2^62
         return (i64)d < 0 ? v : d;
     }
-    // Forward Cooley-Tukey butterfly X <- X + W Y, Y <- X - W Y, in the i-th stage of a register block. RED: the
-    // first operand is reduced (SHOUP; NEAR60 in every other stage).
-    template <bool RED>
+    // Forward Cooley-Tukey butterfly X <- X + W Y, Y <- X - W Y, in the i-th stage of a register block.
     __device__ __forceinline__ void ct(u64& x, u64& y, const ulonglong2& w, int i) const {
         const u64 t = mul(y, w);
         if constexpr (AR == AR_NEAR50) {
             y = x - t;
             x += t;
         } else {
-            const u64 a = RED && (AR == AR_SHOUP || (i & 1) == 0) ? fold(x) : x;
+            const u64 a = AR == AR_SHOUP || (AR == AR_NEAR60 && (i & 1) == 0) ? fold(x) : x;
             x = a + t;
             y = a + K - t;
         }
@@ -204,9 +203,9 @@ __device__ __forceinline__ int block_elem(int blk, int g, int u) {
 // thread group g, elements block_elem(BLK, g, u), through stages [RB BLK, min(RB BLK + RB, LOGM))
 // (forward ascending, inverse descending). tw(s, k) returns the twiddle of this thread's k-th
 // sub-group at stage s (a block of b stages over 2^RB values holds 2^(RB-b+j) sub-groups at its stage j).
-// FOLD: the inverse NEAR50 values may be large (every block but the first after reduced inputs). RED: see Mod::ct.
-template <int LOGM, int RB, int BLK, bool INV, bool FOLD, bool RED, int AR, class TW>
-__device__ __forceinline__ void stages_of(u64 (&v)[1 << RB], const Mod<AR>& m, TW&& tw) {
+// FOLD: the inverse NEAR50 values may be large (every block but the first after reduced inputs).
+template <int LOGM, int RB, int BLK, bool INV, bool FOLD, int AR, class TW>
+__device__ __forceinline__ void block_stages(u64 (&v)[1 << RB], const Mod<AR>& m, TW&& tw) {
     constexpr int V = 1 << RB, S0 = RB * BLK;
     constexpr int b = (LOGM - S0) < RB ? (LOGM - S0) : RB;
     if (INV && FOLD && AR == AR_NEAR50) {
@@ -222,25 +221,23 @@ __device__ __forceinline__ void stages_of(u64 (&v)[1 << RB], const Mod<AR>& m, T
             if (u & dist) continue;
             const ulonglong2 w = tw(S0 + j, u >> (b - j));
             if (INV) m.gs(v[u], v[u + dist], w);
-            else m.template ct<RED>(v[u], v[u + dist], w, i);
+            else m.ct(v[u], v[u + dist], w, i);
         }
     }
 }
-template <int LOGM, int RB, int BLK, bool INV, bool FOLD, int AR, class TW>
-__device__ __forceinline__ void block_stages(u64 (&v)[1 << RB], const Mod<AR>& m, TW&& tw) {
-    if (!INV && AR == AR_SHOUP && m.lazy) stages_of<LOGM, RB, BLK, INV, FOLD, false>(v, m, tw);
-    else stages_of<LOGM, RB, BLK, INV, FOLD, true>(v, m, tw);
-}
 
-// f is called with the arithmetic of prime p as a compile-time constant.
 template <int V>
 struct Tag {
     static constexpr int value = V;
 };
-template <class F>
+// f is called with the arithmetic of prime p as a compile-time constant, for a transform of the direction INV. (A branch
+// around the butterflies of every register block in place of AR_LAZY keeps their twiddles from loading early: two
+// polynomials of three 32- and 40-bit limbs at N = 2^13, forward and inverse, 29.7 us against 28.8 before it.)
+template <bool INV, class F>
 __device__ __forceinline__ void with_arith(const Prime& p, F&& f) {
     if (p.cls == AR_NEAR50) f(Tag<AR_NEAR50>{});
     else if (p.cls == AR_NEAR60) f(Tag<AR_NEAR60>{});
+    else if (!INV && p.b <= 57) f(Tag<INV ? AR_SHOUP : AR_LAZY>{});
     else f(Tag<AR_SHOUP>{});
 }
 

@@ -38,12 +38,12 @@ bfly_probe_kernel(u64* out, const ulonglong2* __restrict__ tw, const Prime* __re
 #pragma unroll
         for (int blk = 0; blk < 5; blk++) {  // 15 stages
 #pragma unroll
-            for (int u = 0; u < 4; u++) m.template ct<true>(v[u], v[u + 4], w[0], 0);
+            for (int u = 0; u < 4; u++) m.ct(v[u], v[u + 4], w[0], 0);
 #pragma unroll
             for (int u = 0; u < 8; u++)
-                if (!(u & 2)) m.template ct<true>(v[u], v[u + 2], w[1 + (u >> 2)], 1);
+                if (!(u & 2)) m.ct(v[u], v[u + 2], w[1 + (u >> 2)], 1);
 #pragma unroll
-            for (int u = 0; u < 8; u += 2) m.template ct<true>(v[u], v[u + 1], w[3 + (u >> 1)], 2);
+            for (int u = 0; u < 8; u += 2) m.ct(v[u], v[u + 1], w[3 + (u >> 1)], 2);
         }
 #pragma unroll
         for (int u = 0; u < 8; u++) v[u] = m.canon(v[u], one_s);
