@@ -30,8 +30,8 @@ namespace nttc {
 //              products (at most two below the true one), y w < 4 q; values below 8 q, the first
 //              operand of each butterfly brought below 4 q
 //   AR_LAZY    the same for the forward transforms of primes below 2^57, which leave the first operand as it
-//              is: 8 q and 4 q more per stage are below 72 q < 2^64 after 16 stages (1024 polynomials of four 40-bit limbs at N = 2^12 217 -> 197 us, 84 of six 45-bit limbs
-//              at 2^16 477 -> 420)
+//              is: 8 q and 4 q more per stage are below 72 q < 2^64 after 16 stages (1024 polynomials of four 40-bit
+//              limbs at N = 2^12 217 -> 197 us, 84 of six 45-bit limbs at 2^16 477 -> 420)
 // Register-only rate of the forward butterfly (GB300, 10^9 per second, unrolled radix-8 blocks): Shoup
 // with the exact quotient 998, NEAR50 1420 (13 instructions); the same with B's low word shifted by
 // shift and add 1290, with unsigned values and a multiple of q in the difference 1120.
