@@ -13,6 +13,7 @@ namespace fhe {
 
 // ============================================================================ errors
 
+using nttc::AR_LAZY;
 using nttc::AR_NEAR50;
 using nttc::AR_NEAR60;
 using nttc::AR_SHOUP;
@@ -150,7 +151,7 @@ static ulonglong2 words_at(u64 w, const Prime& p, int at) {
     return make_ulonglong2(split_word(w, at), split_word(h_mul(w, ((u64)1 << 32) % p.q, p.q), at));
 }
 static void const_words(u64 w, const Prime& p, u64* out) {
-    const ulonglong2 t = p.cls == AR_SHOUP ? make_ulonglong2(w, h_shoup(w, p.q)) : words_at(w, p, nttc::split_at(p.cls));
+    const ulonglong2 t = nttc::is_near(p.cls) ? words_at(w, p, nttc::split_at(p.cls)) : make_ulonglong2(w, h_shoup(w, p.q));
     out[0] = t.x;
     out[1] = t.y;
 }
@@ -161,11 +162,11 @@ static Prime make_prime(u64 q) {
     p.mu = (u64)(((u128)1 << (2 * p.b)) / q);
     p.one_s = h_shoup(1, q);
     const u64 delta = ((u64)1 << p.b) - q;
-    p.cls = AR_SHOUP;
+    p.cls = p.b <= 57 ? AR_LAZY : AR_SHOUP;
     if (p.b == 50 && delta <= ((u64)1 << 26)) p.cls = AR_NEAR50;
     if (p.b == 60 && delta <= ((u64)1 << 26)) p.cls = AR_NEAR60;
-    p.delta = p.cls == AR_SHOUP ? 0 : (u32)delta;
-    if (p.cls != AR_SHOUP) {
+    p.delta = nttc::is_near(p.cls) ? (u32)delta : 0;
+    if (nttc::is_near(p.cls)) {
         const_words((u64)(((u128)1 << 64) % q), p, p.w64);
         const_words(((u64)1 << 50) % q, p, p.w50);
     }
@@ -307,8 +308,8 @@ static void build_tables(Ctx& c) {
     for (size_t i = 0; i < tw.size(); i++) {
         const Prime& p = c.hprimes[i / n];
         const int at = nttc::split_at(p.cls);
-        tw[i] = p.cls == AR_SHOUP ? make_ulonglong2(psi[i], h_shoup(psi[i], p.q)) : words_at(psi[i], p, at);
-        itw[i] = p.cls == AR_SHOUP ? make_ulonglong2(ipsi[i], h_shoup(ipsi[i], p.q)) : words_at(ipsi[i], p, at);
+        tw[i] = nttc::is_near(p.cls) ? words_at(psi[i], p, at) : make_ulonglong2(psi[i], h_shoup(psi[i], p.q));
+        itw[i] = nttc::is_near(p.cls) ? words_at(ipsi[i], p, at) : make_ulonglong2(ipsi[i], h_shoup(ipsi[i], p.q));
     }
     c.d_tw = dupload(tw);
     c.d_itw = dupload(itw);

@@ -263,7 +263,7 @@ single_pass_kernel(ROWS rows, const Prime* __restrict__ primes, const ulonglong2
 #pragma unroll
         for (int u = 0; u < 8; u++) raw[u] = load_raw<LOAD>(r, addr(u), LOGN);
     }
-    nttc::with_arith<INV>(P, [&](auto ar) {
+    nttc::with_arith<!INV>(P, [&](auto ar) {
         constexpr int AR = decltype(ar)::value;
         const nttc::Mod<AR> m(P);
         const RowConst rc = row_const<LOAD>(r, primes);
@@ -336,7 +336,7 @@ pass_kernel(ROWS rows, int n_rows, int per_cta, const Prime* __restrict__ primes
         auto elem = [&](int blk, int u) { return blk < 0 ? g + T * u : nttc::block_elem<LOGM, RB>(blk, g, u); };
         auto load_addr = [&](int u) { return addr(INV && PASS == 0 ? elem(NB - 1, u) : g + T * u); };
         u64 v[V];
-        nttc::with_arith<INV>(P, [&](auto ar) {
+        nttc::with_arith<!INV && RB == 4>(P, [&](auto ar) {
             constexpr int AR = decltype(ar)::value;
             const nttc::Mod<AR> m(P);
             auto put = [&](int blk) {

@@ -29,14 +29,15 @@ namespace nttc {
 //   AR_SHOUP   any prime up to 61 bits: Shoup products with a quotient from the three upper partial
 //              products (at most two below the true one), y w < 4 q; values below 8 q, the first
 //              operand of each butterfly brought below 4 q
-//   AR_LAZY    the same for the forward transforms of primes below 2^57, which leave the first operand as it
-//              is: 8 q and 4 q more per stage are below 72 q < 2^64 after 16 stages (1024 polynomials of four 40-bit
-//              limbs at N = 2^12 217 -> 197 us, 84 of six 45-bit limbs at 2^16 477 -> 420)
+//   AR_LAZY    the same for primes below 2^57, whose forward transforms (of many or short rows, with_arith) leave
+//              the first operand as it is: 8 q and 4 q more per stage are below 72 q < 2^64 after 16 stages (1024
+//              polynomials of four 40-bit limbs at N = 2^12 217 -> 197 us, 84 of six 45-bit limbs at 2^16 477 -> 420)
 // Register-only rate of the forward butterfly (GB300, 10^9 per second, unrolled radix-8 blocks): Shoup
 // with the exact quotient 998, NEAR50 1420 (13 instructions); the same with B's low word shifted by
 // shift and add 1290, with unsigned values and a multiple of q in the difference 1120.
-// Prime::cls holds one of the first three; with_arith makes AR_SHOUP of a small prime AR_LAZY.
+// Prime::cls holds one of the four (AR_LAZY where it applies).
 enum Arith { AR_SHOUP = 0, AR_NEAR50 = 1, AR_NEAR60 = 2, AR_LAZY = 3 };
+__host__ __device__ constexpr bool is_near(u32 cls) { return cls == AR_NEAR50 || cls == AR_NEAR60; }
 __host__ __device__ constexpr int split_at(int ar) { return ar == AR_NEAR50 ? 20 : 29; }
 
 __device__ __forceinline__ u64 mul_wide(u32 a, u32 b) {
@@ -62,7 +63,7 @@ struct Mod {
     u64 q;
     u64 K;      // multiple of q: 2^13 q (NEAR50: makes any signed value non-negative), 7 q (NEAR60), 4 q (SHOUP)
     u32 delta;  // near primes
-    static constexpr bool shoup = AR == AR_SHOUP || AR == AR_LAZY;
+    static constexpr bool shoup = !is_near(AR);
     __device__ __forceinline__ explicit Mod(const Prime& p) : q(p.q) {
         K = AR == AR_NEAR50 ? p.q << 13 : AR == AR_NEAR60 ? p.q * 7 : p.q << 2;
         delta = p.delta;
@@ -230,14 +231,16 @@ template <int V>
 struct Tag {
     static constexpr int value = V;
 };
-// f is called with the arithmetic of prime p as a compile-time constant, for a transform of the direction INV. (A branch
-// around the butterflies of every register block in place of AR_LAZY keeps their twiddles from loading early: two
-// polynomials of three 32- and 40-bit limbs at N = 2^13, forward and inverse, 29.7 us against 28.8 before it.)
-template <bool INV, class F>
+// f is called with the arithmetic of prime p as a compile-time constant. LAZY: AR_LAZY is one of them, else its primes
+// take AR_SHOUP: for forward transforms of many or short rows. In the passes of few rows a fourth copy of the code costs
+// more than the reductions (two polynomials of three 32- and 40-bit limbs at N = 2^13, forward and inverse, 28.7 us
+// without it and 29.5 with it).
+template <bool LAZY, class F>
 __device__ __forceinline__ void with_arith(const Prime& p, F&& f) {
-    if (p.cls == AR_NEAR50) f(Tag<AR_NEAR50>{});
-    else if (p.cls == AR_NEAR60) f(Tag<AR_NEAR60>{});
-    else if (!INV && p.b <= 57) f(Tag<INV ? AR_SHOUP : AR_LAZY>{});
+    const u32 cls = p.cls;
+    if (cls == AR_NEAR50) f(Tag<AR_NEAR50>{});
+    else if (LAZY && cls == AR_LAZY) f(Tag<LAZY ? AR_LAZY : AR_SHOUP>{});
+    else if (cls == AR_NEAR60) f(Tag<AR_NEAR60>{});
     else f(Tag<AR_SHOUP>{});
 }
 
