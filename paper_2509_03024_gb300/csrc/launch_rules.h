@@ -14,7 +14,7 @@ namespace rules {
 //   fused passes (key switches, rescales) one: a second pass costs every stored row another trip and every
 //     conversion its own launch. 256 rotations of four 40-bit limbs 516 us in two, 496 in one; 64 rescales 58, 48;
 //     one product 60 against 70 (50-bit limbs); 512 products of 60-bit limbs are the one place where two win, by 3 %
-//   plain transforms (us, forward / inverse of 40-bit rows, in two : in one): 32 rows 8 : 10 / 8 : 10, 64 rows
+//   plain transforms (us, forward / inverse of 40-bit rows, reduced in every stage, in two : in one): 32 rows 8 : 10 / 8 : 10, 64 rows
 //     11 : 10 / 12 : 10, 512 rows 31 : 28 / 34 : 31, 768 rows 37 : 39 / 43 : 43, 8192 rows 319 : 328 / 353 : 351.
 //     Two up to a third of a row per SM, where one pass leaves most SMs idle, and in forward transforms of more
 //     than four rows per SM, where the two passes' smaller tiles keep more warps in flight.
